@@ -57,10 +57,7 @@ struct DevBuf {
 void free_graph(gp_graph* g) {
     if (!g) return;
     if (g->labels) cudaFree(g->labels);
-    if (g->row_ptr) cudaFree(g->row_ptr);
-    if (g->col) cudaFree(g->col);
-    if (g->perm) cudaFree(g->perm);
-    if (g->core_bits) cudaFree(g->core_bits);
+    if (g->mem) cudaFree(g->mem);
     delete g;
 }
 
@@ -299,13 +296,12 @@ gp_status gp_graph_create_csr(const int64_t* row_ptr, const int32_t* col, int32_
         dcol = static_cast<const int32_t*>(bcol.p);
     }
     if ((flags & GP_ASSUME_CLEAN) && !(flags & GP_DEGREE_ORDER)) {
-        GP_CUDA_TRY(cudaMalloc(&g->row_ptr, sizeof(int64_t) * ((size_t)n + 1)));
-        GP_CUDA_TRY(cudaMalloc(&g->col, sizeof(int32_t) * (size_t)(nnz ? nnz : 1)));
+        gp_status rc = alloc_graph(g.get(), n, nnz, false);
+        if (rc != GP_OK) return rc;
         GP_CUDA_TRY(cudaMemcpyAsync(g->row_ptr, drp, sizeof(int64_t) * ((size_t)n + 1), cudaMemcpyDeviceToDevice, st));
         if (nnz) GP_CUDA_TRY(cudaMemcpyAsync(g->col, dcol, sizeof(int32_t) * (size_t)nnz, cudaMemcpyDeviceToDevice, st));
-        g->n = n;
-        g->nnz = nnz;
-        gp_status rc = max_degree(g->row_ptr, n, st, &g->max_deg);
+        if (n == 0) GP_CUDA_TRY(cudaStreamSynchronize(st));
+        rc = finish_graph(g.get(), st);
         if (rc != GP_OK) return rc;
         *out = g.release();
         return GP_OK;

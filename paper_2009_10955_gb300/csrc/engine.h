@@ -19,6 +19,7 @@ struct gp_graph {
     int32_t max_deg = 0;
     int64_t heavy_end = 0;        // CSR entries of the leading vertices of degree
                                   // >= kHeavyDegree (degree-ordered graphs only)
+    void* mem = nullptr;          // device, the one allocation behind the arrays below but the labels
     int64_t* row_ptr = nullptr;   // device, n + 1
     int32_t* col = nullptr;       // device, nnz
     int32_t* labels = nullptr;      // device, n vertex labels (graph labelling) or null
@@ -26,6 +27,10 @@ struct gp_graph {
     int32_t core_n = 0;             // the core_n highest-degree vertices (ids
     int32_t core_words = 0;         // 0..core_n-1 of a degree-ordered graph)
     int32_t* perm = nullptr;      // device, n (new id -> input id) or null
+    int32_t* dplus = nullptr;     // device, n: neighbours with a smaller id, per vertex
+    int32_t* roots = nullptr;     // device, n: vertices by dplus, largest first
+    int32_t max_dplus = 0;
+    int64_t roots_ge[32] = {};    // vertices with dplus >= 2^i
     std::mutex mu;
     bool tri_done = false;
     uint64_t tri_cnt = 0;         // ordered triangles (6 x triangles)
@@ -42,14 +47,11 @@ gp_status build_graph(const int32_t* d_src, const int32_t* d_dst, int64_t m, int
 // Expand a device CSR to pairs (graph.cu).
 gp_status csr_to_pairs(const int64_t* d_row_ptr, const int32_t* d_col, int32_t n, int64_t nnz,
                        int32_t* d_src, int32_t* d_dst, cudaStream_t st);
-// Maximum degree of a device CSR (graph.cu).
-gp_status max_degree(const int64_t* d_row_ptr, int32_t n, cudaStream_t st, int32_t* out);
-// Adjacency bit matrix of vertices [0, core_n) among themselves (graph.cu).
-gp_status build_core_bits(gp_graph* g, int32_t core_n, cudaStream_t st);
-// First CSR entry of the first vertex whose degree is below min_deg, for a
-// graph whose degrees do not increase with the id (graph.cu).
-gp_status heavy_prefix(const int64_t* d_row_ptr, int32_t n, int32_t min_deg, cudaStream_t st,
-                       int64_t* out);
+// Allocate the arrays of a graph with nnz entries (graph.cu).
+gp_status alloc_graph(gp_graph* g, int32_t n, int64_t nnz, bool ordered);
+// From row_ptr and col (and perm): dplus, roots, the core bit matrix and the
+// host's facts; synchronises the stream (graph.cu).
+gp_status finish_graph(gp_graph* g, cudaStream_t st);
 
 // One counting job for the device (count.cu).
 struct CountJob {

@@ -2,12 +2,13 @@
 // directions, sort, deduplicate, optionally relabel by degree, and lay the
 // result out as CSR with sorted neighbour lists (GraphPi Section IV-E).
 //
-// Each directed pair (u, v) travels as one 64-bit key (u << 32) | v, so a
-// single radix sort orders the pairs by source and then by target, which is
-// exactly the CSR order. The sort and the unique pass are CUB library calls.
+// Each directed pair (u, v) travels as one key with u above v, so a single
+// radix sort orders the pairs by source and then by target, which is exactly
+// the CSR order. The sorts, the unique pass and the scan are CUB library calls.
 #include <algorithm>
 
 #include <cub/device/device_radix_sort.cuh>
+#include <cub/device/device_scan.cuh>
 #include <cub/device/device_select.cuh>
 
 #include "engine.h"
@@ -29,35 +30,36 @@ int bits_for(uint64_t x) {     // bits needed to represent x
     return b;
 }
 
-__global__ void k_check_ids(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
-                            int64_t m, int32_t n, int* __restrict__ bad) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t u = src[i], v = dst[i];
-        if (u < 0 || u >= n || v < 0 || v >= n) atomicExch(bad, 1);
-    }
-}
+// What the host reads back of the pairs: kInfoBad is set by an id outside
+// [0, n), kInfoLoop by a self loop, kInfoUnique receives the number of
+// distinct keys.
+enum { kInfoBad, kInfoLoop, kInfoUnique, kInfoPairs };
 
-// Pair i yields keys 2i (u -> v) and 2i + 1 (v -> u); a self loop yields two
-// copies of the sentinel n << 32, which sorts after every real key.
+// Pair i yields keys 2i (u -> v) and 2i + 1 (v -> u), written as one 16-byte
+// store; a key is (u << shift) | v, with `shift` the bits of the largest id,
+// so that the sort sees no dead bits between the two. A self loop or an id out
+// of range yields two copies of the sentinel n << shift, which sorts after
+// every real key.
 __global__ void k_make_keys(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
-                            int64_t m, int32_t n, uint64_t* __restrict__ keys) {
+                            int64_t m, int32_t n, int shift, ulonglong2* __restrict__ keys,
+                            int64_t* __restrict__ info) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
          i += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t u = (uint32_t)src[i], v = (uint32_t)dst[i];
-        uint64_t a = (u << 32) | v, b = (v << 32) | u;
-        if (u == v) a = b = (uint64_t)(uint32_t)n << 32;
-        keys[2 * i] = a;
-        keys[2 * i + 1] = b;
+        const int32_t u = src[i], v = dst[i];
+        const bool ok = u >= 0 && u < n && v >= 0 && v < n;
+        if (!ok) info[kInfoBad] = 1;
+        else if (u == v) info[kInfoLoop] = 1;
+        const uint64_t a = (uint32_t)u, b = (uint32_t)v, none = (uint64_t)(uint32_t)n << shift;
+        keys[i] = (ok && u != v) ? make_ulonglong2((a << shift) | b, (b << shift) | a) : make_ulonglong2(none, none);
     }
 }
 
 // row_ptr[u] = first key whose source is >= u (binary search in sorted keys).
-__global__ void k_row_ptr(const uint64_t* __restrict__ keys, int64_t nnz, int32_t n,
+__global__ void k_row_ptr(const uint64_t* __restrict__ keys, int64_t nnz, int32_t n, int shift,
                           int64_t* __restrict__ row_ptr) {
     for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u <= n;
          u += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t target = (uint64_t)u << 32;
+        uint64_t target = (uint64_t)u << shift;
         int64_t lo = 0, hi = nnz;
         while (lo < hi) {
             int64_t mid = lo + ((hi - lo) >> 1);
@@ -67,10 +69,10 @@ __global__ void k_row_ptr(const uint64_t* __restrict__ keys, int64_t nnz, int32_
     }
 }
 
-__global__ void k_col(const uint64_t* __restrict__ keys, int64_t nnz, int32_t* __restrict__ col) {
+__global__ void k_col(const uint64_t* __restrict__ keys, int64_t nnz, int shift, int32_t* __restrict__ col) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nnz;
          i += (int64_t)gridDim.x * blockDim.x)
-        col[i] = (int32_t)(uint32_t)keys[i];
+        col[i] = (int32_t)(keys[i] & (((uint64_t)1 << shift) - 1));
 }
 
 __global__ void k_max_deg(const int64_t* __restrict__ row_ptr, int32_t n, int* __restrict__ out) {
@@ -82,39 +84,47 @@ __global__ void k_max_deg(const int64_t* __restrict__ row_ptr, int32_t n, int* _
     if ((threadIdx.x & 31) == 0) atomicMax(out, best);
 }
 
-// Degree-order key: (max_deg - deg) in the high half sorts high degrees first,
-// the vertex id in the low half breaks ties by id.
-__global__ void k_degree_keys(const int64_t* __restrict__ row_ptr, int32_t n, int32_t max_deg,
-                              uint64_t* __restrict__ keys) {
+// Degree and id of every vertex, to sort by degree (the sort is stable, so
+// ties keep the id order).
+__global__ void k_degrees(const int64_t* __restrict__ row_ptr, int32_t n, int32_t* __restrict__ deg,
+                          int32_t* __restrict__ ids) {
     for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n;
          u += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t deg = (uint64_t)(row_ptr[u + 1] - row_ptr[u]);
-        keys[u] = (((uint64_t)max_deg - deg) << 32) | (uint64_t)u;
+        deg[u] = (int32_t)(row_ptr[u + 1] - row_ptr[u]);
+        ids[u] = (int32_t)u;
     }
 }
 
-__global__ void k_perm_from_keys(const uint64_t* __restrict__ keys, int32_t n,
-                                 int32_t* __restrict__ new2old, int32_t* __restrict__ old2new) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+// The inverse of new2old, and the new degrees in 64 bits with a zero behind
+// them (their exclusive sum is the new row_ptr).
+__global__ void k_inverse(const int32_t* __restrict__ new2old, const int32_t* __restrict__ sorted_deg, int32_t n,
+                          int32_t* __restrict__ old2new, int64_t* __restrict__ deg64) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= n;
          i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t old = (int32_t)(uint32_t)keys[i];
-        new2old[i] = old;
-        old2new[old] = (int32_t)i;
+        deg64[i] = i < n ? sorted_deg[i] : 0;
+        if (i < n) old2new[new2old[i]] = (int32_t)i;
     }
 }
 
-// Entry e of row u becomes key (old2new[u] << 32) | old2new[col[e]].
-__global__ void k_relabel_keys(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                               int32_t n, int64_t nnz, const int32_t* __restrict__ old2new,
-                               uint64_t* __restrict__ keys) {
+// The entries (u, v) of the old graph in the order of the new id of u: entry
+// e of old row u goes to its place in the new row of u, as the pair (target =
+// new id of v, source = new id of u). The graph is symmetric, so these are
+// also the entries of every new row `target`, and a stable sort by target
+// alone leaves each row's sources ascending: half the key bits of sorting
+// whole relabelled entries. The key itself names u and v (no row search:
+// 0.53 -> 0.16 ms for 31 M entries).
+__global__ void k_relabel(const uint64_t* __restrict__ keys, int64_t nnz, int shift,
+                          const int64_t* __restrict__ old_row, const int64_t* __restrict__ new_row,
+                          const int32_t* __restrict__ old2new, int32_t* __restrict__ target,
+                          int32_t* __restrict__ source) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nnz;
          e += (int64_t)gridDim.x * blockDim.x) {
-        int64_t lo = 0, hi = n;                 // row of e: last u with row_ptr[u] <= e
-        while (hi - lo > 1) {
-            int64_t mid = (lo + hi) >> 1;
-            if (row_ptr[mid] <= e) lo = mid; else hi = mid;
-        }
-        keys[e] = ((uint64_t)(uint32_t)old2new[lo] << 32) | (uint32_t)old2new[col[e]];
+        const uint64_t key = keys[e];
+        const int32_t u = (int32_t)(key >> shift), v = (int32_t)(key & (((uint64_t)1 << shift) - 1));
+        const int32_t nu = old2new[u];
+        const int64_t at = new_row[nu] + (e - old_row[u]);
+        target[at] = old2new[v];
+        source[at] = nu;
     }
 }
 
@@ -143,52 +153,14 @@ struct Scratch {
     template <class T> T* as() const { return static_cast<T*>(p); }
 };
 
-// Sorted unique keys -> (row_ptr, col) allocated into g.
-gp_status keys_to_csr(const uint64_t* d_keys, int64_t nnz, int32_t n, cudaStream_t st, gp_graph* g) {
-    int64_t* row_ptr = nullptr;
-    int32_t* col = nullptr;
-    GP_CUDA_TRY(cudaMalloc(&row_ptr, sizeof(int64_t) * ((size_t)n + 1)));
-    if (cudaMalloc(&col, sizeof(int32_t) * (size_t)(nnz ? nnz : 1)) != cudaSuccess) {
-        cudaFree(row_ptr);
-        set_error("cudaMalloc of %lld column ids failed", (long long)nnz);
-        return GP_ERR_NOMEM;
-    }
-    k_row_ptr<<<blocks_for((int64_t)n + 1), kThreads, 0, st>>>(d_keys, nnz, n, row_ptr);
-    if (nnz) k_col<<<blocks_for(nnz), kThreads, 0, st>>>(d_keys, nnz, col);
-    count_launch(nnz ? 2 : 1);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-        cudaFree(row_ptr); cudaFree(col);
-        set_error("CSR kernels failed: %s", cudaGetErrorString(e));
-        return GP_ERR_CUDA;
-    }
-    g->row_ptr = row_ptr;
-    g->col = col;
-    g->nnz = nnz;
-    g->n = n;
-    return GP_OK;
-}
-
-// One thread: binary search for the first vertex of degree < min_deg.
-__global__ void k_heavy_prefix(const int64_t* __restrict__ row_ptr, int32_t n, int32_t min_deg,
-                               int64_t* __restrict__ out) {
-    int32_t lo = 0, hi = n;
-    while (lo < hi) {
-        int32_t mid = lo + ((hi - lo) >> 1);
-        if (row_ptr[mid + 1] - row_ptr[mid] >= min_deg) lo = mid + 1; else hi = mid;
-    }
-    *out = row_ptr[lo];
-}
-
-// One warp per core vertex u: set bit x of row u for every neighbour x of u
-// below core_n (a prefix of u's sorted list).
+// One block per core vertex u: set bit x of row u for every neighbour x of u
+// below core_n (a prefix of u's sorted list; up to core_n entries, so a warp
+// would walk it for 0.1 ms).
 __global__ void k_core_bits(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                             int32_t core_n, int32_t words, uint32_t* __restrict__ bits) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t u = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; u < core_n;
-         u += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    for (int64_t u = blockIdx.x; u < core_n; u += gridDim.x) {
         const int64_t b = row_ptr[u], e = row_ptr[u + 1];
-        for (int64_t i = b + lane; i < e; i += 32) {
+        for (int64_t i = b + threadIdx.x; i < e; i += blockDim.x) {
             const int32_t x = col[i];
             if (x >= core_n) break;
             atomicOr(bits + u * words + (x >> 5), 1u << (x & 31));
@@ -196,63 +168,120 @@ __global__ void k_core_bits(const int64_t* __restrict__ row_ptr, const int32_t* 
     }
 }
 
+// dplus[u]: entries of row u below u (a prefix of the sorted row); the keys
+// and ids to sort by it.
+__global__ void k_dplus(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int32_t n,
+                        int32_t* __restrict__ dplus, int32_t* __restrict__ ids) {
+    for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n;
+         u += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t b = row_ptr[u];
+        int64_t lo = b, hi = row_ptr[u + 1];
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (col[mid] < u) lo = mid + 1; else hi = mid;
+        }
+        dplus[u] = (int32_t)(lo - b);
+        ids[u] = (int32_t)u;
+    }
+}
+
+// What the host keeps about the finished graph.
+struct GraphInfo {
+    int64_t roots_ge[32];     // entries of the non-increasing `sorted` that are >= 2^i
+    int64_t heavy_end;        // degree-ordered graphs: first entry of the first row shorter than kHeavyDegree
+    int32_t max_dplus;
+    int32_t max_deg;
+};
+
+// One thread per fact; max_deg arrives from k_max_deg unless the rows are
+// ordered by degree.
+__global__ void k_graph_info(const int32_t* __restrict__ sorted, const int64_t* __restrict__ row_ptr, int32_t n,
+                             bool ordered, GraphInfo* __restrict__ out) {
+    const int i = threadIdx.x;
+    if (i > 32) return;
+    if (i == 32) {
+        out->max_dplus = sorted[0];
+        if (ordered) out->max_deg = (int32_t)(row_ptr[1] - row_ptr[0]);
+    }
+    int32_t lo = 0, hi = (i == 32 && !ordered) ? 0 : n;
+    while (lo < hi) {
+        const int32_t mid = lo + ((hi - lo) >> 1);
+        const bool in = i == 32 ? row_ptr[mid + 1] - row_ptr[mid] >= kHeavyDegree
+                                : (int64_t)sorted[mid] >= ((int64_t)1 << i);
+        if (in) lo = mid + 1; else hi = mid;
+    }
+    if (i == 32) out->heavy_end = ordered ? row_ptr[lo] : 0;
+    else out->roots_ge[i] = lo;
+}
+
+inline size_t padded(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
+
 }  // namespace
 
-gp_status build_core_bits(gp_graph* g, int32_t core_n, cudaStream_t st) {
-    if (core_n <= 0) return GP_OK;
-    // rows padded to a multiple of 4 words: 16-byte loads stay aligned
-    const int32_t words = (((core_n + 31) / 32) + 3) & ~3;
-    const size_t bytes = sizeof(uint32_t) * (size_t)core_n * (size_t)words;
-    uint32_t* bits = nullptr;
-    GP_CUDA_TRY(cudaMalloc(&bits, bytes));
-    cudaError_t e = cudaMemsetAsync(bits, 0, bytes, st);
-    if (e == cudaSuccess) {
-        const int blocks = (int)std::min<int64_t>(((int64_t)core_n * 32 + kThreads - 1) / kThreads, 4096);
-        k_core_bits<<<blocks, kThreads, 0, st>>>(g->row_ptr, g->col, core_n, words, bits);
-        count_launch();
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+gp_status alloc_graph(gp_graph* g, int32_t n, int64_t nnz, bool ordered) {
+    // one allocation for all arrays: each costs a synchronising driver call
+    const int32_t core_n = ordered ? std::min(n, kCoreMax) : 0;
+    const int32_t words = (((core_n + 31) / 32) + 3) & ~3;   // rows of whole 16-byte groups
+    const size_t rows_b = padded(sizeof(int64_t) * ((size_t)n + 1)), col_b = padded(sizeof(int32_t) * (size_t)(nnz + 1));
+    const size_t vert_b = padded(sizeof(int32_t) * (size_t)n), core_b = sizeof(uint32_t) * (size_t)core_n * (size_t)words;
+    char* p = nullptr;
+    const cudaError_t e = cudaMalloc((void**)&p, rows_b + col_b + (ordered ? 3 : 2) * vert_b + core_b);
     if (e != cudaSuccess) {
-        cudaFree(bits);
-        set_error("core bit matrix: %s", cudaGetErrorString(e));
-        return GP_ERR_CUDA;
+        cudaGetLastError();
+        set_error("cudaMalloc of a graph with %lld entries failed: %s", (long long)nnz, cudaGetErrorString(e));
+        return e == cudaErrorMemoryAllocation ? GP_ERR_NOMEM : GP_ERR_CUDA;
     }
-    g->core_bits = bits;
-    g->core_n = core_n;
-    g->core_words = words;
+    g->mem = p;
+    g->n = n;
+    g->nnz = nnz;
+    g->row_ptr = reinterpret_cast<int64_t*>(p);
+    g->col = reinterpret_cast<int32_t*>(p += rows_b);
+    g->dplus = reinterpret_cast<int32_t*>(p += col_b);
+    g->roots = reinterpret_cast<int32_t*>(p += vert_b);
+    p += vert_b;
+    if (ordered) {
+        g->perm = reinterpret_cast<int32_t*>(p);
+        g->core_bits = reinterpret_cast<uint32_t*>(p + vert_b);
+        g->core_n = core_n;
+        g->core_words = words;
+    }
     return GP_OK;
 }
 
-gp_status heavy_prefix(const int64_t* d_row_ptr, int32_t n, int32_t min_deg, cudaStream_t st,
-                       int64_t* out) {
-    Scratch s(st);
-    GP_CUDA_TRY(s.alloc(sizeof(int64_t)));
-    k_heavy_prefix<<<1, 1, 0, st>>>(d_row_ptr, n, min_deg, s.as<int64_t>());
-    count_launch();
-    GP_CUDA_TRY(cudaGetLastError());
-    int64_t h = 0;
-    GP_CUDA_TRY(cudaMemcpyAsync(&h, s.p, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    GP_CUDA_TRY(cudaStreamSynchronize(st));
-    *out = h;
-    return GP_OK;
-}
-
-gp_status max_degree(const int64_t* d_row_ptr, int32_t n, cudaStream_t st, int32_t* out) {
-    Scratch s(st);
-    GP_CUDA_TRY(s.alloc(sizeof(int)));
-    GP_CUDA_TRY(cudaMemsetAsync(s.p, 0, sizeof(int), st));
-    if (n > 0) {
-        int blocks = blocks_for(n);
-        if (blocks > 4096) blocks = 4096;
-        k_max_deg<<<blocks, kThreads, 0, st>>>(d_row_ptr, n, s.as<int>());
+gp_status finish_graph(gp_graph* g, cudaStream_t st) {
+    const int32_t n = g->n;
+    if (n == 0) return GP_OK;
+    const bool ordered = g->perm != nullptr;
+    Scratch ids(st), keys(st), temp(st), info(st);
+    GP_CUDA_TRY(ids.alloc(sizeof(int32_t) * (size_t)n));
+    GP_CUDA_TRY(keys.alloc(sizeof(int32_t) * (size_t)n));
+    GP_CUDA_TRY(info.alloc(sizeof(GraphInfo)));
+    GraphInfo* d_info = info.as<GraphInfo>();
+    GP_CUDA_TRY(cudaMemsetAsync(d_info, 0, sizeof(GraphInfo), st));
+    k_dplus<<<blocks_for(n), kThreads, 0, st>>>(g->row_ptr, g->col, n, g->dplus, ids.as<int32_t>());
+    size_t tb = 0;
+    const int bits = std::max(1, bits_for((uint64_t)n - 1));
+    GP_CUDA_TRY(cub::DeviceRadixSort::SortPairsDescending(nullptr, tb, g->dplus, keys.as<int32_t>(), ids.as<int32_t>(),
+                                                          g->roots, n, 0, bits, st));
+    GP_CUDA_TRY(temp.alloc(tb));
+    GP_CUDA_TRY(cub::DeviceRadixSort::SortPairsDescending(temp.p, tb, g->dplus, keys.as<int32_t>(), ids.as<int32_t>(),
+                                                          g->roots, n, 0, bits, st));
+    if (!ordered) k_max_deg<<<std::min(blocks_for(n), 4096), kThreads, 0, st>>>(g->row_ptr, n, &d_info->max_deg);
+    k_graph_info<<<1, 64, 0, st>>>(keys.as<int32_t>(), g->row_ptr, n, ordered, d_info);
+    count_launch(ordered ? 3 : 4);
+    if (g->core_n > 0) {
+        GP_CUDA_TRY(cudaMemsetAsync(g->core_bits, 0, sizeof(uint32_t) * (size_t)g->core_n * (size_t)g->core_words, st));
+        k_core_bits<<<g->core_n, kThreads, 0, st>>>(g->row_ptr, g->col, g->core_n, g->core_words, g->core_bits);
         count_launch();
-        GP_CUDA_TRY(cudaGetLastError());
     }
-    int h = 0;
-    GP_CUDA_TRY(cudaMemcpyAsync(&h, s.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+    GP_CUDA_TRY(cudaGetLastError());
+    GraphInfo h;
+    GP_CUDA_TRY(cudaMemcpyAsync(&h, d_info, sizeof(h), cudaMemcpyDeviceToHost, st));
     GP_CUDA_TRY(cudaStreamSynchronize(st));
-    *out = h;
+    for (int i = 0; i < 32; ++i) g->roots_ge[i] = h.roots_ge[i];
+    g->max_dplus = h.max_dplus;
+    g->max_deg = h.max_deg;
+    g->heavy_end = h.heavy_end;
     return GP_OK;
 }
 
@@ -267,105 +296,87 @@ gp_status csr_to_pairs(const int64_t* d_row_ptr, const int32_t* d_col, int32_t n
 
 gp_status build_graph(const int32_t* d_src, const int32_t* d_dst, int64_t m, int32_t n,
                       bool degree_order, cudaStream_t st, gp_graph* g) {
-    // 1. ids in range
-    {
-        Scratch bad(st);
-        GP_CUDA_TRY(bad.alloc(sizeof(int)));
-        GP_CUDA_TRY(cudaMemsetAsync(bad.p, 0, sizeof(int), st));
-        if (m > 0) {
-            k_check_ids<<<blocks_for(m), kThreads, 0, st>>>(d_src, d_dst, m, n, bad.as<int>());
-            count_launch();
-            GP_CUDA_TRY(cudaGetLastError());
-        }
-        int h = 0;
-        GP_CUDA_TRY(cudaMemcpyAsync(&h, bad.p, sizeof(int), cudaMemcpyDeviceToHost, st));
-        GP_CUDA_TRY(cudaStreamSynchronize(st));
-        if (h) { set_error("edge endpoint outside [0, %d)", n); return GP_ERR_ARG; }
-    }
     const int64_t nkeys = 2 * m;
-    const int end_bit = 32 + bits_for((uint64_t)(uint32_t)n);
-    Scratch keys_a(st), keys_b(st), nsel(st), temp(st);
+    const int id_bits = std::max(1, n > 0 ? bits_for((uint64_t)n - 1) : 0);
+    const int end_bit = id_bits + bits_for((uint64_t)(uint32_t)n);
+    Scratch keys_a(st), keys_b(st), info(st), temp(st);
     GP_CUDA_TRY(keys_a.alloc(sizeof(uint64_t) * (size_t)nkeys));
     GP_CUDA_TRY(keys_b.alloc(sizeof(uint64_t) * (size_t)nkeys));
-    GP_CUDA_TRY(nsel.alloc(sizeof(int64_t)));
-    int64_t nnz = 0;
+    cub::DoubleBuffer<uint64_t> keys(keys_a.as<uint64_t>(), keys_b.as<uint64_t>());
+    int64_t h[kInfoPairs] = {};
     if (m > 0) {
-        // 2-3. both directions as 64-bit keys, self loops to the sentinel
-        k_make_keys<<<blocks_for(m), kThreads, 0, st>>>(d_src, d_dst, m, n, keys_a.as<uint64_t>());
+        // both directions as keys, sorted (CUB), each kept once
+        GP_CUDA_TRY(info.alloc(sizeof(h)));
+        GP_CUDA_TRY(cudaMemsetAsync(info.p, 0, sizeof(h), st));
+        k_make_keys<<<blocks_for(m), kThreads, 0, st>>>(d_src, d_dst, m, n, id_bits,
+                                                        reinterpret_cast<ulonglong2*>(keys.Current()), info.as<int64_t>());
         count_launch();
         GP_CUDA_TRY(cudaGetLastError());
-        // 4. radix sort (CUB)
-        size_t tbytes = 0, tbytes2 = 0;
-        GP_CUDA_TRY(cub::DeviceRadixSort::SortKeys(nullptr, tbytes, keys_a.as<uint64_t>(),
-                                                   keys_b.as<uint64_t>(), nkeys, 0, end_bit, st));
-        GP_CUDA_TRY(cub::DeviceSelect::Unique(nullptr, tbytes2, keys_b.as<uint64_t>(),
-                                              keys_a.as<uint64_t>(), nsel.as<int64_t>(), nkeys, st));
-        GP_CUDA_TRY(temp.alloc(tbytes > tbytes2 ? tbytes : tbytes2));
-        GP_CUDA_TRY(cub::DeviceRadixSort::SortKeys(temp.p, tbytes, keys_a.as<uint64_t>(),
-                                                   keys_b.as<uint64_t>(), nkeys, 0, end_bit, st));
-        // 5. unique
-        GP_CUDA_TRY(cub::DeviceSelect::Unique(temp.p, tbytes2, keys_b.as<uint64_t>(),
-                                              keys_a.as<uint64_t>(), nsel.as<int64_t>(), nkeys, st));
+        size_t tb = 0, tb2 = 0;
+        GP_CUDA_TRY(cub::DeviceRadixSort::SortKeys(nullptr, tb, keys, nkeys, 0, end_bit, st));
+        GP_CUDA_TRY(cub::DeviceSelect::Unique(nullptr, tb2, keys.Current(), keys.Alternate(),
+                                              info.as<int64_t>() + kInfoUnique, nkeys, st));
+        GP_CUDA_TRY(temp.alloc(std::max(tb, tb2)));
+        GP_CUDA_TRY(cub::DeviceRadixSort::SortKeys(temp.p, tb, keys, nkeys, 0, end_bit, st));
+        GP_CUDA_TRY(cub::DeviceSelect::Unique(temp.p, tb2, keys.Current(), keys.Alternate(),
+                                              info.as<int64_t>() + kInfoUnique, nkeys, st));
+        keys.selector ^= 1;
         count_launch(2);
-        int64_t h = 0;
-        GP_CUDA_TRY(cudaMemcpyAsync(&h, nsel.p, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-        uint64_t last = 0;
+        GP_CUDA_TRY(cudaMemcpyAsync(h, info.p, sizeof(h), cudaMemcpyDeviceToHost, st));
         GP_CUDA_TRY(cudaStreamSynchronize(st));
-        if (h > 0) {
-            GP_CUDA_TRY(cudaMemcpyAsync(&last, keys_a.as<uint64_t>() + (h - 1), sizeof(uint64_t),
-                                        cudaMemcpyDeviceToHost, st));
-            GP_CUDA_TRY(cudaStreamSynchronize(st));
-        }
-        nnz = h - ((h > 0 && last == ((uint64_t)(uint32_t)n << 32)) ? 1 : 0);
+        if (h[kInfoBad]) { set_error("edge endpoint outside [0, %d)", n); return GP_ERR_ARG; }
     }
-    // 7. CSR from the sorted unique keys
-    gp_status rc = keys_to_csr(keys_a.as<uint64_t>(), nnz, n, st, g);
+    const int64_t nnz = h[kInfoUnique] - (h[kInfoLoop] ? 1 : 0);    // without the sentinel
+    const bool ordered = degree_order && n > 0;
+    gp_status rc = alloc_graph(g, n, nnz, ordered);
     if (rc != GP_OK) return rc;
-    rc = max_degree(g->row_ptr, n, st, &g->max_deg);
-    if (rc != GP_OK) return rc;
-    if (!degree_order || n == 0) return GP_OK;
+    if (!ordered) {
+        k_row_ptr<<<blocks_for((int64_t)n + 1), kThreads, 0, st>>>(keys.Current(), nnz, n, id_bits, g->row_ptr);
+        if (nnz) k_col<<<blocks_for(nnz), kThreads, 0, st>>>(keys.Current(), nnz, id_bits, g->col);
+        count_launch(nnz ? 2 : 1);
+        GP_CUDA_TRY(cudaGetLastError());
+        if (n == 0) GP_CUDA_TRY(cudaStreamSynchronize(st));
+        return finish_graph(g, st);
+    }
 
-    // 6. relabel by non-increasing degree, then rebuild the CSR
-    Scratch vkeys(st), vkeys2(st), old2new(st), temp2(st);
-    int32_t* new2old = nullptr;
-    GP_CUDA_TRY(vkeys.alloc(sizeof(uint64_t) * (size_t)n));
-    GP_CUDA_TRY(vkeys2.alloc(sizeof(uint64_t) * (size_t)n));
-    GP_CUDA_TRY(old2new.alloc(sizeof(int32_t) * (size_t)n));
-    GP_CUDA_TRY(cudaMalloc(&new2old, sizeof(int32_t) * (size_t)n));
-    k_degree_keys<<<blocks_for(n), kThreads, 0, st>>>(g->row_ptr, n, g->max_deg, vkeys.as<uint64_t>());
-    count_launch();
-    size_t tb = 0, tb2 = 0;
-    const int vend = 32 + bits_for((uint64_t)g->max_deg);
-    GP_CUDA_TRY(cub::DeviceRadixSort::SortKeys(nullptr, tb, vkeys.as<uint64_t>(), vkeys2.as<uint64_t>(),
-                                               (int64_t)n, 0, vend, st));
-    if (nnz > 0)
-        GP_CUDA_TRY(cub::DeviceRadixSort::SortKeys(nullptr, tb2, keys_b.as<uint64_t>(),
-                                                   keys_a.as<uint64_t>(), nnz, 0, end_bit, st));
-    GP_CUDA_TRY(temp2.alloc(tb > tb2 ? tb : tb2));
-    GP_CUDA_TRY(cub::DeviceRadixSort::SortKeys(temp2.p, tb, vkeys.as<uint64_t>(), vkeys2.as<uint64_t>(),
-                                               (int64_t)n, 0, vend, st));
-    k_perm_from_keys<<<blocks_for(n), kThreads, 0, st>>>(vkeys2.as<uint64_t>(), n, new2old,
-                                                         old2new.as<int32_t>());
+    // relabel by non-increasing degree (ties by id)
+    Scratch old_row(st), vert(st), deg64(st), temp2(st);
+    GP_CUDA_TRY(old_row.alloc(sizeof(int64_t) * ((size_t)n + 1)));
+    GP_CUDA_TRY(vert.alloc(4 * sizeof(int32_t) * (size_t)n));
+    GP_CUDA_TRY(deg64.alloc(sizeof(int64_t) * ((size_t)n + 1)));
+    int32_t* deg = vert.as<int32_t>();
+    int32_t *sorted_deg = deg + n, *ids = deg + 2 * (size_t)n, *old2new = deg + 3 * (size_t)n;
+    k_row_ptr<<<blocks_for((int64_t)n + 1), kThreads, 0, st>>>(keys.Current(), nnz, n, id_bits, old_row.as<int64_t>());
+    k_degrees<<<blocks_for(n), kThreads, 0, st>>>(old_row.as<int64_t>(), n, deg, ids);
     count_launch(2);
+    GP_CUDA_TRY(cudaGetLastError());
+    // the pairs to sort: targets and sources in the free key buffer. The
+    // sources of the last pass land in g->col whichever number of passes
+    // the sort makes (it swaps its buffers once per 8 bits).
+    const bool odd = ((id_bits + 7) / 8) & 1;
+    int32_t* free_b = reinterpret_cast<int32_t*>(keys.Alternate());
+    cub::DoubleBuffer<int32_t> target(free_b, reinterpret_cast<int32_t*>(keys.Current()));
+    cub::DoubleBuffer<int32_t> source(odd ? free_b + nnz : g->col, odd ? g->col : free_b + nnz);
+    size_t tb = 0, tb2 = 0, tb3 = 0;
+    GP_CUDA_TRY(cub::DeviceRadixSort::SortPairsDescending(nullptr, tb, deg, sorted_deg, ids, g->perm, n, 0, id_bits, st));
+    GP_CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb2, deg64.as<int64_t>(), g->row_ptr, (int64_t)n + 1, st));
+    if (nnz > 0) GP_CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tb3, target, source, nnz, 0, id_bits, st));
+    GP_CUDA_TRY(temp2.alloc(std::max(std::max(tb, tb2), tb3)));
+    GP_CUDA_TRY(cub::DeviceRadixSort::SortPairsDescending(temp2.p, tb, deg, sorted_deg, ids, g->perm, n, 0, id_bits, st));
+    k_inverse<<<blocks_for((int64_t)n + 1), kThreads, 0, st>>>(g->perm, sorted_deg, n, old2new, deg64.as<int64_t>());
+    GP_CUDA_TRY(cub::DeviceScan::ExclusiveSum(temp2.p, tb2, deg64.as<int64_t>(), g->row_ptr, (int64_t)n + 1, st));
+    count_launch(3);
     if (nnz > 0) {
-        k_relabel_keys<<<blocks_for(nnz), kThreads, 0, st>>>(g->row_ptr, g->col, n, nnz,
-                                                             old2new.as<int32_t>(), keys_b.as<uint64_t>());
-        GP_CUDA_TRY(cub::DeviceRadixSort::SortKeys(temp2.p, tb2, keys_b.as<uint64_t>(),
-                                                   keys_a.as<uint64_t>(), nnz, 0, end_bit, st));
+        k_relabel<<<blocks_for(nnz), kThreads, 0, st>>>(keys.Current(), nnz, id_bits, old_row.as<int64_t>(), g->row_ptr,
+                                                        old2new, target.Current(), source.Current());
+        GP_CUDA_TRY(cudaGetLastError());
+        GP_CUDA_TRY(cub::DeviceRadixSort::SortPairs(temp2.p, tb3, target, source, nnz, 0, id_bits, st));
         count_launch(2);
+        if (source.Current() != g->col)
+            GP_CUDA_TRY(cudaMemcpyAsync(g->col, source.Current(), sizeof(int32_t) * (size_t)nnz, cudaMemcpyDeviceToDevice, st));
     }
     GP_CUDA_TRY(cudaGetLastError());
-    GP_CUDA_TRY(cudaStreamSynchronize(st));
-    cudaFree(g->row_ptr);
-    cudaFree(g->col);
-    g->row_ptr = nullptr;
-    g->col = nullptr;
-    rc = keys_to_csr(keys_a.as<uint64_t>(), nnz, n, st, g);
-    if (rc != GP_OK) { cudaFree(new2old); return rc; }
-    g->perm = new2old;
-    rc = heavy_prefix(g->row_ptr, n, kHeavyDegree, st, &g->heavy_end);
-    if (rc != GP_OK) return rc;
-    return build_core_bits(g, std::min(n, kCoreMax), st);
+    return finish_graph(g, st);
 }
 
 }  // namespace gp

@@ -94,7 +94,8 @@ gp_status triangle_count(gp_graph* g, cudaStream_t st, uint64_t* out) {
     job.core_words = g->core_words;
     uint64_t res2[2] = {0, 0};
     int64_t done = 0;
-    gp_status rc = run_count(&job, 1, LaunchOpts(), st, res2, &done);
+    gp_status rc = clique_applies(job, g, LaunchOpts()) ? run_clique(job, g, st, res2)
+                                                        : run_count(&job, 1, LaunchOpts(), st, res2, &done);
     if (rc != GP_OK) return rc;
     if (res2[1]) return fail(GP_ERR_OVERFLOW, "triangle count overflows 64 bits");
     *out = res2[0];
@@ -583,8 +584,13 @@ gp_status gp_count(gp_graph* g, const gp_schedules* s, int32_t idx, const gp_cou
     const bool want_ms = opts && opts->kernel_ms;
     int aborted = 0;
     uint64_t ops = 0, busy[2] = {0, 0};
-    rc = run_count(&job, 1, launch_opts(opts), static_cast<cudaStream_t>(stream), res, &done,
-                   want_ms ? &ms : nullptr, &bytes, &aborted, &ops, busy);
+    if (clique_applies(job, g, launch_opts(opts))) {
+        done = job.nvirt;
+        rc = run_clique(job, g, static_cast<cudaStream_t>(stream), res, want_ms ? &ms : nullptr, busy);
+    } else {
+        rc = run_count(&job, 1, launch_opts(opts), static_cast<cudaStream_t>(stream), res, &done,
+                       want_ms ? &ms : nullptr, &bytes, &aborted, &ops, busy);
+    }
     if (rc != GP_OK) return rc;
     if (aborted) return fail(GP_ERR_TIMEOUT, "a work item outlived opts.task_cycles; the count was abandoned");
     uint64_t total = 0;
@@ -643,7 +649,7 @@ gp_status gp_count_batch(gp_graph* const* graphs, const gp_schedules* const* sch
     // register budgets (or the general inclusion-exclusion code) would
     // otherwise all run with the build the most demanding one needs
     std::vector<int> key((size_t)njobs);
-    for (int32_t j = 0; j < njobs; ++j) key[j] = kernel_variant(jobs[j], lo);
+    for (int32_t j = 0; j < njobs; ++j) key[j] = clique_applies(jobs[j], graphs[j], lo) ? -1 : kernel_variant(jobs[j], lo);
     std::vector<int> keys(key);
     std::sort(keys.begin(), keys.end());
     keys.erase(std::unique(keys.begin(), keys.end()), keys.end());
@@ -651,7 +657,19 @@ gp_status gp_count_batch(gp_graph* const* graphs, const gp_schedules* const* sch
     GP_CUDA_TRY(cudaGetDevice(&dev));
     GP_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     const int user_chunk = lo.chunk;
+    for (int32_t j = 0; j < njobs; ++j) {     // cliques: a launch each (a block works on one root)
+        if (key[j] != -1) continue;
+        float jms = 0.f;
+        uint64_t jbusy[2] = {0, 0};
+        rc = run_clique(jobs[j], graphs[j], static_cast<cudaStream_t>(stream), &res[2 * j], want_ms ? &jms : nullptr,
+                        jbusy);
+        if (rc != GP_OK) return rc;
+        ms += jms;
+        busy[0] += jbusy[0];
+        busy[1] = std::max(busy[1], jbusy[1]);
+    }
     for (int kv : keys) {
+        if (kv == -1) continue;
         std::vector<CountJob> group;
         std::vector<int32_t> members;
         int64_t goff = 0;

@@ -37,6 +37,7 @@
 
 #include <cub/device/device_scan.cuh>
 
+#include "acc.cuh"
 #include "engine.h"
 
 namespace gp {
@@ -74,32 +75,6 @@ __device__ __forceinline__ unsigned long long intersect_bytes(int na, int nb) {
     const int sectors = (lo > 8) ? (32 - __clz((lo >> 3) | 1)) + 1 : 1;
     const unsigned long long search = (unsigned long long)sh * (4ull + 32ull * (unsigned long long)sectors);
     return merge < search ? merge : search;
-}
-
-struct Acc {   // per-lane 128-bit counter
-    unsigned long long lo = 0, hi = 0;
-    __device__ __forceinline__ void add(unsigned long long x) { lo += x; hi += (lo < x); }
-    __device__ __forceinline__ void sub(unsigned long long x) { hi -= (lo < x); lo -= x; }
-    __device__ __forceinline__ void add128(unsigned long long xl, unsigned long long xh) {
-        lo += xl;
-        hi += xh + (lo < xl);
-    }
-};
-
-__device__ void flush(Acc& acc, unsigned long long* res) {
-    unsigned long long lo = acc.lo, hi = acc.hi;
-    for (int o = 16; o; o >>= 1) {
-        unsigned long long l2 = __shfl_down_sync(kFull, lo, o);
-        unsigned long long h2 = __shfl_down_sync(kFull, hi, o);
-        lo += l2;
-        hi += h2 + (lo < l2);
-    }
-    if ((threadIdx.x & 31) == 0 && (lo | hi)) {
-        unsigned long long old = atomicAdd(res, lo);
-        unsigned long long carry = (old + lo < old) ? 1ull : 0ull;
-        if (hi + carry) atomicAdd(res + 1, hi + carry);
-    }
-    acc.lo = acc.hi = 0;
 }
 
 struct TaskCtx {

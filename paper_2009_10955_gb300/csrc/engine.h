@@ -105,6 +105,14 @@ gp_status run_count(const CountJob* jobs, int njobs, const LaunchOpts& lo, cudaS
                     uint64_t* algo_bytes = nullptr, int* aborted = nullptr, uint64_t* algo_ops = nullptr,
                     uint64_t* busy = nullptr);
 
+// True when the local bit matrices of clique.cu count the job: a clique's
+// plan, no option that asks for the general kernel's paths, and a graph
+// whose lists below each vertex are short enough.
+bool clique_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt);
+// The job's 128-bit total (clique.cu); kernel_ms and busy as for run_count.
+gp_status run_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, uint64_t* results,
+                     float* kernel_ms = nullptr, uint64_t* busy = nullptr);
+
 // run_count without allocating: results, job table and intermediate sets all
 // live in the caller's device buffer d_scratch (256-byte aligned); the grid
 // shrinks to what that buffer holds. GP_ERR_SCRATCH when not even one block

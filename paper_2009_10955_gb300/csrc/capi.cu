@@ -187,6 +187,15 @@ LaunchOpts launch_opts(const gp_count_opts* o) {
     return lo;
 }
 
+// Jobs that the local bit matrices of clique.cu and join.cu count.
+bool local_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& lo) {
+    return clique_applies(job, g, lo) || join_applies(job, g, lo);
+}
+
+gp_status run_local(const CountJob& job, const gp_graph* g, cudaStream_t st, uint64_t* res, float* ms, uint64_t* busy) {
+    return job.plan.iep ? run_join(job, g, st, res, ms, busy) : run_clique(job, g, st, res, ms, busy);
+}
+
 bool opts_ok(const gp_count_opts* o) {
     return !o || (o->struct_size == (int32_t)sizeof(gp_count_opts));
 }
@@ -584,9 +593,9 @@ gp_status gp_count(gp_graph* g, const gp_schedules* s, int32_t idx, const gp_cou
     const bool want_ms = opts && opts->kernel_ms;
     int aborted = 0;
     uint64_t ops = 0, busy[2] = {0, 0};
-    if (clique_applies(job, g, launch_opts(opts))) {
+    if (local_applies(job, g, launch_opts(opts))) {
         done = job.nvirt;
-        rc = run_clique(job, g, static_cast<cudaStream_t>(stream), res, want_ms ? &ms : nullptr, busy);
+        rc = run_local(job, g, static_cast<cudaStream_t>(stream), res, want_ms ? &ms : nullptr, busy);
     } else {
         rc = run_count(&job, 1, launch_opts(opts), static_cast<cudaStream_t>(stream), res, &done,
                        want_ms ? &ms : nullptr, &bytes, &aborted, &ops, busy);
@@ -649,7 +658,7 @@ gp_status gp_count_batch(gp_graph* const* graphs, const gp_schedules* const* sch
     // register budgets (or the general inclusion-exclusion code) would
     // otherwise all run with the build the most demanding one needs
     std::vector<int> key((size_t)njobs);
-    for (int32_t j = 0; j < njobs; ++j) key[j] = clique_applies(jobs[j], graphs[j], lo) ? -1 : kernel_variant(jobs[j], lo);
+    for (int32_t j = 0; j < njobs; ++j) key[j] = local_applies(jobs[j], graphs[j], lo) ? -1 : kernel_variant(jobs[j], lo);
     std::vector<int> keys(key);
     std::sort(keys.begin(), keys.end());
     keys.erase(std::unique(keys.begin(), keys.end()), keys.end());
@@ -657,11 +666,11 @@ gp_status gp_count_batch(gp_graph* const* graphs, const gp_schedules* const* sch
     GP_CUDA_TRY(cudaGetDevice(&dev));
     GP_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     const int user_chunk = lo.chunk;
-    for (int32_t j = 0; j < njobs; ++j) {     // cliques: a launch each (a block works on one root)
+    for (int32_t j = 0; j < njobs; ++j) {     // local bit matrices: a launch each (a block works on one root)
         if (key[j] != -1) continue;
         float jms = 0.f;
         uint64_t jbusy[2] = {0, 0};
-        rc = run_clique(jobs[j], graphs[j], static_cast<cudaStream_t>(stream), &res[2 * j], want_ms ? &jms : nullptr,
+        rc = run_local(jobs[j], graphs[j], static_cast<cudaStream_t>(stream), &res[2 * j], want_ms ? &jms : nullptr,
                         jbusy);
         if (rc != GP_OK) return rc;
         ms += jms;

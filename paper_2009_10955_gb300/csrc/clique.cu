@@ -20,13 +20,14 @@
 #include <vector>
 
 #include "acc.cuh"
+#include "bits.cuh"
 #include "engine.h"
 
 namespace gp {
 
 namespace {
 
-constexpr unsigned kFull = 0xffffffffu;
+constexpr unsigned kFull = kAllLanes;
 // Largest matrix a single warp works on, in rows: 128 rows of 4 words are
 // 2 KB of shared memory per level, and the pass over it takes a few
 // microseconds.
@@ -38,18 +39,8 @@ constexpr int kBlockRows = 640;
 // Largest root matrix at all; beyond it the general kernel counts.
 constexpr int kMostRows = 4096;
 
-// Row stride in words for n columns: whole 16-byte groups, an odd number of
-// them, so that eight lanes reading 16 bytes of eight consecutive rows hit
-// all 32 banks once.
-__host__ __device__ constexpr int row_stride(int n) { return 4 * (((n + 127) / 128) | 1); }
-
 struct CliqueArgs {
-    const int64_t* row_ptr;
-    const int32_t* col;
-    const uint32_t* core_bits;
-    int core_n, core_words;
-    const int32_t* roots;     // vertices by |U|, largest first
-    const int32_t* dplus;     // |U| by vertex
+    DeviceGraph g;            // dplus is |U|, roots are the vertices by |U|
     int64_t task_begin, task_end;
     int64_t n_block;          // leading roots handled by a whole block each ...
     int parts;                // ... in this many parts (the rows modulo parts)
@@ -60,29 +51,21 @@ struct CliqueArgs {
     int64_t big_words;        // words of one of the matrices there
     int big_stride;
     uint32_t* sets;           // 4 sets per warp for masked_cliques (global)
-    unsigned long long* cursor;     // 2: block items, warp roots
-    unsigned long long* results;
-    unsigned long long* busy;
+    ResultWords* words;       // cursors: block items, warp roots
 };
-
-__device__ __forceinline__ unsigned lt_mask() {
-    unsigned m;
-    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
-    return m;
-}
 
 // Is y (below x) a neighbour of x? Core rows answer with one bit; other
 // lists are searched below their own vertex.
 __device__ __forceinline__ bool adjacent(const CliqueArgs& a, int x, int y) {
-    if (x < a.core_n)
-        return (__ldg(a.core_bits + (size_t)x * a.core_words + (y >> 5)) >> (y & 31)) & 1u;
-    const int32_t* p = a.col + __ldg(a.row_ptr + x);
-    int n = __ldg(a.dplus + x), base = 0;
+    if (x < a.g.core_n)
+        return (__ldg(a.g.core_bits + (size_t)x * a.g.core_words + (y >> 5)) >> (y & 31)) & 1u;
+    const int32_t* p = a.g.col + __ldg(a.g.row_ptr + x);
+    int n = __ldg(a.g.dplus + x), base = 0;
     while (n > 0) {
         const int half = n >> 1;
         if (__ldg(p + base + half) < y) { base += half + 1; n -= half + 1; } else n = half;
     }
-    return base < __ldg(a.dplus + x) && __ldg(p + base) == y;
+    return base < __ldg(a.g.dplus + x) && __ldg(p + base) == y;
 }
 
 // Row i of the root's matrix, one warp: a ballot per 32 columns. The words
@@ -108,7 +91,7 @@ __device__ __forceinline__ void build_rows4(const CliqueArgs& a, const int32_t* 
 #pragma unroll
     for (int t = 0; t < 4; ++t) x[t] = __ldg(U + min(i0 + t, last));
     // ids grow with the position: the last row is outside the core first
-    if (x[3] >= a.core_n) {
+    if (x[3] >= a.g.core_n) {
         for (int i = i0; i <= last; ++i) build_row(a, U, i, M + (size_t)i * stride, stride, lane);
         return;
     }
@@ -119,7 +102,7 @@ __device__ __forceinline__ void build_rows4(const CliqueArgs& a, const int32_t* 
         const uint32_t bit = 1u << (y & 31);
         uint32_t v[4];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) v[t] = __ldg(a.core_bits + (size_t)x[t] * a.core_words + (y >> 5));
+        for (int t = 0; t < 4; ++t) v[t] = __ldg(a.g.core_bits + (size_t)x[t] * a.g.core_words + (y >> 5));
         uint32_t mine = 0;
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
@@ -225,7 +208,7 @@ __device__ __forceinline__ int expand(const uint32_t* S, int nw, int stride, Mem
     for (int w = 0; w < nw; ++w) {
         const uint32_t x = S[w];
         if (x >> lane & 1u) {
-            const int at = n + __popc(x & lt_mask()), p = 32 * w + lane;
+            const int at = n + __popc(x & lanes_below()), p = 32 * w + lane;
             mem.pos[at] = (uint16_t)p;
             mem.off[at] = (uint32_t)(p * stride);
         }
@@ -284,16 +267,12 @@ __device__ __forceinline__ void compact(const uint32_t* M, Members mem, int s, u
     }
 }
 
-__device__ __forceinline__ void clear(uint32_t* M, int words, int first, int step) {
-    for (int q = 4 * first; q < words; q += 4 * step) *reinterpret_cast<uint4*>(M + q) = make_uint4(0, 0, 0, 0);
-}
-
 // The members' matrix (s <= kWarpRows) in a warp's own buffer.
 __device__ __forceinline__ void compact_own(const uint32_t* M, Members mem, int s, uint32_t* out, int lane) {
     if (s <= 32) {
         compact32(M, mem, s, out, lane);
     } else {
-        clear(out, s * kWarpWords, lane, 32);
+        clear_words(out, s * kWarpWords, lane, 32);
         __syncwarp();
         compact(M, mem, s, out, kWarpWords, lane, 0, 1);
     }
@@ -365,7 +344,7 @@ __device__ __forceinline__ void block_row(const uint32_t* L, int stride, int i, 
     const int nw = (i >> 5) + 1, t = size_of(S, nw), cs = row_stride(t);
     __syncthreads();                                 // C, bmem and the warps' buffers are free
     if (warp == 0) expand(S, nw, stride, bmem, lane);
-    clear(C, t * cs, threadIdx.x, blockDim.x);
+    clear_words(C, t * cs, threadIdx.x, blockDim.x);
     if (threadIdx.x == 0) bs->next = 0;
     __syncthreads();
     compact(L, bmem, t, C, cs, lane, warp, nwarps);
@@ -453,7 +432,7 @@ __device__ __forceinline__ unsigned edges_of(const CliqueArgs& a, const int32_t*
         int x[4];
 #pragma unroll
         for (int t = 0; t < 4; ++t) x[t] = __ldg(U + min(i0 + t, last));
-        if (x[3] >= a.core_n) {
+        if (x[3] >= a.g.core_n) {
             for (int i = i0; i <= last; ++i)
                 for (int j = lane; j < i; j += 32) c += adjacent(a, __ldg(U + i), __ldg(U + j));
             continue;
@@ -462,7 +441,7 @@ __device__ __forceinline__ unsigned edges_of(const CliqueArgs& a, const int32_t*
             const int y = __ldg(U + j);
             uint32_t v[4];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) v[t] = __ldg(a.core_bits + (size_t)x[t] * a.core_words + (y >> 5));
+            for (int t = 0; t < 4; ++t) v[t] = __ldg(a.g.core_bits + (size_t)x[t] * a.g.core_words + (y >> 5));
 #pragma unroll
             for (int t = 0; t < 4; ++t)
                 if (j < i0 + t && i0 + t <= last) c += (v[t] >> (y & 31)) & 1u;
@@ -506,17 +485,17 @@ k_clique(const __grid_constant__ CliqueArgs a) {
     // large roots: one block each, largest first
     for (;;) {
         __syncthreads();
-        if (threadIdx.x == 0) s_item = atomicAdd(a.cursor, 1ull);
+        if (threadIdx.x == 0) s_item = atomicAdd(&a.words->cursor[0], 1ull);
         __syncthreads();
         const unsigned long long item = s_item;
         if (item >= (unsigned long long)a.n_block * a.parts) break;
-        const int v0 = __ldg(a.roots + item / a.parts), part = (int)(item % a.parts);
-        const int64_t rb = __ldg(a.row_ptr + v0);
-        const int n = __ldg(a.dplus + v0);
+        const int v0 = __ldg(a.g.roots + item / a.parts), part = (int)(item % a.parts);
+        const int64_t rb = __ldg(a.g.row_ptr + v0);
+        const int n = __ldg(a.g.dplus + v0);
         const int lo = (int)max((int64_t)0, min((int64_t)n, a.task_begin - rb));
         const int hi = (int)max((int64_t)0, min((int64_t)n, a.task_end - rb));
         if (lo >= hi) continue;
-        const int32_t* U = a.col + rb;
+        const int32_t* U = a.g.col + rb;
         if constexpr (K == 3) {
             acc.add(edges_of(a, U, lo, hi, warp, nwarps, lane));
         } else {
@@ -549,21 +528,21 @@ k_clique(const __grid_constant__ CliqueArgs a) {
     uint32_t* const own = area + Y::kList;
     for (;;) {
         unsigned long long t0 = 0;
-        if (lane == 0) t0 = atomicAdd(a.cursor + 1, (unsigned long long)a.warp_chunk);
+        if (lane == 0) t0 = atomicAdd(&a.words->cursor[1], (unsigned long long)a.warp_chunk);
         t0 = __shfl_sync(kFull, t0, 0);
         if (t0 >= n_warp) break;
         // lane l fetches root l of the chunk
         const bool have = lane < a.warp_chunk && t0 + lane < n_warp;
-        const int lv = have ? __ldg(a.roots + a.n_block + t0 + lane) : 0;
-        const int64_t lrb = have ? __ldg(a.row_ptr + lv) : 0;
-        const int ln = have ? __ldg(a.dplus + lv) : 0;
+        const int lv = have ? __ldg(a.g.roots + a.n_block + t0 + lane) : 0;
+        const int64_t lrb = have ? __ldg(a.g.row_ptr + lv) : 0;
+        const int ln = have ? __ldg(a.g.dplus + lv) : 0;
         for (int q = 0; q < a.warp_chunk; ++q) {
             const int64_t rb = __shfl_sync(kFull, lrb, q);
             const int n = __shfl_sync(kFull, ln, q);
             const int lo = (int)max((int64_t)0, min((int64_t)n, a.task_begin - rb));
             const int hi = (int)max((int64_t)0, min((int64_t)n, a.task_end - rb));
             if (lo >= hi || hi < K - 1) continue;
-            const int32_t* U = a.col + rb;
+            const int32_t* U = a.g.col + rb;
             if constexpr (K == 3) {
                 acc.add(edges_of(a, U, lo, hi, 0, 1, lane));
             } else {
@@ -577,8 +556,8 @@ k_clique(const __grid_constant__ CliqueArgs a) {
             }
         }
     }
-    flush(acc, a.results);
-    if (lane == 0) atomicAdd(a.busy, (unsigned long long)(clock64() - t_start));
+    flush(acc, a.words->total);
+    if (lane == 0) atomicAdd(&a.words->busy, (unsigned long long)(clock64() - t_start));
 }
 
 struct Variant {
@@ -629,13 +608,7 @@ gp_status run_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, ui
     GP_CUDA_TRY(cudaGetDevice(&dev));
     GP_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     CliqueArgs a = {};
-    a.row_ptr = g->row_ptr;
-    a.col = g->col;
-    a.core_bits = g->core_bits;
-    a.core_n = g->core_bits ? g->core_n : 0;
-    a.core_words = g->core_words;
-    a.roots = g->roots;
-    a.dplus = g->dplus;
+    a.g = device_graph(g);
     a.task_begin = job.task_begin;
     a.task_end = job.task_begin + job.ntasks;
     // a root goes to a whole block from |U| = 128 (the largest warp matrix);
@@ -661,7 +634,6 @@ gp_status run_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, ui
               : (int)std::max<int64_t>(1, std::min<int64_t>(k == 5 ? 8 : 64, (k == 5 ? 16 : 64) * blocks / a.n_block));
     const int64_t n_warp = a.n_roots - a.n_block;
     a.warp_chunk = (int)std::max<int64_t>(1, std::min<int64_t>(32, n_warp / (blocks * (threads / 32) * 8)));
-    // device buffer: results, cursors, busy cycles, then the large matrices
     const bool big = (k > 3 && g->max_dplus > kBlockRows) || (k > 4 && g->max_dplus > kWarpRows);
     if (big) {
         a.big_stride = row_stride(g->max_dplus);
@@ -670,44 +642,15 @@ gp_status run_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, ui
     const size_t big_b = big ? sizeof(uint32_t) * (size_t)blocks * (2 * (size_t)a.big_words + 2 * kMostRows) : 0;
     const size_t sets_b = k >= 6 && a.n_block > 0
         ? sizeof(uint32_t) * (size_t)blocks * (size_t)(threads / 32) * 4 * (kMostRows / 32) : 0;
-    const size_t bytes = 64 + big_b + sets_b;
-    char* mem = nullptr;
-    GP_CUDA_TRY(cudaMallocAsync((void**)&mem, bytes, st));
-    unsigned long long* words = reinterpret_cast<unsigned long long*>(mem);
-    a.results = words;
-    a.cursor = words + 2;
-    a.busy = words + 4;
-    a.big = reinterpret_cast<uint32_t*>(mem + 64);
-    a.sets = reinterpret_cast<uint32_t*>(mem + 64 + big_b);
-    cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-    unsigned long long h[5] = {};
-    cudaError_t e = cudaSuccess;
-    if (kernel_ms) {
-        e = cudaEventCreate(&ev0);
-        if (e == cudaSuccess) e = cudaEventCreate(&ev1);
-    }
-    if (e == cudaSuccess) e = cudaMemsetAsync(mem, 0, 64, st);
-    if (e == cudaSuccess && ev0) e = cudaEventRecord(ev0, st);
-    if (e == cudaSuccess) {
+    const gp_status rc = run_with_words(st, big_b + sets_b, kernel_ms, results, busy, "clique",
+                                        [&](ResultWords* words, char* mem) {
+        a.words = words;
+        a.big = reinterpret_cast<uint32_t*>(mem);
+        a.sets = reinterpret_cast<uint32_t*>(mem + big_b);
         fn<<<(unsigned)blocks, threads, smem, st>>>(a);
-        count_launch();
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess && ev1) e = cudaEventRecord(ev1, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h, words, sizeof(h), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e == cudaSuccess && ev1) e = cudaEventElapsedTime(kernel_ms, ev0, ev1);
-    if (ev0) cudaEventDestroy(ev0);
-    if (ev1) cudaEventDestroy(ev1);
-    cudaFreeAsync(mem, st);
-    if (e != cudaSuccess) {
-        set_error("clique kernel failed: %s", cudaGetErrorString(e));
-        return GP_ERR_CUDA;
-    }
-    results[0] = h[0];
-    results[1] = h[1];
-    if (busy) { busy[0] = h[4]; busy[1] = (uint64_t)blocks * (threads / 32); }
-    return GP_OK;
+    });
+    if (busy) busy[1] = (uint64_t)blocks * (threads / 32);
+    return rc;
 }
 
 }  // namespace gp

@@ -31,6 +31,8 @@ struct gp_graph {
     int32_t* roots = nullptr;     // device, n: vertices by dplus, largest first
     int32_t max_dplus = 0;
     int64_t roots_ge[32] = {};    // vertices with dplus >= 2^i
+    int64_t n_hubs = 0;           // degree-ordered graphs: vertices of degree > kHubDegree (a prefix)
+    int64_t max_root_words = 0;   // largest dplus x words of a row of degree bits (join.cu)
     std::mutex mu;
     bool tri_done = false;
     uint64_t tri_cnt = 0;         // ordered triangles (6 x triangles)
@@ -81,6 +83,12 @@ constexpr int32_t kCoreMax = 8192;
 // one per grab (degree-ordered graphs put them first).
 constexpr int32_t kHeavyDegree = 256;
 
+// Vertices above this degree are hubs for join.cu, whose warps take matrices
+// of at most this many columns; root matrices beyond kMostRootWords words
+// (16 MB) go to the general kernel.
+constexpr int32_t kHubDegree = 512;
+constexpr int64_t kMostRootWords = (int64_t)1 << 22;
+
 struct LaunchOpts {
     int warps_per_block = 8;
     int blocks_per_sm = 0;   // 0 = occupancy maximum
@@ -112,6 +120,13 @@ bool clique_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& op
 // The job's 128-bit total (clique.cu); kernel_ms and busy as for run_count.
 gp_status run_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, uint64_t* results,
                      float* kernel_ms = nullptr, uint64_t* busy = nullptr);
+
+// True when join.cu counts the job: an inclusion-exclusion plan of a clique
+// and vertices adjacent to all of it, on a degree-ordered graph whose root
+// matrices are small enough.
+bool join_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt);
+gp_status run_join(const CountJob& job, const gp_graph* g, cudaStream_t st, uint64_t* results,
+                   float* kernel_ms = nullptr, uint64_t* busy = nullptr);
 
 // run_count without allocating: results, job table and intermediate sets all
 // live in the caller's device buffer d_scratch (256-byte aligned); the grid

@@ -171,7 +171,9 @@ __global__ void k_core_bits(const int64_t* __restrict__ row_ptr, const int32_t* 
 // dplus[u]: entries of row u below u (a prefix of the sorted row); the keys
 // and ids to sort by it.
 __global__ void k_dplus(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int32_t n,
-                        int32_t* __restrict__ dplus, int32_t* __restrict__ ids) {
+                        int32_t* __restrict__ dplus, int32_t* __restrict__ ids,
+                        unsigned long long* __restrict__ max_words) {
+    unsigned long long best = 0;
     for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n;
          u += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = row_ptr[u];
@@ -182,13 +184,18 @@ __global__ void k_dplus(const int64_t* __restrict__ row_ptr, const int32_t* __re
         }
         dplus[u] = (int32_t)(lo - b);
         ids[u] = (int32_t)u;
+        best = max(best, (unsigned long long)(lo - b) * (4 * (unsigned long long)((row_ptr[u + 1] - b + 127) >> 7)));
     }
+    for (int o = 16; o; o >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, o));
+    if ((threadIdx.x & 31) == 0 && best) atomicMax(max_words, best);
 }
 
 // What the host keeps about the finished graph.
 struct GraphInfo {
     int64_t roots_ge[32];     // entries of the non-increasing `sorted` that are >= 2^i
     int64_t heavy_end;        // degree-ordered graphs: first entry of the first row shorter than kHeavyDegree
+    int64_t n_hubs;           // degree-ordered graphs: rows longer than kHubDegree
+    unsigned long long max_root_words;
     int32_t max_dplus;
     int32_t max_deg;
 };
@@ -198,19 +205,21 @@ struct GraphInfo {
 __global__ void k_graph_info(const int32_t* __restrict__ sorted, const int64_t* __restrict__ row_ptr, int32_t n,
                              bool ordered, GraphInfo* __restrict__ out) {
     const int i = threadIdx.x;
-    if (i > 32) return;
+    if (i > 33) return;
     if (i == 32) {
         out->max_dplus = sorted[0];
         if (ordered) out->max_deg = (int32_t)(row_ptr[1] - row_ptr[0]);
     }
-    int32_t lo = 0, hi = (i == 32 && !ordered) ? 0 : n;
+    int32_t lo = 0, hi = (i >= 32 && !ordered) ? 0 : n;
     while (lo < hi) {
         const int32_t mid = lo + ((hi - lo) >> 1);
-        const bool in = i == 32 ? row_ptr[mid + 1] - row_ptr[mid] >= kHeavyDegree
+        const int64_t deg = i >= 32 ? row_ptr[mid + 1] - row_ptr[mid] : 0;
+        const bool in = i == 32 ? deg >= kHeavyDegree : i == 33 ? deg > kHubDegree
                                 : (int64_t)sorted[mid] >= ((int64_t)1 << i);
         if (in) lo = mid + 1; else hi = mid;
     }
     if (i == 32) out->heavy_end = ordered ? row_ptr[lo] : 0;
+    else if (i == 33) out->n_hubs = lo;
     else out->roots_ge[i] = lo;
 }
 
@@ -258,7 +267,8 @@ gp_status finish_graph(gp_graph* g, cudaStream_t st) {
     GP_CUDA_TRY(info.alloc(sizeof(GraphInfo)));
     GraphInfo* d_info = info.as<GraphInfo>();
     GP_CUDA_TRY(cudaMemsetAsync(d_info, 0, sizeof(GraphInfo), st));
-    k_dplus<<<blocks_for(n), kThreads, 0, st>>>(g->row_ptr, g->col, n, g->dplus, ids.as<int32_t>());
+    k_dplus<<<blocks_for(n), kThreads, 0, st>>>(g->row_ptr, g->col, n, g->dplus, ids.as<int32_t>(),
+                                               &d_info->max_root_words);
     size_t tb = 0;
     const int bits = std::max(1, bits_for((uint64_t)n - 1));
     GP_CUDA_TRY(cub::DeviceRadixSort::SortPairsDescending(nullptr, tb, g->dplus, keys.as<int32_t>(), ids.as<int32_t>(),
@@ -282,6 +292,8 @@ gp_status finish_graph(gp_graph* g, cudaStream_t st) {
     g->max_dplus = h.max_dplus;
     g->max_deg = h.max_deg;
     g->heavy_end = h.heavy_end;
+    g->n_hubs = h.n_hubs;
+    g->max_root_words = (int64_t)h.max_root_words;
     return GP_OK;
 }
 

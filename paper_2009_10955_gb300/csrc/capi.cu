@@ -187,13 +187,15 @@ LaunchOpts launch_opts(const gp_count_opts* o) {
     return lo;
 }
 
-// Jobs that the local bit matrices of clique.cu and join.cu count.
+// Jobs that a kernel of their own counts (clique.cu, join.cu, wedge.cu).
 bool local_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& lo) {
-    return clique_applies(job, g, lo) || join_applies(job, g, lo);
+    return clique_applies(job, g, lo) || join_applies(job, g, lo) || wedge_applies(job, g, lo);
 }
 
 gp_status run_local(const CountJob& job, const gp_graph* g, cudaStream_t st, uint64_t* res, float* ms, uint64_t* busy) {
-    return job.plan.iep ? run_join(job, g, st, res, ms, busy) : run_clique(job, g, st, res, ms, busy);
+    if (!job.plan.iep) return run_clique(job, g, st, res, ms, busy);
+    return wedge_applies(job, g, LaunchOpts()) ? run_wedge(job, g, st, res, ms, busy)
+                                               : run_join(job, g, st, res, ms, busy);
 }
 
 bool opts_ok(const gp_count_opts* o) {
@@ -666,7 +668,7 @@ gp_status gp_count_batch(gp_graph* const* graphs, const gp_schedules* const* sch
     GP_CUDA_TRY(cudaGetDevice(&dev));
     GP_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     const int user_chunk = lo.chunk;
-    for (int32_t j = 0; j < njobs; ++j) {     // local bit matrices: a launch each (a block works on one root)
+    for (int32_t j = 0; j < njobs; ++j) {     // a kernel of their own: a launch each
         if (key[j] != -1) continue;
         float jms = 0.f;
         uint64_t jbusy[2] = {0, 0};

@@ -613,8 +613,9 @@ gp_status run_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, ui
     a.task_end = job.task_begin + job.ntasks;
     // a root goes to a whole block from |U| = 128 (the largest warp matrix);
     // from fewer for 6- and 7-cliques, whose work grows with a higher power
-    // of |U|.
-    const int block_class = k <= 5 ? 7 : k == 6 ? 6 : 5;
+    // of |U|, and where the smaller roots are no more than the SMs
+    int block_class = k <= 5 ? 7 : k == 6 ? 6 : 5;
+    while (k >= 5 && block_class > 4 && g->roots_ge[block_class - 1] <= 2 * (int64_t)nsm) --block_class;
     a.n_block = g->roots_ge[block_class];
     a.n_roots = g->roots_ge[k <= 4 ? 1 : 2];
     const Variant var = variant_for(k);

@@ -128,6 +128,12 @@ bool join_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt)
 gp_status run_join(const CountJob& job, const gp_graph* g, cudaStream_t st, uint64_t* results,
                    float* kernel_ms = nullptr, uint64_t* busy = nullptr);
 
+// True when wedge.cu counts the job: the House's inclusion-exclusion plan
+// over all tasks.
+bool wedge_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt);
+gp_status run_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, uint64_t* results,
+                    float* kernel_ms = nullptr, uint64_t* busy = nullptr);
+
 // run_count without allocating: results, job table and intermediate sets all
 // live in the caller's device buffer d_scratch (256-byte aligned); the grid
 // shrinks to what that buffer holds. GP_ERR_SCRATCH when not even one block

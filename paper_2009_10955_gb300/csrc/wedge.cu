@@ -1,0 +1,193 @@
+// wedge.cu -- the House's two-loop inclusion-exclusion count with its sums
+// exchanged.
+//
+// The plan binds an edge (v0, v1) and a neighbour v2 of one end p; the inner
+// sets are F = N(v_q) ∩ N(v2), q the other end, and O = N(v0) ∩ N(v1)
+// (Section IV-D). Written out, with t = |O| and W(a, b) = |N(a) ∩ N(b)|, the
+// sum over v2 of (|F| - 1)(t - [v2 in O]) - |F ∩ O| needs W(v_q, v2) for all
+// wedges v_q - v_p - v2, which the general kernel intersects anew for every
+// one of them. Here a block takes one vertex a, counts W(a, .) for all
+// vertices at once by walking the lists of its neighbours into an array of
+// counters, and reads off, for each neighbour b above a,
+//   t = W(a, b),  P = sum of W(a, x) over the neighbours x of b.
+// Over the whole graph the terms |F ∩ O| add up to the same sum of supports
+// from both ends of every triangle's edges, so that
+//   total = sum over edges of t (P - d(a) - d(b) + 3) - 2 t^2.
+//
+// What bounds it: the counter updates, sum of squared degrees in all (shared
+// memory atomics where n counters fit, L2 atomics otherwise). Taking b above
+// a reads the shorter lists of a degree-ordered graph.
+#include <algorithm>
+
+#include "acc.cuh"
+#include "bits.cuh"
+#include "engine.h"
+
+namespace gp {
+
+namespace {
+
+// Lists longer than this are walked by the whole block, shorter ones by a
+// warp each (in a degree-ordered graph the long ones come first in a row).
+constexpr int kLongList = 1024;
+
+struct WedgeArgs {
+    DeviceGraph g;
+    int32_t n;
+    bool ordered;
+    uint32_t* counters;        // n per block, zero (null: in shared memory)
+    ResultWords* words;        // cursor: vertices
+};
+
+template <bool kShared>
+__global__ void __launch_bounds__(1024)
+k_wedge(const __grid_constant__ WedgeArgs a) {
+    extern __shared__ __align__(16) uint32_t smem[];
+    __shared__ unsigned long long s_item;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const long long t_start = clock64();
+    uint32_t* const y = kShared ? smem : a.counters + (size_t)blockIdx.x * a.n;
+    Acc acc;
+    for (;;) {
+        __syncthreads();                             // the last vertex's counters are done with
+        if (threadIdx.x == 0) s_item = atomicAdd(&a.words->cursor[0], 1ull);
+        if (kShared)
+            for (int i = 4 * threadIdx.x; i < a.n; i += 4 * blockDim.x)
+                *reinterpret_cast<uint4*>(y + i) = make_uint4(0, 0, 0, 0);
+        __syncthreads();
+        if (s_item >= (unsigned long long)a.n) break;
+        const int v = (int)s_item;
+        const int64_t rb = __ldg(a.g.row_ptr + v);
+        const int d = (int)(__ldg(a.g.row_ptr + v + 1) - rb), above = __ldg(a.g.dplus + v);
+        if (d < 2) continue;
+        if (above == d) continue;                    // no neighbour above: nothing to read off
+        // the lists of the neighbours, in two passes where counters are global
+        // (count, then back to zero)
+        auto walk = [&](auto touch) {
+            int first = 0;
+            for (; a.ordered && first < d; ++first) {
+                const int u = __ldg(a.g.col + rb + first);
+                const int64_t b = __ldg(a.g.row_ptr + u), e = __ldg(a.g.row_ptr + u + 1);
+                if (e - b <= kLongList) break;
+                for (int64_t i = b + threadIdx.x; i < e; i += blockDim.x) touch(__ldg(a.g.col + i));
+            }
+            // lane l holds the l-th of this warp's next 32 neighbours
+            for (int base = first + warp; base < d; base += 32 * nwarps) {
+                const int mine = base + lane * nwarps;
+                int64_t b = 0;
+                int len = 0;
+                if (mine < d) {
+                    const int u = __ldg(a.g.col + rb + mine);
+                    b = __ldg(a.g.row_ptr + u);
+                    len = (int)(__ldg(a.g.row_ptr + u + 1) - b);
+                }
+                const int count = min(32, (d - base + nwarps - 1) / nwarps);
+                for (int q = 0; q < count; ++q) {
+                    const int64_t qb = __shfl_sync(kAllLanes, b, q);
+                    const int ql = __shfl_sync(kAllLanes, len, q);
+                    for (int i = lane; i < ql; i += 32) touch(__ldg(a.g.col + qb + i));
+                }
+            }
+        };
+        walk([&](int w) { atomicAdd(y + w, 1u); });
+        __syncthreads();
+        // the neighbours above v, eight lanes each
+        const int sub = threadIdx.x & 7, groups = blockDim.x >> 3;
+        for (int base = above; base < d; base += groups) {
+            const int i = base + (threadIdx.x >> 3);
+            unsigned t = 0;
+            unsigned long long P = 0;
+            int db = 0;
+            if (i < d) {
+                const int b = __ldg(a.g.col + rb + i);
+                t = kShared ? y[b] : __ldcg(y + b);
+                if (t) {
+                    const int64_t e0 = __ldg(a.g.row_ptr + b);
+                    db = (int)(__ldg(a.g.row_ptr + b + 1) - e0);
+                    for (int x = sub; x < db; x += 8) {
+                        const int w = __ldg(a.g.col + e0 + x);
+                        P += kShared ? y[w] : __ldcg(y + w);
+                    }
+                }
+            }
+            for (int o = 4; o; o >>= 1) P += __shfl_xor_sync(kAllLanes, P, o);
+            if (sub == 0 && t) {
+                const unsigned long long more = P + 3, less = (unsigned long long)d + (unsigned)db + 2ull * t;
+                const unsigned __int128 plus = (unsigned __int128)t * more, minus = (unsigned __int128)t * less;
+                const unsigned __int128 diff = plus - minus;
+                acc.add128((unsigned long long)diff, (unsigned long long)(diff >> 64));
+            }
+        }
+        if (!kShared) {
+            __syncthreads();
+            walk([&](int w) { __stcg(y + w, 0u); });
+        }
+    }
+    flush(acc, a.words->total);
+    if (lane == 0) atomicAdd(&a.words->busy, (unsigned long long)(clock64() - t_start));
+}
+
+// The House as an inclusion-exclusion plan: v2 joined to one end of the edge
+// (v0, v1), one inner vertex to the other end and v2, the other to both ends;
+// the only restriction left orders v0 and v1.
+bool is_house_plan(const GpPlan& P) {
+    if (P.labeled || P.k != 5 || P.iep != 2) return false;
+    if (P.lvl[1].op_mask != 1 || (P.lvl[1].lo_mask | P.lvl[1].hi_mask) != 1) return false;
+    for (int d = 2; d < 5; ++d)
+        if (P.lvl[d].lo_mask || P.lvl[d].hi_mask) return false;
+    const int far = P.lvl[2].op_mask == 1 ? 2 : P.lvl[2].op_mask == 2 ? 1 : 0;   // bit of the end not joined to v2
+    const int f = far | 4, o = 3;
+    return far && ((P.lvl[3].op_mask == f && P.lvl[4].op_mask == o) || (P.lvl[3].op_mask == o && P.lvl[4].op_mask == f));
+}
+
+}  // namespace
+
+bool wedge_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt) {
+    if (opt.stats || opt.no_core || opt.bitmap_mode != 2 || opt.budget_cycles > 0 || opt.task_cycles > 0) return false;
+    // the exchanged sums hold for all tasks together
+    return g->dplus && job.task_begin == 0 && job.ntasks == g->nnz && is_house_plan(job.plan);
+}
+
+gp_status run_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, uint64_t* results, float* kernel_ms,
+                    uint64_t* busy) {
+    (void)job;
+    int dev = 0, nsm = 0;
+    GP_CUDA_TRY(cudaGetDevice(&dev));
+    GP_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    WedgeArgs a = {};
+    a.g = device_graph(g);
+    a.n = g->n;
+    a.ordered = g->perm != nullptr;
+    // counters in shared memory up to 56 K vertices: several blocks an SM
+    // while they fit, one of 1024 threads beyond
+    const size_t bytes = ((size_t)g->n * sizeof(uint32_t) + 15) & ~(size_t)15;
+    const bool shared = bytes <= 224 * 1024;
+    const int threads = shared && bytes > 110 * 1024 ? 1024 : 512;
+    auto fn = shared ? k_wedge<true> : k_wedge<false>;
+    const size_t smem = shared ? bytes : 0;
+    if (smem > 40 * 1024)
+        GP_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int occ = 0;
+    GP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem));
+    int64_t blocks = (int64_t)nsm * std::max(occ, 1);
+    blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, g->n));
+    size_t extra = 0;
+    if (!shared) {
+        size_t free_b = 0, total_b = 0;
+        GP_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
+        while (blocks > 1 && bytes * (size_t)blocks > free_b / 4) blocks = (blocks + 1) / 2;
+        extra = sizeof(uint32_t) * (size_t)g->n * (size_t)blocks;
+    }
+    cudaError_t e = cudaSuccess;
+    const gp_status rc = run_with_words(st, extra, kernel_ms, results, busy, "wedge", [&](ResultWords* words, char* mem) {
+        a.words = words;
+        a.counters = reinterpret_cast<uint32_t*>(mem);
+        if (extra) e = cudaMemsetAsync(mem, 0, extra, st);
+        fn<<<(unsigned)blocks, threads, smem, st>>>(a);
+    });
+    if (rc == GP_OK && e != cudaSuccess) { set_error("wedge counters: %s", cudaGetErrorString(e)); return GP_ERR_CUDA; }
+    if (busy) busy[1] = (uint64_t)blocks * (threads / 32);
+    return rc;
+}
+
+}  // namespace gp

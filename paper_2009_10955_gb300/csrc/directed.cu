@@ -12,23 +12,25 @@
 // Graph: every arc once, as sorted out-lists and sorted in-lists (CSR each),
 // built on the device with one radix sort per direction (CUB).
 //
-// Count kernel: a persistent grid, one warp per root vertex taken from a
-// global cursor; the warp runs the matching order depth-first. At depth d
-// the candidates are the out- or in-list of the image of one earlier vertex
-// joined to it by an arc; the 32 lanes test 32 candidates at a time (distinct
-// from the matched vertices, the other arcs to matched vertices by binary
-// search in out-lists, the restrictions as comparisons) and a ballot keeps
-// the survivors; at the last depth the survivors are counted, not visited.
+// Count kernel: every arc that can take the first two vertices of the matching
+// order is one task; a persistent grid's warps take them from a global cursor
+// and run the remaining loops depth-first. Each matched vertex joined to the
+// next one contributes a sorted list that holds its candidates; the shortest
+// is walked, cut to the window the restrictions leave, and its elements are
+// looked up in the others by binary search. The last two depths run eight
+// lanes to a candidate: the last one is counted, not visited.
 #include <cub/device/device_radix_sort.cuh>
 #include <cub/device/device_select.cuh>
 
 #include <algorithm>
+#include <climits>
 #include <cstring>
 #include <memory>
 #include <new>
 #include <string>
 #include <vector>
 
+#include "acc.cuh"
 #include "engine.h"
 #include "planner.h"
 
@@ -223,16 +225,14 @@ void free_dgraph(gp_dgraph* g) {
 
 // ------------------------------------------------------------------ plan
 
-constexpr int kMaxChecks = 2 * GP_MAX_K;
+constexpr int kMaxCons = 2 * GP_MAX_K;
 
 struct DPlan {
     int k;
     int order[GP_MAX_K];
-    int anchor[GP_MAX_K];                  // earlier depth whose image's list holds the candidates
-    int anchor_out[GP_MAX_K];              // 1: its out-list, 0: its in-list
-    int nchk[GP_MAX_K];
-    int chk_depth[GP_MAX_K][kMaxChecks];   // further arcs to matched vertices ...
-    int chk_fwd[GP_MAX_K][kMaxChecks];     // ... 1: image(j) -> v, 0: v -> image(j)
+    int ncon[GP_MAX_K];                    // arcs that join depth d to matched vertices:
+    int con_depth[GP_MAX_K][kMaxCons];     // the other end's depth j, and
+    int con_out[GP_MAX_K][kMaxCons];       // 1: image(j) -> v, 0: v -> image(j)
     int nres[GP_MAX_K];
     int res_depth[GP_MAX_K][GP_MAX_K];     // restrictions acting at depth d
     int res_gt[GP_MAX_K][GP_MAX_K];        // 1: v > image(j), 0: v < image(j)
@@ -256,21 +256,12 @@ bool compile_dplan(const gp_dpattern& p, const int8_t* sched, ResMask res, DPlan
     }
     for (int d = 1; d < k; ++d) {
         const int x = P.order[d];
-        P.anchor[d] = -1;
         for (int j = 0; j < d; ++j) {
             const int y = P.order[j];
-            const bool to_x = p.arc[y][x], from_x = p.arc[x][y];
-            if (!to_x && !from_x) continue;
-            if (P.anchor[d] < 0) {
-                P.anchor[d] = j;
-                P.anchor_out[d] = to_x ? 1 : 0;   // y -> x: x is among the out-arcs of image(y)
-                if (to_x && from_x) { P.chk_depth[d][P.nchk[d]] = j; P.chk_fwd[d][P.nchk[d]++] = 0; }
-                continue;
-            }
-            if (to_x) { P.chk_depth[d][P.nchk[d]] = j; P.chk_fwd[d][P.nchk[d]++] = 1; }
-            if (from_x) { P.chk_depth[d][P.nchk[d]] = j; P.chk_fwd[d][P.nchk[d]++] = 0; }
+            if (p.arc[y][x]) { P.con_depth[d][P.ncon[d]] = j; P.con_out[d][P.ncon[d]++] = 1; }
+            if (p.arc[x][y]) { P.con_depth[d][P.ncon[d]] = j; P.con_out[d][P.ncon[d]++] = 0; }
         }
-        if (P.anchor[d] < 0) { err = "every prefix of the order must be weakly connected"; return false; }
+        if (P.ncon[d] == 0) { err = "every prefix of the order must be weakly connected"; return false; }
     }
     for (int a = 0; a < k; ++a)
         for (int b = 0; b < k; ++b) {
@@ -286,92 +277,203 @@ bool compile_dplan(const gp_dpattern& p, const int8_t* sched, ResMask res, DPlan
 
 // ---------------------------------------------------------------- kernel
 
-__device__ __forceinline__ bool arc_in(const int64_t* __restrict__ out_ptr, const int32_t* __restrict__ out_col,
-                                       int32_t u, int32_t v) {   // u -> v ?
-    int64_t lo = out_ptr[u], hi = out_ptr[u + 1];
-    const int64_t end = hi;
-    while (lo < hi) {
-        const int64_t mid = lo + (hi - lo) / 2;
-        if (out_col[mid] < v) lo = mid + 1; else hi = mid;
-    }
-    return lo < end && out_col[lo] == v;
+struct DLists {
+    const int64_t* __restrict__ out_ptr;
+    const int32_t* __restrict__ out_col;
+    const int64_t* __restrict__ in_ptr;
+    const int32_t* __restrict__ in_col;
+};
+
+struct DList { const int32_t* p; int n; };
+
+__device__ __forceinline__ DList list_of(const DLists& g, int out, int u) {
+    const int64_t* ptr = out ? g.out_ptr : g.in_ptr;
+    const int64_t b = __ldg(ptr + u);
+    return {(out ? g.out_col : g.in_col) + b, (int)(__ldg(ptr + u + 1) - b)};
 }
 
+__device__ __forceinline__ int first_not_below(DList a, int x) {
+    int base = 0, n = a.n;
+    while (n > 0) {
+        const int half = n >> 1;
+        if (__ldg(a.p + base + half) < x) { base += half + 1; n -= half + 1; } else n = half;
+    }
+    return base;
+}
+
+// The list that depth d walks: the shortest of those its arcs give, inside
+// the restrictions' window; *which receives the arc it stands for. img(j) is
+// the vertex matched at depth j.
+template <class Img>
+__device__ __forceinline__ DList walk_list(const DPlan& P, const DLists& g, int d, Img img, int* which) {
+    DList best = list_of(g, P.con_out[d][0], img(P.con_depth[d][0]));
+    *which = 0;
+    for (int c = 1; c < P.ncon[d]; ++c) {
+        const DList l = list_of(g, P.con_out[d][c], img(P.con_depth[d][c]));
+        if (l.n < best.n) { best = l; *which = c; }
+    }
+    int lo = -1, hi = INT_MAX;                     // lo < v < hi
+    for (int r = 0; r < P.nres[d]; ++r) {
+        const int o = img(P.res_depth[d][r]);
+        if (P.res_gt[d][r]) lo = max(lo, o); else hi = min(hi, o);
+    }
+    if (lo >= 0) { const int b = first_not_below(best, lo + 1); best.p += b; best.n -= b; }
+    if (hi != INT_MAX) best.n = first_not_below(best, hi);
+    return best;
+}
+
+// May v (taken from the list of arc `which`, inside the window) be matched at
+// depth d: none of the matched vertices, joined by all other arcs?
+template <class Img>
+__device__ __forceinline__ bool fits(const DPlan& P, const DLists& g, int d, Img img, int which, int v) {
+    for (int j = 0; j < d; ++j)
+        if (img(j) == v) return false;
+    for (int c = 0; c < P.ncon[d]; ++c) {
+        if (c == which) continue;
+        const DList l = list_of(g, P.con_out[d][c], img(P.con_depth[d][c]));
+        const int at = first_not_below(l, v);
+        if (at >= l.n || __ldg(l.p + at) != v) return false;
+    }
+    return true;
+}
+
+// Does the arc u -> v of a task (or v -> u: con_out[1][0]) carry what else
+// depth 1 asks for?
+__device__ __forceinline__ bool task_fits(const DPlan& P, const DLists& g, int u, int v) {
+    for (int r = 0; r < P.nres[1]; ++r)
+        if (P.res_gt[1][r] ? v <= u : v >= u) return false;
+    return fits(P, g, 1, [&](int) { return u; }, 0, v);
+}
+
+// Lanes to a last-depth list, and the length from which the whole warp takes
+// it instead (a few rounds of eight lanes cost less than the warp's turn).
+constexpr int kGroup = 8;
+constexpr int kGroupMost = 256;
+
+// Last-depth counts for the candidates of depth k - 2 in `mask` (bit l: lane
+// l's x; u: its depth-0 vertex), four at a time, eight lanes each. Vertices of
+// the depths between are in `mid`.
+__device__ __forceinline__ unsigned long long count_last_depth(const DPlan& P, const DLists& g, const int* mid,
+                                                               int u, int x, unsigned mask, int lane) {
+    const int L = P.k - 1, sub = lane & (kGroup - 1), grp = lane / kGroup;
+    unsigned long long cnt = 0;
+    while (mask) {
+        int src = -1;
+#pragma unroll
+        for (int q = 0; q < 32 / kGroup; ++q)
+            if (mask) {
+                if (q == grp) src = __ffs(mask) - 1;
+                mask &= mask - 1;
+            }
+        const int gu = __shfl_sync(kAll, u, max(src, 0)), gx = __shfl_sync(kAll, x, max(src, 0));
+        auto img = [&](int j) { return j == L - 1 ? gx : j == 0 ? gu : mid[j]; };
+        int which = 0;
+        DList l{nullptr, 0};
+        if (src >= 0) l = walk_list(P, g, L, img, &which);
+        const bool large = l.n > kGroupMost;
+        if (!large)
+            for (int i = sub; i < l.n; i += kGroup) cnt += fits(P, g, L, img, which, __ldg(l.p + i));
+        unsigned big = __ballot_sync(kAll, large && sub == 0);
+        while (big) {
+            const int from = __ffs(big) - 1;
+            big &= big - 1;
+            const int wu = __shfl_sync(kAll, gu, from), wx = __shfl_sync(kAll, gx, from);
+            auto wimg = [&](int j) { return j == L - 1 ? wx : j == 0 ? wu : mid[j]; };
+            const DList wl = walk_list(P, g, L, wimg, &which);
+            for (int i = lane; i < wl.n; i += 32) cnt += fits(P, g, L, wimg, which, __ldg(wl.p + i));
+        }
+    }
+    return cnt;
+}
+
+// One warp per task; three-vertex patterns take 32 tasks at a time.
 __global__ void __launch_bounds__(kDThreads)
-k_dcount(const __grid_constant__ DPlan P, int32_t n, const int64_t* __restrict__ out_ptr, const int32_t* __restrict__ out_col,
-         const int64_t* __restrict__ in_ptr, const int32_t* __restrict__ in_col,
+k_dcount(const __grid_constant__ DPlan P, int32_t n, int64_t narcs, const __grid_constant__ DLists g, int chunk,
          unsigned long long* __restrict__ cursor, unsigned long long* __restrict__ result) {
+    __shared__ int s_img[kDThreads / 32][GP_MAX_K];
     const int lane = threadIdx.x & 31;
-    unsigned long long lo_acc = 0, hi_acc = 0;      // lane 0's 128-bit sum
-    int32_t img[GP_MAX_K];
-    const int32_t* lst[GP_MAX_K];
-    int64_t len[GP_MAX_K], next[GP_MAX_K], taken[GP_MAX_K];
-    unsigned mask[GP_MAX_K];
+    int* const mid = s_img[threadIdx.x >> 5];
+    const int64_t* const ptr = P.con_out[1][0] ? g.out_ptr : g.in_ptr;
+    const int32_t* const col = P.con_out[1][0] ? g.out_col : g.in_col;
+    Acc acc;
     for (;;) {
-        unsigned long long root = 0;
-        if (lane == 0) root = atomicAdd(cursor, 1ull);
-        root = __shfl_sync(kAll, root, 0);
-        if (root >= (unsigned long long)n) break;
-        img[0] = (int32_t)root;
-        int d = 1;
-        auto open = [&](int dd) {
-            const int32_t a = img[P.anchor[dd]];
-            const int64_t* ptr = P.anchor_out[dd] ? out_ptr : in_ptr;
-            const int32_t* col = P.anchor_out[dd] ? out_col : in_col;
-            lst[dd] = col + ptr[a];
-            len[dd] = ptr[a + 1] - ptr[a];
-            next[dd] = 0;
-            mask[dd] = 0;
-        };
-        open(1);
-        while (d >= 1) {
-            if (mask[d] == 0) {
-                if (next[d] >= len[d]) { --d; continue; }
-                const int64_t i = next[d] + lane;
-                bool ok = false;
-                if (i < len[d]) {
-                    const int32_t v = lst[d][i];
-                    ok = true;
-                    for (int j = 0; j < d; ++j) ok = ok && (img[j] != v);                 // injective
-                    for (int c = 0; c < P.nchk[d] && ok; ++c) {                         // other arcs
-                        const int32_t o = img[P.chk_depth[d][c]];
-                        ok = P.chk_fwd[d][c] ? arc_in(out_ptr, out_col, o, v) : arc_in(out_ptr, out_col, v, o);
+        unsigned long long t0 = 0;
+        if (lane == 0) t0 = atomicAdd(cursor, (unsigned long long)chunk);
+        t0 = __shfl_sync(kAll, t0, 0);
+        if ((int64_t)t0 >= narcs) break;
+        const int64_t end = min((int64_t)t0 + chunk, narcs);
+        // a lane per task: its first two vertices
+        const int64_t e = (int64_t)t0 + lane;
+        int u = 0, v = 0;
+        bool ok = false;
+        if (e < end) {
+            int lo = 0, hi = n - 1;                  // row of entry e
+            while (lo < hi) {
+                const int m = lo + (hi - lo + 1) / 2;
+                if (__ldg(ptr + m) <= e) lo = m; else hi = m - 1;
+            }
+            u = lo;
+            v = __ldg(col + e);
+            ok = task_fits(P, g, u, v);
+        }
+        unsigned tasks = __ballot_sync(kAll, ok);
+        if (P.k == 3) {
+            acc.add(count_last_depth(P, g, mid, u, v, tasks, lane));
+            continue;
+        }
+        while (tasks) {
+            const int from = __ffs(tasks) - 1;
+            tasks &= tasks - 1;
+            const int t_u = __shfl_sync(kAll, u, from), t_v = __shfl_sync(kAll, v, from);
+            __syncwarp();
+            if (lane == 0) { mid[0] = t_u; mid[1] = t_v; }
+            __syncwarp();
+            auto img = [&](int j) { return mid[j]; };
+            DList lst[GP_MAX_K];
+            int next[GP_MAX_K], which[GP_MAX_K], held[GP_MAX_K];
+            unsigned mask[GP_MAX_K];
+            int d = 2;
+            lst[2] = walk_list(P, g, 2, img, &which[2]);
+            next[2] = 0;
+            mask[2] = 0;
+            while (d >= 2) {
+                if (mask[d] == 0) {
+                    if (next[d] >= lst[d].n) { --d; continue; }
+                    const int i = next[d] + lane;
+                    int x = 0;
+                    bool in = false;
+                    if (i < lst[d].n) {
+                        x = __ldg(lst[d].p + i);
+                        in = fits(P, g, d, img, which[d], x);
                     }
-                    for (int r = 0; r < P.nres[d] && ok; ++r) {                         // restrictions
-                        const int32_t o = img[P.res_depth[d][r]];
-                        ok = P.res_gt[d][r] ? (v > o) : (v < o);
-                    }
-                }
-                const unsigned m = __ballot_sync(kAll, ok);
-                taken[d] = next[d];
-                next[d] += 32;
-                if (d == P.k - 1) {                                   // last depth: count
-                    if (lane == 0) {
-                        const unsigned long long add = (unsigned long long)__popc(m);
-                        lo_acc += add;
-                        hi_acc += (lo_acc < add) ? 1ull : 0ull;
+                    const unsigned m = __ballot_sync(kAll, in);
+                    next[d] += 32;
+                    if (d == P.k - 2) {
+                        acc.add(count_last_depth(P, g, mid, t_u, x, m, lane));
+                    } else {
+                        mask[d] = m;
+                        held[d] = x;
                     }
                     continue;
                 }
-                mask[d] = m;
-                continue;
+                const int b = __ffs(mask[d]) - 1;
+                mask[d] &= mask[d] - 1;
+                const int x = __shfl_sync(kAll, held[d], b);
+                __syncwarp();
+                if (lane == 0) mid[d] = x;
+                __syncwarp();
+                ++d;
+                lst[d] = walk_list(P, g, d, img, &which[d]);
+                next[d] = 0;
+                mask[d] = 0;
             }
-            const int b = __ffs(mask[d]) - 1;
-            mask[d] &= mask[d] - 1;
-            img[d] = lst[d][taken[d] + b];
-            ++d;
-            open(d);
         }
     }
-    if (lane == 0 && (lo_acc | hi_acc)) {
-        const unsigned long long old = atomicAdd(result, lo_acc);
-        const unsigned long long carry = (old + lo_acc < old) ? 1ull : 0ull;
-        if (hi_acc + carry) atomicAdd(result + 1, hi_acc + carry);
-    }
+    flush(acc, result);
 }
 
 gp_status run_dcount(const gp_dgraph* g, const DPlan& P, uint64_t div, cudaStream_t st, uint64_t* out) {
-    if (g->n == 0) { *out = 0; return GP_OK; }
+    if (g->narcs == 0) { *out = 0; return GP_OK; }
     DScratch mem(st);
     GP_CUDA_TRY(mem.alloc(3 * sizeof(unsigned long long)));
     GP_CUDA_TRY(cudaMemsetAsync(mem.p, 0, 3 * sizeof(unsigned long long), st));
@@ -380,8 +482,15 @@ gp_status run_dcount(const gp_dgraph* g, const DPlan& P, uint64_t div, cudaStrea
     int dev = 0, nsm = 0;
     GP_CUDA_TRY(cudaGetDevice(&dev));
     GP_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    const int blocks = std::max(1, nsm * 8);
-    k_dcount<<<blocks, kDThreads, 0, st>>>(P, g->n, g->out_ptr, g->out_col, g->in_ptr, g->in_col, cursor, res);
+    int occ = 0;
+    GP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_dcount, kDThreads, 0));
+    const int blocks = nsm * std::max(occ, 1);
+    // tasks per grab: three-vertex patterns want full warps; the others up to
+    // 8 (a hub's arcs follow one another) while every warp gets about 16 grabs
+    const int64_t per_warp = g->narcs / ((int64_t)blocks * (kDThreads / 32) * 16);
+    const int chunk = P.k == 3 ? 32 : (int)std::max<int64_t>(1, std::min<int64_t>(8, per_warp));
+    const DLists lists{g->out_ptr, g->out_col, g->in_ptr, g->in_col};
+    k_dcount<<<blocks, kDThreads, 0, st>>>(P, g->n, g->narcs, lists, chunk, cursor, res);
     count_launch();
     GP_CUDA_TRY(cudaGetLastError());
     unsigned long long h[2] = {0, 0};

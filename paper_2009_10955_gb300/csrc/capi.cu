@@ -579,13 +579,14 @@ gp_status gp_count(gp_graph* g, const gp_schedules* s, int32_t idx, const gp_cou
         return fail(GP_ERR_ARG, "an inclusion-exclusion count over part of the tasks needs opts->raw_total");
     rc = ensure_device(g);
     if (rc != GP_OK) return rc;
-    if (job.plan.labeled) {                  // labelled plans: the listing kernel's counting pass
+    if (job.plan.labeled) {                  // labelled plans: a kernel of their own
         if (opts && opts->budget_cycles > 0) return fail(GP_ERR_ARG, "labelled counts take no budget");
-        int64_t w = 0, cut = 0, total = 0;
-        rc = run_list(job, nullptr, -1, static_cast<cudaStream_t>(stream), &w, &cut, &total);
+        uint64_t res[2] = {0, 0}, total = 0;
+        rc = run_labeled(job, static_cast<cudaStream_t>(stream), res);
+        if (rc == GP_OK) rc = finish_total(job.plan, res[0], res[1], &total);
         if (rc != GP_OK) return rc;
         if (opts && opts->resume_cursor) *opts->resume_cursor = job.task_begin + job.ntasks;
-        *out = (uint64_t)total;
+        *out = total;
         return GP_OK;
     }
     uint64_t res[2] = {0, 0};

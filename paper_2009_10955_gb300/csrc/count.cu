@@ -252,10 +252,12 @@ __device__ __forceinline__ int warp_merge(const TaskCtx& c, const int32_t* __res
 // Warp-cooperative intersection of a and b within window w. Writes the
 // (sorted) result to out when out != nullptr and returns its size
 // (warp-uniform). With acc != nullptr each lane also adds its own matches.
+// kLab: only elements that carry `label` count.
+template <bool kLab = false>
 __device__ __forceinline__ int warp_intersect(const TaskCtx& c, List a, List b, Window w,
-                                              int32_t* __restrict__ out, int cap, Acc* acc) {
+                                              int32_t* __restrict__ out, int cap, Acc* acc, int label = 0) {
     const Probe q = choose(c, a, b, w);
-    if (!q.bitmap && q.it.n > 0 && q.pr.n <= kMergeRatio * q.it.n) {
+    if (!kLab && !q.bitmap && q.it.n > 0 && q.pr.n <= kMergeRatio * q.it.n) {
         const int total = warp_merge(c, q.it.p, q.it.n, q.pr.p, q.pr.n, out, cap, acc);
         if (c.sbytes && c.lane == 0) tally(c, a, b, w, out ? 4ull * (unsigned long long)total : 0ull);
         return total;
@@ -275,6 +277,7 @@ __device__ __forceinline__ int warp_intersect(const TaskCtx& c, List a, List b, 
                 f = pos < q.pr.n && __ldg(q.pr.p + pos) == x;
                 searched = true;
             }
+            if (kLab && f) f = __ldg(c.labels + x) == label;
         }
         const unsigned m = __ballot_sync(kFull, f);
         if (out && f) {
@@ -357,6 +360,7 @@ __device__ __forceinline__ bool member(const TaskCtx& c, List a, int x) {
     return p < a.n && __ldg(a.p + p) == x;
 }
 
+template <bool kLab = false>
 __device__ __forceinline__ void run_builds(const TaskCtx& c, int d, const int* v) {
     const GpLevel& L = c.P->lvl[d];
     for (int q = 0; q < L.nbuild; ++q) {
@@ -364,7 +368,8 @@ __device__ __forceinline__ void run_builds(const TaskCtx& c, int d, const int* v
         const List a = (B.base_kind == 1) ? nbr(c, v[B.base]) : slot(c, B.base);
         const Window w = window(B.lo_mask, B.hi_mask, v);
         int32_t* out = c.slots + (size_t)B.dst * c.slot_cap;
-        const int n = warp_intersect(c, a, nbr(c, v[d]), w, out, c.slot_cap, nullptr);
+        const int n = warp_intersect<kLab>(c, a, nbr(c, v[d]), w, out, c.slot_cap, nullptr,
+                                           kLab ? c.P->label[B.depth] : 0);
         if (c.lane == 0) c.slen[B.dst] = n;
         __syncwarp();
     }
@@ -1439,7 +1444,15 @@ k_count(const CountJob* __restrict__ jobs, int njobs, int64_t total,
 // element that is not an already-matched vertex is one embedding. Pass 1
 // (kWrite = false) stores each task's embedding count; pass 2 writes task
 // t's tuples from offset[t], in depth-first order, so the output is
-// deterministic.
+// deterministic. A warp takes up to 32 tasks per grab and its lanes look at
+// them side by side first (row search, restriction between the first two
+// vertices): one at a time, the grabs alone took longer than the
+// intersections (2 M tasks of R-MAT 16, one atomic each).
+//
+// Labelled counts run the same loops (k_label), with the last two levels one
+// candidate per lane where no set is built in between, over a list of the
+// tasks whose first two vertices carry their labels, each cut into parts that
+// share out its depth-2 candidates.
 
 __device__ __forceinline__ int list_last(const TaskCtx& c, const int* v, int32_t* out, int64_t at,
                                          bool write) {
@@ -1451,7 +1464,8 @@ __device__ __forceinline__ int list_last(const TaskCtx& c, const int* v, int32_t
     if (P.last_count_only) {
         const List a = (P.last_base_kind == 1) ? nbr(c, v[P.last_base]) : slot(c, P.last_base);
         int32_t* spare = c.slots + (size_t)P.nslots * c.slot_cap;
-        const int m = warp_intersect(c, a, nbr(c, v[L - 1]), w, spare, c.slot_cap, nullptr);
+        const int m = P.labeled ? warp_intersect<true>(c, a, nbr(c, v[L - 1]), w, spare, c.slot_cap, nullptr, P.label[L])
+                                : warp_intersect(c, a, nbr(c, v[L - 1]), w, spare, c.slot_cap, nullptr);
         __syncwarp();
         S = List{spare, m, -1};
     } else {
@@ -1479,35 +1493,27 @@ __device__ __forceinline__ int list_last(const TaskCtx& c, const int* v, int32_t
     return total;
 }
 
-template <bool kWrite>
-__global__ void __launch_bounds__(kWarps * 32, 4)
-k_list(const CountJob* __restrict__ job, int64_t ntasks, unsigned long long* __restrict__ cursor,
-       int64_t* __restrict__ per_task, int32_t* __restrict__ out, int32_t* __restrict__ slot_pool,
-       int64_t warp_elems, int* __restrict__ err) {
-    __shared__ GpPlan s_plan[kWarps];
-    __shared__ int s_len[kWarps][GP_MAX_SLOTS];
-    __shared__ long long s_deadline[kWarps];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t gw = (int64_t)blockIdx.x * kWarps + w;
-    {
-        const int* src = reinterpret_cast<const int*>(&job->plan);
-        int* dst = reinterpret_cast<int*>(&s_plan[w]);
-        for (int i = lane; i < (int)(sizeof(GpPlan) / 4); i += 32) dst[i] = src[i];
-        if (lane == 0) s_deadline[w] = 0;
-        __syncwarp();
-    }
+// A warp's context for the listing loops (set up from the job; the plan goes
+// to shared memory).
+__device__ __forceinline__ TaskCtx list_context(const CountJob* job, GpPlan* plan, int* slen, long long* deadline,
+                                                int32_t* slots, int* err, int lane) {
+    const int* src = reinterpret_cast<const int*>(&job->plan);
+    int* dst = reinterpret_cast<int*>(plan);
+    for (int i = lane; i < (int)(sizeof(GpPlan) / 4); i += 32) dst[i] = src[i];
+    if (lane == 0) *deadline = 0;
+    __syncwarp();
     TaskCtx c;
-    c.P = &s_plan[w];
+    c.P = plan;
     c.iep_cnt = nullptr;                        // listing plans never use inclusion-exclusion
     c.row_ptr = job->row_ptr;
     c.col = job->col;
     c.core_bits = job->core_bits;
     c.core_n = job->core_bits ? job->core_n : 0;
     c.core_words = job->core_words;
-    c.slots = slot_pool + gw * warp_elems;
+    c.slots = slots;
     c.slot_cap = job->slot_cap;
     c.n_vertices = job->n;
-    c.slen = s_len[w];
+    c.slen = slen;
     c.bm = nullptr;
     c.bm_stride = 0;
     c.lane_bitmap = false;
@@ -1517,35 +1523,83 @@ k_list(const CountJob* __restrict__ job, int64_t ntasks, unsigned long long* __r
     c.err = err;
     c.sbytes = nullptr;
     c.sops = nullptr;
-    c.deadline = &s_deadline[w];
+    c.deadline = deadline;
     c.task_cycles = 0;
     c.job_abort = err;
     c.labels = job->labels;
+    return c;
+}
+
+// Row of CSR entry e: the last vertex whose list starts at or before it.
+__device__ __forceinline__ int row_of(const TaskCtx& c, int64_t e) {
+    int lo = 0, hi = c.n_vertices - 1;
+    while (lo < hi) {
+        const int mid = lo + ((hi - lo + 1) >> 1);
+        if (__ldg(c.row_ptr + mid) <= e) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
+// May (v0, v1) be the first two vertices: restriction between them, labels.
+__device__ __forceinline__ bool first_two(const TaskCtx& c, int v0, int v1) {
+    const GpPlan& P = *c.P;
+    if ((P.lvl[1].lo_mask & 1) && !(v1 > v0)) return false;
+    if ((P.lvl[1].hi_mask & 1) && !(v1 < v0)) return false;
+    return !P.labeled || (__ldg(c.labels + v0) == P.label[0] && __ldg(c.labels + v1) == P.label[1]);
+}
+
+__device__ __forceinline__ bool taken(const GpLevel& L, const int* v, int d, int x) {
+    bool hit = false;
+    for (int j = 0; j < d; ++j) hit |= ((L.excl_mask >> j) & 1) && v[j] == x;
+    return hit;
+}
+
+template <bool kWrite>
+__global__ void __launch_bounds__(kWarps * 32, 4)
+k_list(const CountJob* __restrict__ job, int64_t ntasks, int chunk, unsigned long long* __restrict__ cursor,
+       int64_t* __restrict__ per_task, int32_t* __restrict__ out, int32_t* __restrict__ slot_pool,
+       int64_t warp_elems, int* __restrict__ err) {
+    __shared__ GpPlan s_plan[kWarps];
+    __shared__ int s_len[kWarps][GP_MAX_SLOTS];
+    __shared__ long long s_deadline[kWarps];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t gw = (int64_t)blockIdx.x * kWarps + w;
+    const TaskCtx c = list_context(job, &s_plan[w], s_len[w], &s_deadline[w], slot_pool + gw * warp_elems, err, lane);
     const GpPlan& P = s_plan[w];
     const int k = P.k;
     for (;;) {
         unsigned long long t0 = 0;
-        if (lane == 0) t0 = atomicAdd(cursor, 1ull);
+        if (lane == 0) t0 = atomicAdd(cursor, (unsigned long long)chunk);
         t0 = __shfl_sync(kFull, t0, 0);
         if ((int64_t)t0 >= ntasks) break;
-        const int64_t e = job->task_begin + (int64_t)t0;
-        int rl = 0, rh = c.n_vertices - 1;           // source vertex of entry e
-        while (rl < rh) {
-            int mid = (rl + rh + 1) >> 1;
-            if (__ldg(c.row_ptr + mid) <= e) rl = mid; else rh = mid - 1;
+        // a lane per task
+        const int64_t mine = (int64_t)t0 + lane;
+        const bool have = lane < chunk && mine < ntasks;
+        int my0 = 0, my1 = 0;
+        int64_t my_at = 0;
+        bool ok = false;
+        if (have) {
+            my0 = row_of(c, job->task_begin + mine);
+            my1 = __ldg(c.col + job->task_begin + mine);
+            ok = first_two(c, my0, my1);
+            if (kWrite) {
+                my_at = per_task[mine];
+                ok = ok && per_task[mine + 1] > my_at;       // tasks without an embedding
+            }
         }
-        int v[GP_MAX_K];
+        int64_t my_found = 0;
+        unsigned todo = __ballot_sync(kFull, ok);
+        while (todo) {
+            const int from = __ffs(todo) - 1;
+            todo &= todo - 1;
+            int v[GP_MAX_K];
 #pragma unroll
-        for (int i = 0; i < GP_MAX_K; ++i) v[i] = -1;
-        v[0] = rl;
-        v[1] = __ldg(c.col + e);
-        int64_t found = 0;
-        const int64_t at = kWrite ? per_task[t0] : 0;
-        bool ok1 = !((P.lvl[1].lo_mask & 1) && !(v[1] > v[0])) && !((P.lvl[1].hi_mask & 1) && !(v[1] < v[0]));
-        if (P.labeled)
-            ok1 = ok1 && __ldg(c.labels + v[0]) == P.label[0] && __ldg(c.labels + v[1]) == P.label[1];
-        if (ok1) {
-            run_builds(c, 1, v);
+            for (int i = 0; i < GP_MAX_K; ++i) v[i] = -1;
+            v[0] = __shfl_sync(kFull, my0, from);
+            v[1] = __shfl_sync(kFull, my1, from);
+            int64_t found = 0;
+            const int64_t at = __shfl_sync(kFull, my_at, from);
+            if (P.labeled) run_builds<true>(c, 1, v); else run_builds(c, 1, v);
             if (k == 3) {
                 found += list_last(c, v, out, at + found, kWrite);
             } else {
@@ -1559,13 +1613,11 @@ k_list(const CountJob* __restrict__ job, int64_t ntasks, unsigned long long* __r
                     if (cur[d] >= lst[d].n) { --d; continue; }
                     const int x = __ldg(lst[d].p + cur[d]);
                     ++cur[d];
-                    const uint8_t ex = P.lvl[d].excl_mask;
-                    bool skip = false;
-                    for (int j = 0; j < d; ++j) skip |= ((ex >> j) & 1) && v[j] == x;
+                    bool skip = taken(P.lvl[d], v, d, x);
                     if (P.labeled) skip |= __ldg(c.labels + x) != P.label[d];
                     if (skip) continue;
                     v[d] = x;
-                    run_builds(c, d, v);
+                    if (P.labeled) run_builds<true>(c, d, v); else run_builds(c, d, v);
                     if (d == k - 2) {
                         found += list_last(c, v, out, at + found, kWrite);
                     } else {
@@ -1577,9 +1629,193 @@ k_list(const CountJob* __restrict__ job, int64_t ntasks, unsigned long long* __r
                     }
                 }
             }
+            if (lane == from) my_found = found;
+            __syncwarp();
         }
-        if (!kWrite && lane == 0) per_task[t0] = found;
+        if (!kWrite && have) per_task[mine] = my_found;
     }
+}
+
+// Tasks whose first two vertices may stand there, as (v0, v1) pairs in any
+// order (labelled counts: a few tasks in a hundred).
+__global__ void k_label_tasks(const CountJob* __restrict__ job, unsigned long long* __restrict__ count,
+                              int2* __restrict__ tasks) {
+    TaskCtx c;
+    c.P = &job->plan;
+    c.row_ptr = job->row_ptr;
+    c.n_vertices = job->n;
+    c.labels = job->labels;
+    const int lane = threadIdx.x & 31;
+    for (int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; t0 < job->ntasks;
+         t0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t t = t0 + lane;
+        int v0 = 0, v1 = 0;
+        bool ok = false;
+        if (t < job->ntasks) {
+            v1 = __ldg(job->col + job->task_begin + t);
+            if (__ldg(job->labels + v1) == job->plan.label[1]) {
+                v0 = row_of(c, job->task_begin + t);
+                ok = first_two(c, v0, v1);
+            }
+        }
+        const unsigned m = __ballot_sync(kFull, ok);
+        unsigned long long at = 0;
+        if (lane == 0 && m) at = atomicAdd(count, (unsigned long long)__popc(m));
+        at = __shfl_sync(kFull, at, 0);
+        if (ok) tasks[at + __popc(m & lanemask_lt())] = make_int2(v0, v1);
+    }
+}
+
+// The last level's count for one lane's v[0..k-2], elements with the last
+// vertex's label only; false (nothing counted) above the work limit.
+__device__ __forceinline__ bool label_last_lane(const TaskCtx& c, const int* v, Acc& acc) {
+    const GpPlan& P = *c.P;
+    const int L = P.k - 1;
+    const GpLevel& lv = P.lvl[L];
+    const Window w = window(lv.lo_mask, lv.hi_mask, v);
+    const bool two = P.last_count_only;
+    Probe q;
+    if (two) {
+        const List a = (P.last_base_kind == 1) ? nbr(c, v[P.last_base]) : slot(c, P.last_base);
+        q = choose(c, a, nbr(c, v[L - 1]), w);
+    } else {
+        q.it = clip((lv.src_kind == 1) ? nbr(c, v[lv.src]) : slot(c, lv.src), w);
+    }
+    if (q.it.n > c.lane_work) return false;
+    int cnt = 0, from = two && q.bitmap ? q.tail : 0;
+    for (int i = 0; i < q.it.n; ++i) {
+        const int x = __ldg(q.it.p + i);
+        if (__ldg(c.labels + x) != P.label[L] || taken(lv, v, L, x)) continue;
+        bool in = true;
+        if (two) {
+            if (q.bitmap && x < c.core_n) {
+                in = core_bit(c, q.pr.v, x);
+            } else {
+                from += lower_bound(q.pr.p + from, q.pr.n - from, x);
+                in = from < q.pr.n && __ldg(q.pr.p + from) == x;
+            }
+        }
+        cnt += in;
+    }
+    acc.add((unsigned long long)cnt);
+    return true;
+}
+
+// The same by the whole warp.
+__device__ __forceinline__ void label_last_warp(const TaskCtx& c, const int* v, Acc& acc) {
+    const int n = list_last(c, v, nullptr, 0, false);
+    if (c.lane == 0) acc.add((unsigned long long)n);
+}
+
+__global__ void __launch_bounds__(kWarps * 32, 4)
+k_label(const CountJob* __restrict__ job, const unsigned long long* __restrict__ n_tasks,
+        const int2* __restrict__ tasks, unsigned long long* __restrict__ cursor,
+        unsigned long long* __restrict__ total, int32_t* __restrict__ slot_pool, int64_t warp_elems,
+        int* __restrict__ err) {
+    __shared__ GpPlan s_plan[kWarps];
+    __shared__ int s_len[kWarps][GP_MAX_SLOTS];
+    __shared__ long long s_deadline[kWarps];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t gw = (int64_t)blockIdx.x * kWarps + w;
+    const TaskCtx c = list_context(job, &s_plan[w], s_len[w], &s_deadline[w], slot_pool + gw * warp_elems, err, lane);
+    const GpPlan& P = s_plan[w];
+    const int k = P.k;
+    const long long n = (long long)*n_tasks;
+    const long long warps = (long long)gridDim.x * kWarps;
+    // parts per task: about 16 work items a warp, so that the hubs' tasks
+    // spread; three-vertex patterns have no depth-2 loop to share out and go
+    // one task per lane
+    const int parts = k == 3 ? 1 : (int)min(64ll, max(1ll, 16 * warps / max(1ll, n)));
+    const int grab = k == 3 ? 32 : 1;
+    const bool lanes_last = P.lvl[k - 2].nbuild == 0;
+    Acc acc;
+    for (;;) {
+        unsigned long long t0 = 0;
+        if (lane == 0) t0 = atomicAdd(cursor, (unsigned long long)grab);
+        t0 = __shfl_sync(kFull, t0, 0);
+        if ((long long)t0 >= n * parts) break;
+        int v[GP_MAX_K];
+#pragma unroll
+        for (int i = 0; i < GP_MAX_K; ++i) v[i] = -1;
+        if (k == 3) {
+            const bool have = (long long)t0 + lane < n;
+            const int2 t = have ? tasks[t0 + lane] : make_int2(0, 0);
+            bool defer = false;
+            if (P.lvl[1].nbuild == 0) {
+                v[0] = t.x;
+                v[1] = t.y;
+                defer = have && !label_last_lane(c, v, acc);
+            } else {
+                defer = have;
+            }
+            unsigned dm = __ballot_sync(kFull, defer);
+            while (dm) {
+                const int src = __ffs(dm) - 1;
+                dm &= dm - 1;
+                v[0] = __shfl_sync(kFull, t.x, src);
+                v[1] = __shfl_sync(kFull, t.y, src);
+                run_builds<true>(c, 1, v);
+                label_last_warp(c, v, acc);
+            }
+            continue;
+        }
+        const int part = (int)(t0 % parts);
+        const int2 t = tasks[t0 / parts];
+        v[0] = t.x;
+        v[1] = t.y;
+        run_builds<true>(c, 1, v);
+        List lst[GP_MAX_K];
+        int cur[GP_MAX_K];
+        auto open = [&](int dd) {
+            const GpLevel& L = P.lvl[dd];
+            lst[dd] = clip((L.src_kind == 1) ? nbr(c, v[L.src]) : slot(c, L.src), window(L.lo_mask, L.hi_mask, v));
+            cur[dd] = 0;
+        };
+        int d = 2;
+        open(2);
+        if (parts > 1) {
+            const int len = lst[2].n;
+            const int b = (int)((int64_t)len * part / parts), e = (int)((int64_t)len * (part + 1) / parts);
+            lst[2].p += b;
+            lst[2].n = e - b;
+        }
+        while (d >= 2) {
+            if (d == k - 2 && lanes_last) {
+                for (int base = 0; base < lst[d].n; base += 32) {
+                    const int i = base + lane;
+                    int x = -1;
+                    bool in = false;
+                    if (i < lst[d].n) {
+                        x = __ldg(lst[d].p + i);
+                        in = __ldg(c.labels + x) == P.label[d] && !taken(P.lvl[d], v, d, x);
+                    }
+                    bool defer = false;
+                    if (in) {
+                        v[d] = x;
+                        defer = !label_last_lane(c, v, acc);
+                    }
+                    unsigned dm = __ballot_sync(kFull, defer);
+                    while (dm) {
+                        const int src = __ffs(dm) - 1;
+                        dm &= dm - 1;
+                        v[d] = __shfl_sync(kFull, x, src);
+                        label_last_warp(c, v, acc);
+                    }
+                }
+                --d;
+                continue;
+            }
+            if (cur[d] >= lst[d].n) { --d; continue; }
+            const int x = __ldg(lst[d].p + cur[d]);
+            ++cur[d];
+            if (__ldg(c.labels + x) != P.label[d] || taken(P.lvl[d], v, d, x)) continue;
+            v[d] = x;
+            run_builds<true>(c, d, v);
+            if (d == k - 2) label_last_warp(c, v, acc);
+            else open(++d);
+        }
+    }
+    flush(acc, total);
 }
 
 // Largest c <= ntasks with offsets[c] <= capacity (offsets is an exclusive
@@ -1863,25 +2099,85 @@ gp_status run_count_in_scratch(const CountJob* jobs, int njobs, void* d_scratch,
     return GP_OK;
 }
 
-gp_status run_list(const CountJob& job, int32_t* d_out, int64_t capacity, cudaStream_t st,
-                   int64_t* n_written, int64_t* cut_tasks, int64_t* total) {
-    const bool count_only = capacity < 0;      // per-task counts and their sum only
-    const int64_t T = job.ntasks;
-    *n_written = 0;
-    *cut_tasks = 0;
-    if (total) *total = 0;
-    if (T == 0) return GP_OK;
+namespace {
+
+// Grid of a listing kernel: all resident blocks, reduced (in whole waves of
+// SMs) until the per-warp sets fit a quarter of the free device memory.
+gp_status list_grid(const void* fn, const CountJob& job, int64_t* blocks, int64_t* warp_elems, size_t* per_block) {
     int dev = 0, nsm = 0, occ = 0;
     GP_CUDA_TRY(cudaGetDevice(&dev));
     GP_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    GP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_list<false>, kWarps * 32, 0));
-    const int64_t warp_elems = (int64_t)(job.plan.nslots + 1) * job.slot_cap;
-    const size_t per_block = (size_t)kWarps * (size_t)warp_elems * sizeof(int32_t);
+    GP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kWarps * 32, 0));
+    *warp_elems = (int64_t)(job.plan.nslots + 1) * job.slot_cap;
+    *per_block = (size_t)kWarps * (size_t)*warp_elems * sizeof(int32_t);
     size_t free_b = 0, total_b = 0;
     GP_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
-    int64_t blocks = (int64_t)nsm * std::max(occ, 1);
-    while (blocks > nsm && per_block * (size_t)blocks > free_b / 4) blocks -= nsm;
-    if (per_block * (size_t)blocks > free_b / 2) { set_error("listing scratch does not fit"); return GP_ERR_SCRATCH; }
+    *blocks = (int64_t)nsm * std::max(occ, 1);
+    while (*blocks > nsm && *per_block * (size_t)*blocks > free_b / 4) *blocks -= nsm;
+    if (*per_block * (size_t)*blocks > free_b / 2) { set_error("listing scratch does not fit"); return GP_ERR_SCRATCH; }
+    return GP_OK;
+}
+
+}  // namespace
+
+gp_status run_labeled(const CountJob& job, cudaStream_t st, uint64_t* results) {
+    results[0] = results[1] = 0;
+    if (job.ntasks == 0) return GP_OK;
+    int64_t blocks = 0, warp_elems = 0;
+    size_t per_block = 0;
+    gp_status rc = list_grid((const void*)k_label, job, &blocks, &warp_elems, &per_block);
+    if (rc != GP_OK) return rc;
+    // words (total, cursor, task count, error), job, tasks; then the sets
+    struct Words { unsigned long long total[2], cursor, n_tasks; int err; };
+    const size_t head_b = 256, job_b = (sizeof(CountJob) + 255) & ~(size_t)255;
+    char* mem = nullptr;
+    int32_t* slots = nullptr;
+    GP_CUDA_TRY(cudaMallocAsync((void**)&mem, head_b + job_b + sizeof(int2) * (size_t)job.ntasks, st));
+    if (cudaMallocAsync((void**)&slots, per_block * (size_t)blocks, st) != cudaSuccess) {
+        cudaFreeAsync(mem, st);
+        cudaGetLastError();
+        set_error("cannot allocate listing scratch");
+        return GP_ERR_NOMEM;
+    }
+    Words* words = reinterpret_cast<Words*>(mem);
+    CountJob* d_job = reinterpret_cast<CountJob*>(mem + head_b);
+    int2* tasks = reinterpret_cast<int2*>(mem + head_b + job_b);
+    Words h = {};
+    cudaError_t e = cudaMemsetAsync(mem, 0, head_b, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d_job, &job, sizeof(CountJob), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) {
+        const int64_t want = (job.ntasks + 255) / 256;
+        k_label_tasks<<<(unsigned)std::min<int64_t>(want, blocks * 8), 256, 0, st>>>(d_job, &words->n_tasks, tasks);
+        k_label<<<(unsigned)blocks, kWarps * 32, 0, st>>>(d_job, &words->n_tasks, tasks, &words->cursor, words->total,
+                                                         slots, warp_elems, &words->err);
+        count_launch(2);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, words, sizeof(h), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    cudaFreeAsync(slots, st);
+    cudaFreeAsync(mem, st);
+    if (e != cudaSuccess) { set_error("labelled count failed: %s", cudaGetErrorString(e)); return GP_ERR_CUDA; }
+    if (h.err) { set_error("labelled count reported internal error %d", h.err); return GP_ERR_INTERNAL; }
+    results[0] = h.total[0];
+    results[1] = h.total[1];
+    return GP_OK;
+}
+
+gp_status run_list(const CountJob& job, int32_t* d_out, int64_t capacity, cudaStream_t st,
+                   int64_t* n_written, int64_t* cut_tasks) {
+    const int64_t T = job.ntasks;
+    *n_written = 0;
+    *cut_tasks = 0;
+    if (T == 0) return GP_OK;
+    int64_t blocks = 0, warp_elems = 0;
+    size_t per_block = 0;
+    gp_status rc = list_grid((const void*)k_list<false>, job, &blocks, &warp_elems, &per_block);
+    if (rc != GP_OK) return rc;
+    // tasks per grab: a warp's 32 lanes look at as many side by side, fewer
+    // where the tasks would not go around (about 8 grabs a warp; 64 where a
+    // task runs loops of its own: 4-cliques of R-MAT 12 lost 9 % in threes)
+    const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(32, T / (blocks * kWarps * (job.plan.k == 3 ? 8 : 64))));
     size_t scan_b = 0;
     GP_CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, scan_b, (int64_t*)nullptr, (int64_t*)nullptr, T + 1, st));
     void* mem = nullptr;
@@ -1903,30 +2199,29 @@ gp_status run_list(const CountJob& job, int32_t* d_out, int64_t capacity, cudaSt
     int64_t* counts = reinterpret_cast<int64_t*>(b + head_b + ((sizeof(CountJob) + 63) & ~(size_t)63));
     int64_t* offsets = counts + (T + 1);
     void* scan_tmp = offsets + (T + 1);
-    int64_t h[2] = {0, 0}, h_total = 0;
+    int64_t h[2] = {0, 0};
     int h_err = 0;
     cudaError_t e = cudaMemsetAsync(b, 0, head_b, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_job, &job, sizeof(CountJob), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(counts, 0, cnt_b, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(counts + T, 0, sizeof(int64_t), st);   // the scan reads one more
     if (e == cudaSuccess) {
-        k_list<false><<<(unsigned)blocks, kWarps * 32, 0, st>>>(d_job, T, cursor, counts, nullptr, slots,
+        k_list<false><<<(unsigned)blocks, kWarps * 32, 0, st>>>(d_job, T, chunk, cursor, counts, nullptr, slots,
                                                                warp_elems, err);
         count_launch();
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cub::DeviceScan::ExclusiveSum(scan_tmp, scan_b, counts, offsets, T + 1, st);
     if (e == cudaSuccess) {
-        k_list_cut<<<1, 1, 0, st>>>(offsets, T, count_only ? 0 : capacity, cut);
+        k_list_cut<<<1, 1, 0, st>>>(offsets, T, capacity, cut);
         count_launch(2);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, cut, sizeof(h), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h_total, offsets + T, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e == cudaSuccess && h[0] > 0 && !count_only) {
+    if (e == cudaSuccess && h[0] > 0) {
         e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), st);
         if (e == cudaSuccess) {
-            k_list<true><<<(unsigned)blocks, kWarps * 32, 0, st>>>(d_job, h[0], cursor, offsets, d_out, slots,
+            k_list<true><<<(unsigned)blocks, kWarps * 32, 0, st>>>(d_job, h[0], chunk, cursor, offsets, d_out, slots,
                                                                   warp_elems, err);
             count_launch();
             e = cudaGetLastError();
@@ -1940,7 +2235,6 @@ gp_status run_list(const CountJob& job, int32_t* d_out, int64_t capacity, cudaSt
     if (h_err) { set_error("listing kernel reported internal error %d", h_err); return GP_ERR_INTERNAL; }
     *cut_tasks = h[0];
     *n_written = h[1];
-    if (total) *total = h_total;
     return GP_OK;
 }
 

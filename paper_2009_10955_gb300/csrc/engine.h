@@ -150,10 +150,12 @@ gp_status job_total(const CountJob& job, const uint64_t* res, uint64_t* out);
 
 // Listing: the embeddings of the longest prefix of the job's tasks whose
 // total fits `capacity` tuples, written to d_out (k int32 per embedding).
-// *cut_tasks receives that prefix's length, *n_written its embeddings,
-// *total the embeddings of all the job's tasks. capacity < 0: count only.
+// *cut_tasks receives that prefix's length, *n_written its embeddings.
 gp_status run_list(const CountJob& job, int32_t* d_out, int64_t capacity, cudaStream_t st,
-                   int64_t* n_written, int64_t* cut_tasks, int64_t* total = nullptr);
+                   int64_t* n_written, int64_t* cut_tasks);
+
+// The 128-bit count of a labelled plan's job (count.cu).
+gp_status run_labeled(const CountJob& job, cudaStream_t st, uint64_t* results);
 
 // Key of the kernel build geometry() would pick for this job alone (its
 // register budget and whether it carries general inclusion-exclusion); jobs

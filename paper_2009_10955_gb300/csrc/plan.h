@@ -24,7 +24,8 @@ struct GpBuild {
     int8_t base;
     uint8_t lo_mask;   // depths j <= d with candidate > v_j
     uint8_t hi_mask;   // depths j <= d with candidate < v_j
-    int8_t pad[3];
+    int8_t depth;      // labelled plans: the set is for this depth, elements carry its label
+    int8_t pad[2];
 };
 
 struct GpLevel {

@@ -350,12 +350,14 @@ bool compile_plan(const PatternInfo& p, const int8_t* sched, ResMask res, GpPlan
     for (int x = 0; x < k; ++x)
         if (gt[x][x]) { err = "restriction set is cyclic"; return false; }
 
-    struct SlotKey { uint8_t prefix, lo, hi; int8_t id; };
+    // a labelled plan's sets hold one label's vertices only, so that a set is
+    // shared by depths of the same label
+    struct SlotKey { uint8_t prefix, lo, hi; int8_t id; int32_t label; };
     std::vector<SlotKey> keys;
     int nslots = 0;
-    auto find_slot = [&](uint8_t prefix, uint8_t lo, uint8_t hi) -> int {
+    auto find_slot = [&](uint8_t prefix, uint8_t lo, uint8_t hi, int32_t label) -> int {
         for (const SlotKey& s : keys)
-            if (s.prefix == prefix && s.lo == lo && s.hi == hi) return s.id;
+            if (s.prefix == prefix && s.lo == lo && s.hi == hi && s.label == label) return s.id;
         return -1;
     };
 
@@ -374,6 +376,9 @@ bool compile_plan(const PatternInfo& p, const int8_t* sched, ResMask res, GpPlan
         L.hi_mask = hi;
         L.op_mask = opmask;
         L.excl_mask = (uint8_t)(((1u << x) - 1) & ~opmask & ~lo & ~hi);
+        if (p.labeled)                       // a vertex of another label is no candidate
+            for (int j = 0; j < x; ++j)
+                if (p.labels[sched[j]] != p.labels[sched[x]]) L.excl_mask &= (uint8_t)~(1u << j);
         if (nops == 1) { L.src_kind = 1; L.src = (int8_t)ops[0]; continue; }
         int prev_slot = -1;
         for (int q = 1; q < nops; ++q) {
@@ -391,11 +396,12 @@ bool compile_plan(const PatternInfo& p, const int8_t* sched, ResMask res, GpPlan
                 L.src = -1;
                 break;
             }
-            int id = find_slot(prefix, clo, chi);
+            const int32_t label = p.labeled ? p.labels[sched[x]] : -1;
+            int id = find_slot(prefix, clo, chi, label);
             if (id < 0) {
                 if (nslots >= GP_MAX_SLOTS) { err = "plan needs too many intermediate sets"; return false; }
                 id = nslots++;
-                keys.push_back({prefix, clo, chi, (int8_t)id});
+                keys.push_back({prefix, clo, chi, (int8_t)id, label});
                 GpLevel& B = plan.lvl[d];
                 if (B.nbuild >= GP_MAX_BUILDS) { err = "too many intersections in one loop"; return false; }
                 GpBuild& b = B.build[B.nbuild++];
@@ -404,6 +410,7 @@ bool compile_plan(const PatternInfo& p, const int8_t* sched, ResMask res, GpPlan
                 else { b.base_kind = 2; b.base = (int8_t)prev_slot; }
                 b.lo_mask = clo;
                 b.hi_mask = chi;
+                b.depth = (int8_t)x;
             }
             prev_slot = id;
             if (q == nops - 1) { L.src_kind = 2; L.src = (int8_t)id; }

@@ -9,6 +9,7 @@
 #include <new>
 #include <vector>
 
+#include "bits.cuh"
 #include "engine.h"
 #include "planner.h"
 
@@ -68,6 +69,58 @@ gp_status ensure_device(const gp_graph* g) {
     return GP_OK;
 }
 
+// Jobs that a kernel of their own counts (clique.cu, join.cu, wedge.cu).
+bool local_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& lo) {
+    return clique_applies(job, g, lo) || join_applies(job, g, lo) || wedge_applies(job, g, lo);
+}
+
+// Count such jobs: one launch each, their results read back together. res has
+// two words a job; busy as for run_count.
+gp_status run_local(const CountJob* const* jobs, gp_graph* const* graphs, int n, cudaStream_t st,
+                    uint64_t* const* res, float* ms, uint64_t* busy) {
+    LaunchScratch mem(st);
+    const size_t bytes = sizeof(ResultWords) * (size_t)n;
+    GP_CUDA_TRY(mem.alloc(bytes));
+    ResultWords* words = reinterpret_cast<ResultWords*>(mem.p);
+    std::vector<ResultWords> h((size_t)n);
+    cudaEvent_t ev[2] = {nullptr, nullptr};
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; ms && i < 2 && e == cudaSuccess; ++i) e = cudaEventCreate(&ev[i]);
+    if (e == cudaSuccess) e = cudaMemsetAsync(words, 0, bytes, st);
+    if (e == cudaSuccess && ms) e = cudaEventRecord(ev[0], st);
+    gp_status rc = GP_OK;
+    busy[0] = busy[1] = 0;
+    for (int j = 0; j < n && e == cudaSuccess && rc == GP_OK; ++j) {
+        int64_t warps = 0;
+        const GpPlan& P = jobs[j]->plan;
+        if (!P.iep) rc = launch_clique(*jobs[j], graphs[j], st, words + j, &warps);
+        else if (wedge_applies(*jobs[j], graphs[j], LaunchOpts())) rc = launch_wedge(*jobs[j], graphs[j], st, words + j, &warps);
+        else rc = launch_join(*jobs[j], graphs[j], st, words + j, &warps);
+        busy[1] = std::max<uint64_t>(busy[1], (uint64_t)warps);
+    }
+    if (e == cudaSuccess && ms) e = cudaEventRecord(ev[1], st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), words, bytes, cudaMemcpyDeviceToHost, st);
+    const cudaError_t es = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) e = es;
+    if (e == cudaSuccess && ms && rc == GP_OK) e = cudaEventElapsedTime(ms, ev[0], ev[1]);
+    for (cudaEvent_t x : ev) if (x) cudaEventDestroy(x);
+    if (rc != GP_OK) return rc;
+    if (e != cudaSuccess) { set_error("count kernel failed: %s", cudaGetErrorString(e)); return GP_ERR_CUDA; }
+    for (int j = 0; j < n; ++j) {
+        res[j][0] = h[j].total[0];
+        res[j][1] = h[j].total[1];
+        busy[0] += h[j].busy;
+    }
+    return GP_OK;
+}
+
+gp_status run_local(const CountJob& job, gp_graph* g, cudaStream_t st, uint64_t* res, float* ms, uint64_t* busy) {
+    const CountJob* jobs[1] = {&job};
+    gp_graph* graphs[1] = {g};
+    uint64_t* out[1] = {res};
+    return run_local(jobs, graphs, 1, st, out, ms, busy);
+}
+
 // Triangle plan: schedule (0, 1, 2) with id(0) > id(1) > id(2).
 gp_status triangle_count(gp_graph* g, cudaStream_t st, uint64_t* out) {
     static const uint8_t tri[9] = {0, 1, 1, 1, 0, 1, 1, 1, 0};
@@ -94,8 +147,9 @@ gp_status triangle_count(gp_graph* g, cudaStream_t st, uint64_t* out) {
     job.core_words = g->core_words;
     uint64_t res2[2] = {0, 0};
     int64_t done = 0;
-    gp_status rc = clique_applies(job, g, LaunchOpts()) ? run_clique(job, g, st, res2)
-                                                        : run_count(&job, 1, LaunchOpts(), st, res2, &done);
+    uint64_t busy[2] = {0, 0};
+    gp_status rc = local_applies(job, g, LaunchOpts()) ? run_local(job, g, st, res2, nullptr, busy)
+                                                       : run_count(&job, 1, LaunchOpts(), st, res2, &done);
     if (rc != GP_OK) return rc;
     if (res2[1]) return fail(GP_ERR_OVERFLOW, "triangle count overflows 64 bits");
     *out = res2[0];
@@ -185,17 +239,6 @@ LaunchOpts launch_opts(const gp_count_opts* o) {
         if (o->lane_work > 0) lo.lane_work = o->lane_work;
     }
     return lo;
-}
-
-// Jobs that a kernel of their own counts (clique.cu, join.cu, wedge.cu).
-bool local_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& lo) {
-    return clique_applies(job, g, lo) || join_applies(job, g, lo) || wedge_applies(job, g, lo);
-}
-
-gp_status run_local(const CountJob& job, const gp_graph* g, cudaStream_t st, uint64_t* res, float* ms, uint64_t* busy) {
-    if (!job.plan.iep) return run_clique(job, g, st, res, ms, busy);
-    return wedge_applies(job, g, LaunchOpts()) ? run_wedge(job, g, st, res, ms, busy)
-                                               : run_join(job, g, st, res, ms, busy);
 }
 
 bool opts_ok(const gp_count_opts* o) {
@@ -669,16 +712,21 @@ gp_status gp_count_batch(gp_graph* const* graphs, const gp_schedules* const* sch
     GP_CUDA_TRY(cudaGetDevice(&dev));
     GP_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     const int user_chunk = lo.chunk;
-    for (int32_t j = 0; j < njobs; ++j) {     // a kernel of their own: a launch each
-        if (key[j] != -1) continue;
-        float jms = 0.f;
-        uint64_t jbusy[2] = {0, 0};
-        rc = run_local(jobs[j], graphs[j], static_cast<cudaStream_t>(stream), &res[2 * j], want_ms ? &jms : nullptr,
-                        jbusy);
-        if (rc != GP_OK) return rc;
-        ms += jms;
-        busy[0] += jbusy[0];
-        busy[1] = std::max(busy[1], jbusy[1]);
+    {                                         // kernels of their own: a launch each, one wait for all
+        std::vector<const CountJob*> own;
+        std::vector<gp_graph*> own_graphs;
+        std::vector<uint64_t*> own_res;
+        for (int32_t j = 0; j < njobs; ++j)
+            if (key[j] == -1) {
+                own.push_back(&jobs[j]);
+                own_graphs.push_back(graphs[j]);
+                own_res.push_back(&res[2 * (size_t)j]);
+            }
+        if (!own.empty()) {
+            rc = run_local(own.data(), own_graphs.data(), (int)own.size(), static_cast<cudaStream_t>(stream),
+                           own_res.data(), want_ms ? &ms : nullptr, busy);
+            if (rc != GP_OK) return rc;
+        }
     }
     for (int kv : keys) {
         if (kv == -1) continue;

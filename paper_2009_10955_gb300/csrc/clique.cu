@@ -601,8 +601,7 @@ bool clique_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& op
     return descending || (job.task_begin == 0 && job.ntasks == g->nnz);
 }
 
-gp_status run_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, uint64_t* results, float* kernel_ms,
-                     uint64_t* busy) {
+gp_status launch_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps) {
     const int k = job.plan.k;
     int dev = 0, nsm = 0;
     GP_CUDA_TRY(cudaGetDevice(&dev));
@@ -643,15 +642,16 @@ gp_status run_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, ui
     const size_t big_b = big ? sizeof(uint32_t) * (size_t)blocks * (2 * (size_t)a.big_words + 2 * kMostRows) : 0;
     const size_t sets_b = k >= 6 && a.n_block > 0
         ? sizeof(uint32_t) * (size_t)blocks * (size_t)(threads / 32) * 4 * (kMostRows / 32) : 0;
-    const gp_status rc = run_with_words(st, big_b + sets_b, kernel_ms, results, busy, "clique",
-                                        [&](ResultWords* words, char* mem) {
-        a.words = words;
-        a.big = reinterpret_cast<uint32_t*>(mem);
-        a.sets = reinterpret_cast<uint32_t*>(mem + big_b);
-        fn<<<(unsigned)blocks, threads, smem, st>>>(a);
-    });
-    if (busy) busy[1] = (uint64_t)blocks * (threads / 32);
-    return rc;
+    LaunchScratch mem(st);
+    GP_CUDA_TRY(mem.alloc(big_b + sets_b));
+    a.words = words;
+    a.big = reinterpret_cast<uint32_t*>(mem.p);
+    a.sets = reinterpret_cast<uint32_t*>(mem.p + big_b);
+    fn<<<(unsigned)blocks, threads, smem, st>>>(a);
+    count_launch();
+    GP_CUDA_TRY(cudaGetLastError());
+    *warps = blocks * (threads / 32);
+    return GP_OK;
 }
 
 }  // namespace gp

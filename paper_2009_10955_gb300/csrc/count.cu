@@ -38,6 +38,7 @@
 #include <cub/device/device_scan.cuh>
 
 #include "acc.cuh"
+#include "bits.cuh"
 #include "engine.h"
 
 namespace gp {
@@ -739,6 +740,254 @@ __device__ __forceinline__ void lane_parallel_last_two(const TaskCtx& c, int* v,
 }
 
 // ---------------------------------------------------------------------------
+// Lane forms: the loop at the last outer depth with one candidate per lane,
+// for plans where nothing is built per candidate. They live in a kernel build
+// of their own, without the bitmap subtree and the larger inclusion-exclusion:
+// added to the general builds they cost every other plan 3-6 % (spills, and
+// code beyond the instruction cache).
+
+// Lists up to this length are walked by a lane element by element against a
+// core vertex's bits without cutting them to the window first: comparing with
+// the window costs less than the four searches that cut both lists (6-cycles
+// of G(2000, 20000): 765 warp instructions per round of candidates before).
+// Used by the lane forms below.
+constexpr int kLaneWalk = 64;
+
+// Elements of s inside w that are neighbours of core vertex v (four probes in
+// flight); all of s lies in the core.
+__device__ __forceinline__ int lane_walk_core(const TaskCtx& c, List s, int v, Window w) {
+    const uint32_t* row = c.core_bits + (size_t)v * c.core_words;
+    int cnt = 0;
+    for (int i = 0; i < s.n; i += 4) {
+        int x[4];
+        uint32_t word[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) x[t] = __ldg(s.p + min(i + t, s.n - 1));
+        if (x[0] >= w.hi) break;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) word[t] = __ldg(row + (x[t] >> 5));
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+            cnt += (i + t < s.n && x[t] > w.lo && x[t] < w.hi) ? (word[t] >> (x[t] & 31)) & 1u : 0u;
+    }
+    return cnt;
+}
+
+// lane_intersect_count with the walk where it applies.
+__device__ __forceinline__ int lane_count(const TaskCtx& c, List a, List b, Window w) {
+    if (c.core_n > 0) {
+        List s = a.n <= b.n ? a : b, l = a.n <= b.n ? b : a;
+        if (!is_core(c, l.v)) { const List t = s; s = l; l = t; }
+        if (is_core(c, l.v) && s.n <= kLaneWalk) {
+            if (s.n == 0) return 0;
+            if (__ldg(s.p + s.n - 1) < c.core_n) return lane_walk_core(c, s, l.v, w);
+        }
+    }
+    return lane_intersect_count(c, a, b, w);
+}
+
+// Which of the matched vertices 0 .. d-1 lie in list a (bit j), one lane
+// each; the same value on every lane. Lanes whose lists a agree ask once
+// instead of each for every vertex.
+__device__ __forceinline__ unsigned matched_in(const TaskCtx& c, uint8_t mask, int d, const int* v, List a) {
+    bool in = false;
+    if (c.lane < d && (mask >> c.lane & 1)) in = member(c, a, v[c.lane]);
+    return __ballot_sync(kFull, in);
+}
+
+// Matched vertices of `in_a` (bits of depths, known to lie in the one list)
+// that are inside w and in b.
+__device__ __forceinline__ int hits_of(const TaskCtx& c, unsigned in_a, const int* v, Window w, List b) {
+    int hits = 0;
+#pragma unroll 1
+    for (; in_a; in_a &= in_a - 1) {           // rolled: the kernel is short of instruction cache
+        const int x = v[__ffs(in_a) - 1];
+        if (x > w.lo && x < w.hi && member(c, b, x)) ++hits;
+    }
+    return hits;
+}
+
+// lane_parallel_last_two for plans that only count the last intersection. Its
+// base list is bound before depth d = k-2, so the matched vertices in it are
+// found once; a candidate is never in its own list.
+__device__ __forceinline__ void lane_form_last_two(const TaskCtx& c, int* v, List lst, Acc& acc) {
+    const GpPlan& P = *c.P;
+    const int d = P.k - 2, L = P.k - 1;
+    const uint8_t ex = P.lvl[d].excl_mask;
+    const GpLevel& lv = P.lvl[L];
+    const unsigned in_a = matched_in(c, lv.excl_mask, d, v,
+                                     (P.last_base_kind == 1) ? nbr(c, v[P.last_base]) : slot(c, P.last_base));
+    for (int base = 0; base < lst.n; base += 32) {
+        if (over(c)) return;
+        const int i = base + c.lane;
+        int x = -1;
+        bool active = i < lst.n;
+        if (active) {
+            x = __ldg(lst.p + i);
+            for (int j = 0; j < d; ++j) active &= !(((ex >> j) & 1) && v[j] == x);
+        }
+        int cnt = 0;
+        if (active) {
+            v[d] = x;
+            cnt = lane_count(c, (P.last_base_kind == 1) ? nbr(c, v[P.last_base]) : slot(c, P.last_base), nbr(c, x),
+                             window(lv.lo_mask, lv.hi_mask, v));
+        }
+        // the vote brings the lanes together again before the next divergent
+        // part (without it each lane ran the matched vertices alone: 2.2x)
+        unsigned dm = __ballot_sync(kFull, active && cnt < 0);
+        if (active && cnt >= 0)
+            acc.add((unsigned long long)(cnt - hits_of(c, in_a, v, window(lv.lo_mask, lv.hi_mask, v), nbr(c, x))));
+        while (dm) {
+            const int src = __ffs(dm) - 1;
+            dm &= dm - 1;
+            v[d] = __shfl_sync(kFull, x, src);
+            count_last(c, v, acc);
+        }
+    }
+}
+
+// Elements of the short list s (at most kLaneWalk) inside w that lie in l
+// (x); those of them that also lie in O (y).
+__device__ __forceinline__ int2 lane_fused(const TaskCtx& c, List s, List l, List O, Window w) {
+    int2 n = make_int2(0, 0);
+    for (int i = 0; i < s.n; ++i) {
+        const int x = __ldg(s.p + i);
+        if (x >= w.hi) break;
+        if (x <= w.lo || !member(c, l, x)) continue;
+        ++n.x;
+        n.y += member(c, O, x);
+    }
+    return n;
+}
+
+// Two-loop inclusion-exclusion for one lane's v[0..k-3] (iep_count2 runs the
+// same with the whole warp on one candidate, most of it idle on lists of a few
+// dozen), in two steps with a vote of the warp between them. First the sizes:
+// x, y of the two inner sets, z of their intersection, matched vertices still
+// in them; x < 0 when a list is too long for a lane.
+__device__ __forceinline__ int3 iep2_lane_sizes(const TaskCtx& c, const int* v) {
+    const GpPlan& P = *c.P;
+    const int da = P.k - 2, db = P.k - 1, d = P.k - 3;
+    if (P.iep_fuse) {
+        const int dF = P.k - 3 + P.iep_fuse, dO = (dF == da) ? db : da;
+        const GpLevel& LF = P.lvl[dF];
+        const GpLevel& LO = P.lvl[dO];
+        const GpBuild& Bf = P.iep_build;
+        const List base = (Bf.base_kind == 1) ? nbr(c, v[Bf.base]) : slot(c, Bf.base);
+        const List nd = nbr(c, v[d]);
+        const List s = base.n <= nd.n ? base : nd, l = base.n <= nd.n ? nd : base;
+        if (s.n > kLaneWalk) return make_int3(-1, 0, 0);
+        const List O = clip((LO.src_kind == 1) ? nbr(c, v[LO.src]) : slot(c, LO.src),
+                            window(LO.lo_mask, LO.hi_mask, v));
+        const int2 n = lane_fused(c, s, l, O, window(Bf.lo_mask | LF.lo_mask, Bf.hi_mask | LF.hi_mask, v));
+        return make_int3(n.x, O.n, n.y);
+    }
+    const GpLevel& LA = P.lvl[da];
+    const GpLevel& LB = P.lvl[db];
+    const List A = clip((LA.src_kind == 1) ? nbr(c, v[LA.src]) : slot(c, LA.src), window(LA.lo_mask, LA.hi_mask, v));
+    const List B = clip((LB.src_kind == 1) ? nbr(c, v[LB.src]) : slot(c, LB.src), window(LB.lo_mask, LB.hi_mask, v));
+    if (A.p == B.p && A.n == B.n) return make_int3(A.n, A.n, A.n);
+    const int ab = min(A.n, B.n) > kLaneWalk ? -1 : lane_count(c, A, B, Window{-1, INT_MAX});
+    return make_int3(ab < 0 ? -1 : A.n, B.n, ab);
+}
+
+// Then the matched vertices in the sets, and the lane's count. in_a, in_b: the
+// matched vertices in the lists that do not depend on the lane's candidate.
+__device__ __forceinline__ void iep2_lane_add(const TaskCtx& c, const int* v, unsigned in_a, unsigned in_b, int3 n,
+                                              Acc& acc) {
+    const GpPlan& P = *c.P;
+    const int da = P.k - 2, db = P.k - 1, d = P.k - 3;
+    int ma = 0, mb = 0, mab = 0;
+    if (P.iep_fuse) {
+        const int dF = P.k - 3 + P.iep_fuse, dO = (dF == da) ? db : da;
+        const GpLevel& LF = P.lvl[dF];
+        const GpLevel& LO = P.lvl[dO];
+        const GpBuild& Bf = P.iep_build;
+        const List base = (Bf.base_kind == 1) ? nbr(c, v[Bf.base]) : slot(c, Bf.base);
+        const List nd = nbr(c, v[d]), O = (LO.src_kind == 1) ? nbr(c, v[LO.src]) : slot(c, LO.src);
+        const Window wf = window(Bf.lo_mask | LF.lo_mask, Bf.hi_mask | LF.hi_mask, v);
+        const Window wo = window(LO.lo_mask, LO.hi_mask, v);
+#pragma unroll 1
+        for (int j = 0; j <= d; ++j) {
+            const int x = v[j];
+            const bool f = (LF.excl_mask >> j & 1) && x > wf.lo && x < wf.hi && member(c, base, x) && member(c, nd, x);
+            const bool o = (LO.excl_mask >> j & 1) && x > wo.lo && x < wo.hi && member(c, O, x);
+            ma += f;
+            mb += o;
+            mab += f && o;
+        }
+    } else {
+        const GpLevel& LA = P.lvl[da];
+        const GpLevel& LB = P.lvl[db];
+        const Window wa = window(LA.lo_mask, LA.hi_mask, v), wb = window(LB.lo_mask, LB.hi_mask, v);
+        const List A = (LA.src_kind == 1) ? nbr(c, v[LA.src]) : slot(c, LA.src);
+        const List B = (LB.src_kind == 1) ? nbr(c, v[LB.src]) : slot(c, LB.src);
+        const bool own_a = LA.src_kind == 1 && LA.src == d, own_b = LB.src_kind == 1 && LB.src == d;
+#pragma unroll 1
+        for (int j = 0; j <= d; ++j) {
+            const int x = v[j];
+            const bool a = (LA.excl_mask >> j & 1) && x > wa.lo && x < wa.hi &&
+                           (own_a || j == d ? member(c, A, x) : (in_a >> j & 1));
+            const bool b = (LB.excl_mask >> j & 1) && x > wb.lo && x < wb.hi &&
+                           (own_b || j == d ? member(c, B, x) : (in_b >> j & 1));
+            ma += a;
+            mb += b;
+            mab += a && b;
+        }
+    }
+    acc.add((unsigned long long)(n.x - ma) * (unsigned long long)(n.y - mb));
+    acc.sub((unsigned long long)(n.z - mab));
+}
+
+// The loop at the last outer depth of a two-loop inclusion-exclusion plan
+// with one candidate per lane; candidates with long lists go to the warp one
+// at a time.
+__device__ __forceinline__ void lane_form_iep2(const TaskCtx& c, int* v, List lst, Acc& acc) {
+    const GpPlan& P = *c.P;
+    const int d = P.k - 3;
+    const uint8_t ex = P.lvl[d].excl_mask;
+    unsigned in_a = 0, in_b = 0;
+    if (!P.iep_fuse) {
+        const GpLevel& LA = P.lvl[d + 1];
+        const GpLevel& LB = P.lvl[d + 2];
+        if (!(LA.src_kind == 1 && LA.src == d))
+            in_a = matched_in(c, LA.excl_mask, d, v, LA.src_kind == 1 ? nbr(c, v[LA.src]) : slot(c, LA.src));
+        if (!(LB.src_kind == 1 && LB.src == d))
+            in_b = matched_in(c, LB.excl_mask, d, v, LB.src_kind == 1 ? nbr(c, v[LB.src]) : slot(c, LB.src));
+    }
+    for (int base = 0; base < lst.n; base += 32) {
+        if (over(c)) return;
+        const int i = base + c.lane;
+        int x = -1;
+        bool active = i < lst.n;
+        if (active) {
+            x = __ldg(lst.p + i);
+            for (int j = 0; j < d; ++j) active &= !(((ex >> j) & 1) && v[j] == x);
+        }
+        int3 n = make_int3(0, 0, 0);
+        if (active) {
+            v[d] = x;
+            n = iep2_lane_sizes(c, v);
+        }
+        unsigned dm = __ballot_sync(kFull, active && n.x < 0);
+        if (active && n.x >= 0) iep2_lane_add(c, v, in_a, in_b, n, acc);
+        while (dm) {
+            const int src = __ffs(dm) - 1;
+            dm &= dm - 1;
+            v[d] = __shfl_sync(kFull, x, src);
+            iep_count2<true>(c, v, acc);
+        }
+    }
+}
+
+// Is the plan's last outer loop one of the above?
+__host__ __device__ inline bool lane_form(const GpPlan& P) {
+    if (P.labeled || P.core_dfs || P.k < 4) return false;
+    if (P.iep) return P.iep == 2 && P.k >= 5 && P.lvl[P.k - 3].nbuild == 0;
+    return P.last_count_only && P.lvl[P.k - 2].nbuild == 0;
+}
+
+// ---------------------------------------------------------------------------
 // Bitmap subtree: used when every vertex searched after v1 is restricted
 // below v1 and v1 is a core vertex. All later candidates are then core
 // vertices below v1, so a candidate set is the AND of core adjacency rows
@@ -1175,7 +1424,7 @@ __device__ void bitmap_task(const TaskCtx& c, int* v, Acc& acc, int part, int np
 
 // Remaining loops of one edge task (v0, v1), or of part `part` of `nparts`
 // of it: the parts share out the candidates of depth 2.
-template <bool kGeneralIep>
+template <bool kGeneralIep, bool kLanes>
 __device__ void run_task(const TaskCtx& c, int v0, int v1, Acc& acc, int part, int nparts) {
     const GpPlan& P = *c.P;
     const int k = P.k;
@@ -1192,13 +1441,14 @@ __device__ void run_task(const TaskCtx& c, int v0, int v1, Acc& acc, int part, i
     for (int i = 0; i < GP_MAX_K; ++i) v[i] = -1;
     v[0] = v0;
     v[1] = v1;
-    if (P.core_dfs && c.bm && v1 < c.core_n) { bitmap_task(c, v, acc, part, nparts); return; }
+    if constexpr (!kLanes)
+        if (P.core_dfs && c.bm && v1 < c.core_n) { bitmap_task(c, v, acc, part, nparts); return; }
     const int d_iep = P.iep ? k - 1 - P.iep : -1;   // last outer depth of an inclusion-exclusion plan
     if (k == 3 || d_iep == 1) {
         if (part != 0) return;                 // no depth-2 loop to share out
         run_builds(c, 1, v);
         if (k == 3) count_last(c, v, acc);
-        else iep_count<kGeneralIep>(c, v, acc);
+        else if constexpr (!kLanes) iep_count<kGeneralIep>(c, v, acc);   // (no lane form)
         return;
     }
     run_builds(c, 1, v);
@@ -1207,7 +1457,7 @@ __device__ void run_task(const TaskCtx& c, int v0, int v1, Acc& acc, int part, i
         lst[dd] = clip((L.src_kind == 1) ? nbr(c, v[L.src]) : slot(c, L.src), window(L.lo_mask, L.hi_mask, v));
         cur[dd] = 0;
     };
-    const bool lane_last = !P.iep && P.lvl[k - 2].nbuild == 0;
+    const bool lane_last = !kLanes && !P.iep && P.lvl[k - 2].nbuild == 0;
     int d = 2;
     prepare(2);
     if (nparts > 1) {                          // this part's share of depth 2
@@ -1217,6 +1467,14 @@ __device__ void run_task(const TaskCtx& c, int v0, int v1, Acc& acc, int part, i
         lst[2].n = e - b;
     }
     while (d >= 2) {
+        if constexpr (kLanes) {                // every plan of this build has a lane form
+            if (d == (P.iep ? d_iep : k - 2)) {
+                if (P.iep) lane_form_iep2(c, v, lst[d], acc);
+                else lane_form_last_two(c, v, lst[d], acc);
+                --d;
+                continue;
+            }
+        }
         if (lane_last && d == k - 2) {
             lane_parallel_last_two(c, v, lst[d], acc);
             --d;
@@ -1233,13 +1491,16 @@ __device__ void run_task(const TaskCtx& c, int v0, int v1, Acc& acc, int part, i
         if (skip) continue;
         v[d] = x;
         run_builds(c, d, v);
-        if (d == d_iep) iep_count<kGeneralIep>(c, v, acc);
-        else if (d == k - 2) count_last(c, v, acc);
-        else { ++d; prepare(d); }
+        if constexpr (!kLanes) {
+            if (d == d_iep) { iep_count<kGeneralIep>(c, v, acc); continue; }
+            if (d == k - 2) { count_last(c, v, acc); continue; }
+        }
+        ++d;
+        prepare(d);
     }
 }
 
-template <bool kStats, int kMinBlocks, bool kGeneralIep>
+template <bool kStats, int kMinBlocks, bool kGeneralIep, bool kLanes = false>
 __global__ void __launch_bounds__(kWarps * 32, kMinBlocks)
 k_count(const CountJob* __restrict__ jobs, int njobs, int64_t total,
         unsigned long long* __restrict__ cursor, unsigned long long* __restrict__ results,
@@ -1363,7 +1624,7 @@ k_count(const CountJob* __restrict__ jobs, int njobs, int64_t total,
                 const int hv1 = __ldg(c.col + eh);
                 if (lo1s && !(hv1 > rl)) continue;
                 if (hi1s && !(hv1 < rl)) continue;
-                run_task<kGeneralIep>(c, rl, hv1, acc, part, job_split);
+                run_task<kGeneralIep, kLanes>(c, rl, hv1, acc, part, job_split);
             }
             if (lt >= lt_end) { t = tend; continue; }
             int64_t e = job_begin + job_heavy + (lt - hp);
@@ -1377,7 +1638,7 @@ k_count(const CountJob* __restrict__ jobs, int njobs, int64_t total,
             int v0 = lo;
             int64_t row_end = __ldg(c.row_ptr + v0 + 1);
             const uint8_t lo1 = s_plan[w].lvl[1].lo_mask & 1, hi1 = s_plan[w].lvl[1].hi_mask & 1;
-            if (s_plan[w].k == 3 && s_plan[w].lvl[1].nbuild == 0) {
+            if (!kLanes && s_plan[w].k == 3 && s_plan[w].lvl[1].nbuild == 0) {
                 // one task per lane; heavy ones go to the whole warp
                 int v[GP_MAX_K];
 #pragma unroll
@@ -1418,7 +1679,7 @@ k_count(const CountJob* __restrict__ jobs, int njobs, int64_t total,
                     const int v1 = __ldg(c.col + e);
                     if (lo1 && !(v1 > v0)) continue;
                     if (hi1 && !(v1 < v0)) continue;
-                    run_task<kGeneralIep>(c, v0, v1, acc, 0, 1);
+                    run_task<kGeneralIep, kLanes>(c, v0, v1, acc, 0, 1);
                 }
             }
             t = tend;
@@ -1882,9 +2143,13 @@ gp_status geometry(const CountJob* jobs, int njobs, const LaunchOpts& opt, Geome
     }
     bool general_iep = false;              // some job replaces three or more loops or fuses two
     for (int j = 0; j < njobs; ++j) general_iep |= jobs[j].plan.iep >= 3 || jobs[j].plan.iep_fuse;
+    bool lanes = opt.blocks_per_sm <= 0;   // every job has a lane form
+    for (int j = 0; j < njobs; ++j) lanes &= lane_form(jobs[j].plan);
     if (opt.stats) {
         g->kern = (want == 1 || want == 2) ? k_count<true, 1, true>
                 : (want == 3) ? k_count<true, 3, true> : k_count<true, 4, true>;
+    } else if (lanes) {
+        g->kern = k_count<false, 4, true, true>;
     } else if (general_iep) {
         g->kern = k_count<false, 4, true>;
     } else {
@@ -1935,6 +2200,7 @@ int kernel_variant(const CountJob& job, const LaunchOpts& opt) {
     if (opt.blocks_per_sm <= 0 && !opt.no_core && opt.bitmap_mode == 2 && P.core_dfs && job.core_bits && P.k >= 5 &&
         P.lvl[P.k - 2].bm_inc && P.lvl[P.k - 1].bm_inc)
         want = 3;
+    if (opt.blocks_per_sm <= 0 && !opt.stats && lane_form(P)) return 16;
     return (P.iep >= 3 || P.iep_fuse ? 8 : 0) + want;
 }
 

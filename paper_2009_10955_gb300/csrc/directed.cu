@@ -485,10 +485,12 @@ gp_status run_dcount(const gp_dgraph* g, const DPlan& P, uint64_t div, cudaStrea
     int occ = 0;
     GP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_dcount, kDThreads, 0));
     const int blocks = nsm * std::max(occ, 1);
-    // tasks per grab: three-vertex patterns want full warps; the others up to
-    // 8 (a hub's arcs follow one another) while every warp gets about 16 grabs
-    const int64_t per_warp = g->narcs / ((int64_t)blocks * (kDThreads / 32) * 16);
-    const int chunk = P.k == 3 ? 32 : (int)std::max<int64_t>(1, std::min<int64_t>(8, per_warp));
+    // tasks per grab: three-vertex patterns take four (eight lanes each) to 32,
+    // the others one to eight, while every warp gets about 8 or 16 grabs (a
+    // hub's arcs follow one another)
+    const int64_t warps = (int64_t)blocks * (kDThreads / 32);
+    const int chunk = P.k == 3 ? (int)std::max<int64_t>(4, std::min<int64_t>(32, g->narcs / (warps * 8)))
+                               : (int)std::max<int64_t>(1, std::min<int64_t>(8, g->narcs / (warps * 16)));
     const DLists lists{g->out_ptr, g->out_col, g->in_ptr, g->in_col};
     k_dcount<<<blocks, kDThreads, 0, st>>>(P, g->n, g->narcs, lists, chunk, cursor, res);
     count_launch();

@@ -89,6 +89,8 @@ constexpr int32_t kHeavyDegree = 256;
 constexpr int32_t kHubDegree = 512;
 constexpr int64_t kMostRootWords = (int64_t)1 << 22;
 
+struct ResultWords;          // bits.cuh
+
 struct LaunchOpts {
     int warps_per_block = 8;
     int blocks_per_sm = 0;   // 0 = occupancy maximum
@@ -117,22 +119,20 @@ gp_status run_count(const CountJob* jobs, int njobs, const LaunchOpts& lo, cudaS
 // plan, no option that asks for the general kernel's paths, and a graph
 // whose lists below each vertex are short enough.
 bool clique_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt);
-// The job's 128-bit total (clique.cu); kernel_ms and busy as for run_count.
-gp_status run_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, uint64_t* results,
-                     float* kernel_ms = nullptr, uint64_t* busy = nullptr);
+// Launch it (clique.cu): the 128-bit total and the busy cycles go to `words`
+// on the device; *warps receives the number of warps.
+gp_status launch_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps);
 
 // True when join.cu counts the job: an inclusion-exclusion plan of a clique
 // and vertices adjacent to all of it, on a degree-ordered graph whose root
 // matrices are small enough.
 bool join_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt);
-gp_status run_join(const CountJob& job, const gp_graph* g, cudaStream_t st, uint64_t* results,
-                   float* kernel_ms = nullptr, uint64_t* busy = nullptr);
+gp_status launch_join(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps);
 
 // True when wedge.cu counts the job: the House's inclusion-exclusion plan
 // over all tasks.
 bool wedge_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt);
-gp_status run_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, uint64_t* results,
-                    float* kernel_ms = nullptr, uint64_t* busy = nullptr);
+gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps);
 
 // run_count without allocating: results, job table and intermediate sets all
 // live in the caller's device buffer d_scratch (256-byte aligned); the grid

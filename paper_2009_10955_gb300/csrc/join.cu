@@ -434,8 +434,7 @@ bool join_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt)
     return descending || (job.task_begin == 0 && job.ntasks == g->nnz);
 }
 
-gp_status run_join(const CountJob& job, const gp_graph* g, cudaStream_t st, uint64_t* results, float* kernel_ms,
-                   uint64_t* busy) {
+gp_status launch_join(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps) {
     bool descending = false;
     const int m = join_outer(job.plan, &descending);
     int dev = 0, nsm = 0;
@@ -473,14 +472,15 @@ gp_status run_join(const CountJob& job, const gp_graph* g, cudaStream_t st, uint
         set_error("root matrices need %zu bytes per block; %zu free", per_block, free_b);
         return GP_ERR_SCRATCH;
     }
-    const gp_status rc = run_with_words(st, per_block * (size_t)blocks, kernel_ms, results, busy, "join",
-                                        [&](ResultWords* words, char* mem) {
-        a.words = words;
-        a.big = reinterpret_cast<uint32_t*>(mem);
-        fn<<<(unsigned)blocks, kThreads, smem, st>>>(a);
-    });
-    if (busy) busy[1] = (uint64_t)blocks * kWarps;
-    return rc;
+    LaunchScratch mem(st);
+    GP_CUDA_TRY(mem.alloc(per_block * (size_t)blocks));
+    a.words = words;
+    a.big = reinterpret_cast<uint32_t*>(mem.p);
+    fn<<<(unsigned)blocks, kThreads, smem, st>>>(a);
+    count_launch();
+    GP_CUDA_TRY(cudaGetLastError());
+    *warps = blocks * kWarps;
+    return GP_OK;
 }
 
 }  // namespace gp

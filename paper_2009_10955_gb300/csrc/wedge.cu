@@ -148,8 +148,7 @@ bool wedge_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt
     return g->dplus && job.task_begin == 0 && job.ntasks == g->nnz && is_house_plan(job.plan);
 }
 
-gp_status run_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, uint64_t* results, float* kernel_ms,
-                    uint64_t* busy) {
+gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps) {
     (void)job;
     int dev = 0, nsm = 0;
     GP_CUDA_TRY(cudaGetDevice(&dev));
@@ -178,16 +177,16 @@ gp_status run_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, uin
         while (blocks > 1 && bytes * (size_t)blocks > free_b / 4) blocks = (blocks + 1) / 2;
         extra = sizeof(uint32_t) * (size_t)g->n * (size_t)blocks;
     }
-    cudaError_t e = cudaSuccess;
-    const gp_status rc = run_with_words(st, extra, kernel_ms, results, busy, "wedge", [&](ResultWords* words, char* mem) {
-        a.words = words;
-        a.counters = reinterpret_cast<uint32_t*>(mem);
-        if (extra) e = cudaMemsetAsync(mem, 0, extra, st);
-        fn<<<(unsigned)blocks, threads, smem, st>>>(a);
-    });
-    if (rc == GP_OK && e != cudaSuccess) { set_error("wedge counters: %s", cudaGetErrorString(e)); return GP_ERR_CUDA; }
-    if (busy) busy[1] = (uint64_t)blocks * (threads / 32);
-    return rc;
+    LaunchScratch mem(st);
+    GP_CUDA_TRY(mem.alloc(extra));
+    if (extra) GP_CUDA_TRY(cudaMemsetAsync(mem.p, 0, extra, st));
+    a.words = words;
+    a.counters = reinterpret_cast<uint32_t*>(mem.p);
+    fn<<<(unsigned)blocks, threads, smem, st>>>(a);
+    count_launch();
+    GP_CUDA_TRY(cudaGetLastError());
+    *warps = blocks * (threads / 32);
+    return GP_OK;
 }
 
 }  // namespace gp

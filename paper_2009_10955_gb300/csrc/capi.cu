@@ -69,9 +69,11 @@ gp_status ensure_device(const gp_graph* g) {
     return GP_OK;
 }
 
-// Jobs that a kernel of their own counts (clique.cu, join.cu, wedge.cu).
+// Jobs that a kernel of their own counts (clique.cu, join.cu, wedge.cu, and
+// k_count_root of count.cu).
 bool local_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& lo) {
-    return clique_applies(job, g, lo) || join_applies(job, g, lo) || wedge_applies(job, g, lo);
+    return clique_applies(job, g, lo) || join_applies(job, g, lo) || wedge_applies(job, g, lo) ||
+           root_applies(job, g, lo);
 }
 
 // Count such jobs: one launch each, their results read back together. res has
@@ -93,7 +95,8 @@ gp_status run_local(const CountJob* const* jobs, gp_graph* const* graphs, int n,
     for (int j = 0; j < n && e == cudaSuccess && rc == GP_OK; ++j) {
         int64_t warps = 0;
         const GpPlan& P = jobs[j]->plan;
-        if (!P.iep) rc = launch_clique(*jobs[j], graphs[j], st, words + j, &warps);
+        if (root_applies(*jobs[j], graphs[j], LaunchOpts())) rc = launch_root(*jobs[j], graphs[j], st, words + j, &warps);
+        else if (!P.iep) rc = launch_clique(*jobs[j], graphs[j], st, words + j, &warps);
         else if (wedge_applies(*jobs[j], graphs[j], LaunchOpts())) rc = launch_wedge(*jobs[j], graphs[j], st, words + j, &warps);
         else rc = launch_join(*jobs[j], graphs[j], st, words + j, &warps);
         busy[1] = std::max<uint64_t>(busy[1], (uint64_t)warps);
@@ -188,6 +191,7 @@ gp_status make_job(gp_graph* g, const gp_schedules* s, int32_t idx, const gp_cou
     job->core_n = g->core_n;
     job->core_words = g->core_words;
     job->labels = g->labels;
+    job->dplus = g->dplus;
     if (job->plan.labeled && !g->labels) return fail(GP_ERR_ARG, "labelled pattern on a graph without labels");
     // a term of the five-set inclusion-exclusion expansion multiplies five
     // set sizes: keep it inside 128 bits

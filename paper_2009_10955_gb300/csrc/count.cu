@@ -2079,6 +2079,226 @@ k_label(const CountJob* __restrict__ job, const unsigned long long* __restrict__
     flush(acc, total);
 }
 
+// ---------------------------------------------------------------------------
+// Root counters: plans whose last set is N(v0) ∩ N(v(k-2)) inside a window
+// that only v0 sets (cycles of five and more vertices). A block takes a few
+// edge tasks of one root v0 and counts |N(v0) ∩ N(x)| for all vertices x at
+// once, by walking the lists of v0's neighbours in the window; the last level
+// of a candidate x is then one counter, less the matched vertices in the set,
+// where the lane form intersects two lists (6-cycles of G(2000, 20000): about
+// 1200 warp instructions a round of candidates). The counters are 16-bit
+// halves in shared memory.
+
+__host__ __device__ inline bool root_form(const GpPlan& P) {
+    if (P.labeled || P.core_dfs || P.iep || P.k < 5 || !P.last_count_only || P.lvl[P.k - 2].nbuild) return false;
+    const GpLevel& L = P.lvl[P.k - 1];
+    return P.last_base_kind == 1 && P.last_base == 0 && ((L.lo_mask | L.hi_mask) & ~1) == 0;
+}
+
+__device__ __forceinline__ void root_last_two(const TaskCtx& c, const uint32_t* y, const int* v, List lst, Acc& acc) {
+    const GpPlan& P = *c.P;
+    const int d = P.k - 2;
+    const GpLevel& lv = P.lvl[d + 1];
+    const uint8_t ex = P.lvl[d].excl_mask;
+    const Window w = window(lv.lo_mask, lv.hi_mask, v);
+    // matched vertices in N(v0) and in the window: they are counted in y[x]
+    // where they are neighbours of x
+    bool in = false;
+    if (c.lane < d && (lv.excl_mask >> c.lane & 1)) {
+        const int m = v[c.lane];
+        in = m > w.lo && m < w.hi && member(c, nbr(c, v[0]), m);
+    }
+    const unsigned matched = __ballot_sync(kFull, in);
+    unsigned long long total = 0;
+    for (int base = 0; base < lst.n; base += 32) {
+        const int i = base + c.lane;
+        int x = -1;
+        bool active = i < lst.n;
+        if (active) {
+            x = __ldg(lst.p + i);
+#pragma unroll 1
+            for (int j = 0; j < d; ++j) active &= !(((ex >> j) & 1) && v[j] == x);
+        }
+        int cnt = active ? (int)((y[x >> 1] >> (16 * (x & 1))) & 0xffffu) : 0;
+        for (unsigned m = matched; m; m &= m - 1) {
+            const List l = nbr(c, v[__ffs(m) - 1]);
+            if (cnt > 0 && member(c, l, x)) --cnt;
+        }
+        total += (unsigned)cnt;
+    }
+    acc.add(total);
+}
+
+// Lists up to this length are walked by one lane in root_last_three; longer
+// ones go to the warp.
+constexpr int kRootWalk = 96;
+
+// The last three depths with one candidate z of depth k-3 per lane, for plans
+// whose depth k-2 ranges over N(z): the lane walks that list, adds the
+// counters of its elements and subtracts the matched vertices in their sets (z
+// itself is a neighbour of every one of them). One lane's walk costs what a
+// whole warp's set-up of the loop below it did.
+__device__ __forceinline__ void root_last_three(const TaskCtx& c, const uint32_t* y, int* v, List lst, Acc& acc) {
+    const GpPlan& P = *c.P;
+    const int d = P.k - 3, e = P.k - 2;
+    const GpLevel& le = P.lvl[e];
+    const GpLevel& lL = P.lvl[P.k - 1];
+    const uint8_t ex = P.lvl[d].excl_mask, below = (uint8_t)((1u << d) - 1u);
+    const Window w = window(lL.lo_mask, lL.hi_mask, v);
+    const List root = nbr(c, v[0]);
+    bool in = false;
+    if (c.lane < d && (lL.excl_mask >> c.lane & 1)) {
+        const int m = v[c.lane];
+        in = m > w.lo && m < w.hi && member(c, root, m);
+    }
+    const unsigned matched = __ballot_sync(kFull, in);
+    unsigned long long total = 0;
+    for (int base = 0; base < lst.n; base += 32) {
+        const int i = base + c.lane;
+        int z = -1;
+        bool active = i < lst.n;
+        if (active) {
+            z = __ldg(lst.p + i);
+#pragma unroll 1
+            for (int j = 0; j < d; ++j) active &= !(((ex >> j) & 1) && v[j] == z);
+        }
+        List l{nullptr, 0, -1};
+        Window we{-1, INT_MAX};
+        unsigned own = 0;
+        if (active) {
+            v[d] = z;
+            l = nbr(c, z);
+            we = window(le.lo_mask, le.hi_mask, v);
+            own = (lL.excl_mask >> d & 1) && z > w.lo && z < w.hi && member(c, root, z);
+        }
+        const bool far = l.n > kRootWalk;
+        unsigned far_lanes = __ballot_sync(kFull, far);
+        if (active && !far) {
+            unsigned sum = 0;
+            for (int q = 0; q < l.n; ++q) {
+                const int x = __ldg(l.p + q);
+                if (x >= we.hi) break;
+                unsigned cnt = (y[x >> 1] >> (16 * (x & 1))) & 0xffffu;
+                if (x <= we.lo || cnt == 0) continue;
+                bool hit = false;
+#pragma unroll 1
+                for (unsigned m = le.excl_mask & below; m; m &= m - 1) hit |= v[__ffs(m) - 1] == x;
+                if (hit) continue;
+                cnt -= own;
+#pragma unroll 1
+                for (unsigned m = matched; m; m &= m - 1) cnt -= member(c, nbr(c, v[__ffs(m) - 1]), x);
+                sum += cnt;
+            }
+            total += sum;
+        }
+        __syncwarp();
+        while (far_lanes) {
+            const int src = __ffs(far_lanes) - 1;
+            far_lanes &= far_lanes - 1;
+            v[d] = __shfl_sync(kFull, z, src);
+            root_last_two(c, y, v, clip(nbr(c, v[d]), window(le.lo_mask, le.hi_mask, v)), acc);
+        }
+    }
+    acc.add(total);
+}
+
+__global__ void __launch_bounds__(kWarps * 32, 4)
+k_count_root(const __grid_constant__ CountJob job, int chunk, ResultWords* __restrict__ words,
+             int32_t* __restrict__ slot_pool, int64_t warp_elems, int* __restrict__ err) {
+    extern __shared__ __align__(16) uint32_t s_y[];
+    __shared__ GpPlan s_plan[kWarps];
+    __shared__ int s_len[kWarps][GP_MAX_SLOTS];
+    __shared__ long long s_deadline[kWarps];
+    __shared__ unsigned long long s_item;
+    __shared__ int s_next;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t gw = (int64_t)blockIdx.x * kWarps + warp;
+    const long long t_start = clock64();
+    const TaskCtx c = list_context(&job, &s_plan[warp], s_len[warp], &s_deadline[warp], slot_pool + gw * warp_elems,
+                                   err, lane);
+    const GpPlan& P = s_plan[warp];
+    const int k = P.k;
+    const int64_t end = job.task_begin + job.ntasks;
+    const GpLevel& L1 = P.lvl[1];
+    const GpLevel& LL = P.lvl[k - 1];
+    const bool three = P.lvl[k - 3].nbuild == 0 && P.lvl[k - 2].src_kind == 1 && P.lvl[k - 2].src == k - 3;
+    Acc acc;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_item = atomicAdd(&words->cursor[0], 1ull);
+        __syncthreads();
+        int64_t e = job.task_begin + (int64_t)s_item * chunk;
+        if (e >= end) break;
+        const int64_t e_end = min(e + chunk, end);
+        while (e < e_end) {
+            // the part of one row, cut to what the restriction of v1 leaves
+            const int v0 = row_of(c, e);
+            const int64_t rb = __ldg(c.row_ptr + v0), re = __ldg(c.row_ptr + v0 + 1), mid = rb + __ldg(job.dplus + v0);
+            int64_t b = e, f = min(e_end, re);
+            e = f;
+            if (L1.hi_mask & 1) f = min(f, mid);
+            if (L1.lo_mask & 1) b = max(b, mid);
+            if (b >= f) continue;
+            __syncthreads();                       // the last part's counters and tasks are done with
+            for (int i = 4 * threadIdx.x; i < (job.n + 1) / 2; i += 4 * blockDim.x)
+                *reinterpret_cast<uint4*>(s_y + i) = make_uint4(0, 0, 0, 0);
+            if (threadIdx.x == 0) s_next = 0;
+            __syncthreads();
+            const int64_t ub = (LL.lo_mask & 1) ? mid : rb, ue = (LL.hi_mask & 1) ? mid : re;
+            for (int64_t i = ub + warp; i < ue; i += kWarps) {
+                const List l = nbr(c, __ldg(c.col + i));
+                for (int q = lane; q < l.n; q += 32) {
+                    const int w = __ldg(l.p + q);
+                    atomicAdd(s_y + (w >> 1), (w & 1) ? 65536u : 1u);
+                }
+            }
+            __syncthreads();
+            for (;;) {
+                int t = 0;
+                if (lane == 0) t = atomicAdd(&s_next, 1);
+                t = __shfl_sync(kFull, t, 0);
+                if (b + t >= f) break;
+                int v[GP_MAX_K];
+#pragma unroll
+                for (int i = 0; i < GP_MAX_K; ++i) v[i] = -1;
+                v[0] = v0;
+                v[1] = __ldg(c.col + b + t);
+                List lst[GP_MAX_K];
+                int cur[GP_MAX_K];
+                run_builds(c, 1, v);
+                int d = 2;
+                auto open = [&](int dd) {
+                    const GpLevel& L = P.lvl[dd];
+                    lst[dd] = clip((L.src_kind == 1) ? nbr(c, v[L.src]) : slot(c, L.src), window(L.lo_mask, L.hi_mask, v));
+                    cur[dd] = 0;
+                };
+                open(2);
+                while (d >= 2) {
+                    if (three && d == k - 3) {
+                        root_last_three(c, s_y, v, lst[d], acc);
+                        --d;
+                        continue;
+                    }
+                    if (d == k - 2) {
+                        root_last_two(c, s_y, v, lst[d], acc);
+                        --d;
+                        continue;
+                    }
+                    if (cur[d] >= lst[d].n) { --d; continue; }
+                    const int x = __ldg(lst[d].p + cur[d]);
+                    ++cur[d];
+                    if (taken(P.lvl[d], v, d, x)) continue;
+                    v[d] = x;
+                    run_builds(c, d, v);
+                    open(++d);
+                }
+            }
+        }
+    }
+    flush(acc, words->total);
+    if (lane == 0) atomicAdd(&words->busy, (unsigned long long)(clock64() - t_start));
+}
+
 // Largest c <= ntasks with offsets[c] <= capacity (offsets is an exclusive
 // prefix sum with ntasks + 1 entries): out[0] = c, out[1] = offsets[c].
 __global__ void k_list_cut(const int64_t* __restrict__ offsets, int64_t ntasks, int64_t capacity,
@@ -2385,6 +2605,50 @@ gp_status list_grid(const void* fn, const CountJob& job, int64_t* blocks, int64_
 }
 
 }  // namespace
+
+// Counters up to this many vertices (56 KB: four blocks an SM stay resident).
+constexpr int32_t kRootCounters = 28 * 1024;
+
+bool root_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt) {
+    if (opt.stats || opt.no_core || opt.bitmap_mode != 2 || opt.budget_cycles > 0 || opt.task_cycles > 0) return false;
+    // the largest degree at most 8 times the mean: the tasks of one root stay
+    // with one block, and hubs leave the others idle (5-cycles of R-MAT 9 took
+    // 1.8 times as long as with the lane form)
+    return g->dplus && g->n <= kRootCounters && g->max_deg < 65536 &&
+           (int64_t)g->max_deg * g->n <= 8 * g->nnz && root_form(job.plan);
+}
+
+gp_status launch_root(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps) {
+    const size_t smem = (((size_t)g->n + 1) / 2 * sizeof(uint32_t) + 15) & ~(size_t)15;
+    if (smem > 32 * 1024)
+        GP_CUDA_TRY(cudaFuncSetAttribute(k_count_root, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int dev = 0, nsm = 0, occ = 0;
+    GP_CUDA_TRY(cudaGetDevice(&dev));
+    GP_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    GP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_count_root, kWarps * 32, smem));
+    const int64_t warp_elems = std::max<int64_t>(1, (int64_t)job.plan.nslots * job.slot_cap);
+    const size_t per_block = (size_t)kWarps * (size_t)warp_elems * sizeof(int32_t);
+    size_t free_b = 0, total_b = 0;
+    GP_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
+    int64_t blocks = (int64_t)nsm * std::max(occ, 1);
+    while (blocks > nsm && per_block * (size_t)blocks > free_b / 4) blocks -= nsm;
+    if (per_block * (size_t)blocks > free_b / 2) {
+        set_error("intermediate sets need %zu bytes per block; %zu free", per_block, free_b);
+        return GP_ERR_SCRATCH;
+    }
+    // tasks per grab: enough to use the counters on (their cost is that of a
+    // few tasks), about 8 grabs a block
+    const int chunk = (int)std::max<int64_t>(4, std::min<int64_t>(64, job.ntasks / (blocks * 8)));
+    LaunchScratch mem(st);
+    GP_CUDA_TRY(mem.alloc(256 + per_block * (size_t)blocks));
+    GP_CUDA_TRY(cudaMemsetAsync(mem.p, 0, 256, st));
+    k_count_root<<<(unsigned)blocks, kWarps * 32, smem, st>>>(job, chunk, words, reinterpret_cast<int32_t*>(mem.p + 256),
+                                                             warp_elems, reinterpret_cast<int*>(mem.p));
+    count_launch();
+    GP_CUDA_TRY(cudaGetLastError());
+    *warps = blocks * kWarps;
+    return GP_OK;
+}
 
 gp_status run_labeled(const CountJob& job, cudaStream_t st, uint64_t* results) {
     results[0] = results[1] = 0;

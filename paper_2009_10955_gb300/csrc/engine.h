@@ -73,6 +73,7 @@ struct CountJob {
     const uint32_t* core_bits;  // core adjacency bit matrix (null: none)
     int32_t core_n;
     int32_t core_words;
+    const int32_t* dplus;       // neighbours with a smaller id, per vertex
 };
 
 // Largest core (in vertices) whose adjacency bit matrix a graph keeps:
@@ -133,6 +134,12 @@ gp_status launch_join(const CountJob& job, const gp_graph* g, cudaStream_t st, R
 // over all tasks.
 bool wedge_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt);
 gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps);
+
+// True when k_count_root (count.cu) counts the job: the last set is
+// N(v0) ∩ N(v(k-2)) in a window set by v0, on a graph small enough for its
+// counters.
+bool root_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt);
+gp_status launch_root(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps);
 
 // run_count without allocating: results, job table and intermediate sets all
 // live in the caller's device buffer d_scratch (256-byte aligned); the grid

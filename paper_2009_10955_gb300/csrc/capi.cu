@@ -96,8 +96,8 @@ gp_status run_local(const CountJob* const* jobs, gp_graph* const* graphs, int n,
         int64_t warps = 0;
         const GpPlan& P = jobs[j]->plan;
         if (root_applies(*jobs[j], graphs[j], LaunchOpts())) rc = launch_root(*jobs[j], graphs[j], st, words + j, &warps);
-        else if (!P.iep) rc = launch_clique(*jobs[j], graphs[j], st, words + j, &warps);
         else if (wedge_applies(*jobs[j], graphs[j], LaunchOpts())) rc = launch_wedge(*jobs[j], graphs[j], st, words + j, &warps);
+        else if (!P.iep) rc = launch_clique(*jobs[j], graphs[j], st, words + j, &warps);
         else rc = launch_join(*jobs[j], graphs[j], st, words + j, &warps);
         busy[1] = std::max<uint64_t>(busy[1], (uint64_t)warps);
     }
@@ -750,7 +750,8 @@ gp_status gp_count_batch(gp_graph* const* graphs, const gp_schedules* const* sch
             members.push_back(j);
             chunk = std::min<int64_t>(chunk, jobs[j].nvirt / ((int64_t)nsm * 4 * 8 * 64));
         }
-        lo.chunk = user_chunk > 0 ? user_chunk : (int)std::max<int64_t>(1, chunk);
+        // (tasks that go one per lane take run_count's own rule)
+        lo.chunk = user_chunk > 0 ? user_chunk : lane_tasks(group[0].plan) ? 0 : (int)std::max<int64_t>(1, chunk);
         std::vector<uint64_t> gres(2 * group.size(), 0);
         std::vector<int> gab(group.size(), 0);
         int64_t done = 0;

@@ -146,6 +146,21 @@ __device__ __forceinline__ List nbr(const TaskCtx& c, int v) {
     return List{c.col + b, (int)(e - b), v};
 }
 
+// Row of CSR entry e (the last vertex whose list starts at or before it), the
+// whole warp: 32 pivots a round, so 4 dependent loads instead of 20 on a
+// million vertices.
+__device__ __forceinline__ int warp_row(const TaskCtx& c, int64_t e) {
+    int lo = 0, n = c.n_vertices;              // the row is in [lo, lo + n), row_ptr[lo] <= e
+    while (n > 1) {
+        const int step = (n + 31) >> 5, at = lo + c.lane * step;
+        const bool in = c.lane == 0 || (at < lo + n && __ldg(c.row_ptr + at) <= e);
+        const int last = 31 - __clz(__ballot_sync(kFull, in));
+        lo += last * step;
+        n = min(step, n - last * step);
+    }
+    return lo;
+}
+
 __device__ __forceinline__ List slot(const TaskCtx& c, int s) {
     return List{c.slots + (size_t)s * c.slot_cap, c.slen[s], -1};
 }
@@ -699,11 +714,29 @@ __device__ __noinline__ void iep_count_sets(const TaskCtx& c, const int* v, Acc&
     }
 }
 
+// kk >= 3 inner vertices that share one set S (plan.iep_equal: the leaves of a
+// star): the sum is the falling factorial s (s - 1) ... (s - kk + 1) of its size
+// without matched vertices; nothing is walked.
+__device__ __noinline__ void iep_count_equal(const TaskCtx& c, const int* v, Acc& acc) {
+    const GpPlan& P = *c.P;
+    const int d0 = P.k - P.iep;
+    const GpLevel& L = P.lvl[d0];
+    const Window w = window(L.lo_mask, L.hi_mask, v);
+    const List S = clip((L.src_kind == 1) ? nbr(c, v[L.src]) : slot(c, L.src), w);
+    const int s = S.n - excluded_hits_warp(c, L, d0, v, w, S, nullptr);
+    if (c.lane == 0 && s >= P.iep) {
+        unsigned __int128 p = (unsigned)s;
+        for (int t = 1; t < P.iep; ++t) p *= (unsigned)(s - t);
+        acc.add128((unsigned long long)p, (unsigned long long)(p >> 64));
+    }
+}
+
 // kGeneralIep: the launch may hold plans with kk >= 3 or a fused two-loop
 // form (kernels launched without such plans carry none of that code).
 template <bool kGeneralIep>
 __device__ __forceinline__ void iep_count(const TaskCtx& c, const int* v, Acc& acc) {
     if (!kGeneralIep || c.P->iep == 2) iep_count2<kGeneralIep>(c, v, acc);
+    else if (c.P->iep_equal) iep_count_equal(c, v, acc);
     else iep_count_sets(c, v, acc);
 }
 
@@ -893,8 +926,9 @@ __device__ __forceinline__ int3 iep2_lane_sizes(const TaskCtx& c, const int* v) 
 
 // Then the matched vertices in the sets, and the lane's count. in_a, in_b: the
 // matched vertices in the lists that do not depend on the lane's candidate.
+// all: no list is shared, every matched vertex is looked up.
 __device__ __forceinline__ void iep2_lane_add(const TaskCtx& c, const int* v, unsigned in_a, unsigned in_b, int3 n,
-                                              Acc& acc) {
+                                              Acc& acc, bool all = false) {
     const GpPlan& P = *c.P;
     const int da = P.k - 2, db = P.k - 1, d = P.k - 3;
     int ma = 0, mb = 0, mab = 0;
@@ -922,7 +956,7 @@ __device__ __forceinline__ void iep2_lane_add(const TaskCtx& c, const int* v, un
         const Window wa = window(LA.lo_mask, LA.hi_mask, v), wb = window(LB.lo_mask, LB.hi_mask, v);
         const List A = (LA.src_kind == 1) ? nbr(c, v[LA.src]) : slot(c, LA.src);
         const List B = (LB.src_kind == 1) ? nbr(c, v[LB.src]) : slot(c, LB.src);
-        const bool own_a = LA.src_kind == 1 && LA.src == d, own_b = LB.src_kind == 1 && LB.src == d;
+        const bool own_a = all || (LA.src_kind == 1 && LA.src == d), own_b = all || (LB.src_kind == 1 && LB.src == d);
 #pragma unroll 1
         for (int j = 0; j <= d; ++j) {
             const int x = v[j];
@@ -980,10 +1014,11 @@ __device__ __forceinline__ void lane_form_iep2(const TaskCtx& c, int* v, List ls
     }
 }
 
-// Is the plan's last outer loop one of the above?
+// Is the plan's last outer loop one of the above, or (k = 4) is an edge task
+// itself the last outer vertex, so that a lane takes a task?
 __host__ __device__ inline bool lane_form(const GpPlan& P) {
     if (P.labeled || P.core_dfs || P.k < 4) return false;
-    if (P.iep) return P.iep == 2 && P.k >= 5 && P.lvl[P.k - 3].nbuild == 0;
+    if (P.iep) return P.iep == 2 && P.k >= 4 && P.lvl[P.k - 3].nbuild == 0;
     return P.last_count_only && P.lvl[P.k - 2].nbuild == 0;
 }
 
@@ -1448,7 +1483,8 @@ __device__ void run_task(const TaskCtx& c, int v0, int v1, Acc& acc, int part, i
         if (part != 0) return;                 // no depth-2 loop to share out
         run_builds(c, 1, v);
         if (k == 3) count_last(c, v, acc);
-        else if constexpr (!kLanes) iep_count<kGeneralIep>(c, v, acc);   // (no lane form)
+        else if constexpr (kLanes) iep_count2<true>(c, v, acc);
+        else iep_count<kGeneralIep>(c, v, acc);
         return;
     }
     run_builds(c, 1, v);
@@ -1616,11 +1652,7 @@ k_count(const CountJob* __restrict__ jobs, int njobs, int64_t total,
             for (; lt < lt_end && lt < hp; ++lt) {
                 const int64_t eh = job_begin + lt / job_split;
                 const int part = (int)(lt % job_split);
-                int rl = 0, rh = c.n_vertices - 1;
-                while (rl < rh) {
-                    int mid = (rl + rh + 1) >> 1;
-                    if (__ldg(c.row_ptr + mid) <= eh) rl = mid; else rh = mid - 1;
-                }
+                const int rl = warp_row(c, eh);
                 const int hv1 = __ldg(c.col + eh);
                 if (lo1s && !(hv1 > rl)) continue;
                 if (hi1s && !(hv1 < rl)) continue;
@@ -1629,16 +1661,11 @@ k_count(const CountJob* __restrict__ jobs, int njobs, int64_t total,
             if (lt >= lt_end) { t = tend; continue; }
             int64_t e = job_begin + job_heavy + (lt - hp);
             const int64_t e_end = job_begin + job_heavy + (lt_end - hp);
-            // source vertex of entry e: last u with row_ptr[u] <= e
-            int lo = 0, hi = c.n_vertices - 1;
-            while (lo < hi) {
-                int mid = (lo + hi + 1) >> 1;
-                if (__ldg(c.row_ptr + mid) <= e) lo = mid; else hi = mid - 1;
-            }
-            int v0 = lo;
+            int v0 = warp_row(c, e);           // source vertex of entry e
             int64_t row_end = __ldg(c.row_ptr + v0 + 1);
             const uint8_t lo1 = s_plan[w].lvl[1].lo_mask & 1, hi1 = s_plan[w].lvl[1].hi_mask & 1;
-            if (!kLanes && s_plan[w].k == 3 && s_plan[w].lvl[1].nbuild == 0) {
+            if (kLanes ? s_plan[w].k == 4 && s_plan[w].iep == 2
+                       : s_plan[w].k == 3 && s_plan[w].lvl[1].nbuild == 0) {
                 // one task per lane; heavy ones go to the whole warp
                 int v[GP_MAX_K];
 #pragma unroll
@@ -1659,18 +1686,23 @@ k_count(const CountJob* __restrict__ jobs, int njobs, int64_t total,
                         if (hi1 && !(a1 < a0)) active = false;
                     }
                     bool deferred = false;
+                    int3 n = make_int3(0, 0, 0);
                     if (active) {
                         v[0] = a0;
                         v[1] = a1;
-                        deferred = !count_last_lane(c, v, acc);
+                        if constexpr (kLanes) { n = iep2_lane_sizes(c, v); deferred = n.x < 0; }
+                        else deferred = !count_last_lane(c, v, acc);
                     }
                     unsigned dm = __ballot_sync(kFull, deferred);
+                    if constexpr (kLanes)
+                        if (active && !deferred) iep2_lane_add(c, v, 0u, 0u, n, acc, true);
                     while (dm) {
                         const int src = __ffs(dm) - 1;
                         dm &= dm - 1;
                         v[0] = __shfl_sync(kFull, a0, src);
                         v[1] = __shfl_sync(kFull, a1, src);
-                        count_last(c, v, acc);
+                        if constexpr (kLanes) iep_count2<true>(c, v, acc);
+                        else count_last(c, v, acc);
                     }
                 }
             } else {
@@ -2411,6 +2443,10 @@ gp_status geometry(const CountJob* jobs, int njobs, const LaunchOpts& opt, Geome
 
 }  // namespace
 
+bool lane_tasks(const GpPlan& P) {
+    return !P.labeled && P.lvl[1].nbuild == 0 && (P.k == 3 || (P.k == 4 && lane_form(P) && P.iep));
+}
+
 int kernel_variant(const CountJob& job, const LaunchOpts& opt) {
     // the variant key geometry() would pick for this job alone: general
     // inclusion-exclusion, and the register budget of the default blocks
@@ -2420,7 +2456,10 @@ int kernel_variant(const CountJob& job, const LaunchOpts& opt) {
     if (opt.blocks_per_sm <= 0 && !opt.no_core && opt.bitmap_mode == 2 && P.core_dfs && job.core_bits && P.k >= 5 &&
         P.lvl[P.k - 2].bm_inc && P.lvl[P.k - 1].bm_inc)
         want = 3;
-    if (opt.blocks_per_sm <= 0 && !opt.stats && lane_form(P)) return 16;
+    if (opt.blocks_per_sm <= 0 && !opt.stats) {
+        if (lane_tasks(P)) return P.iep ? 17 : 18;     // grabs of their own size
+        if (lane_form(P)) return 16;
+    }
     return (P.iep >= 3 || P.iep_fuse ? 8 : 0) + want;
 }
 
@@ -2444,8 +2483,12 @@ gp_status run_count(const CountJob* jobs, int njobs, const LaunchOpts& opt, cuda
     auto kern = geo.kern;
     int chunk = opt.chunk;
     if (chunk <= 0) {
-        int64_t per_warp = total / (blocks * kWarps * 64);
-        chunk = (int)std::max<int64_t>(1, std::min<int64_t>(64, per_warp));
+        // tasks that go one per lane want grabs that fill some of the warp even
+        // on small graphs (3-vertex paths of R-MAT 10: 119 us in grabs of one)
+        bool lanes = opt.blocks_per_sm <= 0 && !opt.stats;
+        for (int j = 0; j < njobs; ++j) lanes &= lane_tasks(jobs[j].plan);
+        const int64_t per_warp = total / (blocks * kWarps * (lanes ? 2 : 64));
+        chunk = (int)std::max<int64_t>(lanes ? 8 : 1, std::min<int64_t>(64, per_warp));
     }
 
     // device buffers: job table, results (2 per job), cursor, error word

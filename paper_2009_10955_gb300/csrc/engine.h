@@ -130,8 +130,8 @@ gp_status launch_clique(const CountJob& job, const gp_graph* g, cudaStream_t st,
 bool join_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt);
 gp_status launch_join(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps);
 
-// True when wedge.cu counts the job: the House's inclusion-exclusion plan
-// over all tasks.
+// True when wedge.cu counts the job: the House's inclusion-exclusion plan or
+// the 4-cycle, over all tasks.
 bool wedge_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt);
 gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps);
 
@@ -163,6 +163,9 @@ gp_status run_list(const CountJob& job, int32_t* d_out, int64_t capacity, cudaSt
 
 // The 128-bit count of a labelled plan's job (count.cu).
 gp_status run_labeled(const CountJob& job, cudaStream_t st, uint64_t* results);
+
+// True when the count kernel takes the plan's edge tasks one per lane.
+bool lane_tasks(const GpPlan& P);
 
 // Key of the kernel build geometry() would pick for this job alone (its
 // register budget and whether it carries general inclusion-exclusion); jobs

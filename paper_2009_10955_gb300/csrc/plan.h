@@ -61,6 +61,8 @@ struct GpPlan {
     // the job's total is divided by iep_div.
     int32_t iep;
     uint32_t iep_div;
+    // 1 when all inner vertices draw from one and the same set
+    int32_t iep_equal;
     // 1 when every vertex searched after depth 1 is restricted below v_1:
     // if v_1 is a core vertex the whole remaining search stays among core
     // vertices and runs on their adjacency bit matrix.

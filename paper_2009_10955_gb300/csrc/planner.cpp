@@ -532,6 +532,14 @@ bool compile_plan_iep(const PatternInfo& p, const int8_t* sched, ResMask res, Gp
         // vertices inside an inner candidate set
         const uint8_t outer_mask = (uint8_t)((1u << (k - kk)) - 1u);
         for (int x = k - kk; x < k; ++x) out->lvl[x].excl_mask &= outer_mask;
+        const GpLevel& A = out->lvl[k - kk];
+        out->iep_equal = 1;
+        for (int x = k - kk + 1; x < k; ++x) {
+            const GpLevel& B = out->lvl[x];
+            if (B.src_kind != A.src_kind || B.src != A.src || B.op_mask != A.op_mask || B.lo_mask != A.lo_mask ||
+                B.hi_mask != A.hi_mask || B.excl_mask != A.excl_mask)
+                out->iep_equal = 0;
+        }
         if (kk == 2) fuse_inner_set(out);
         return true;
     }

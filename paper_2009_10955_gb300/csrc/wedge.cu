@@ -14,9 +14,14 @@
 // from both ends of every triangle's edges, so that
 //   total = sum over edges of t (P - d(a) - d(b) + 3) - 2 t^2.
 //
-// What bounds it: the counter updates, sum of squared degrees in all (shared
-// memory atomics where n counters fit, L2 atomics otherwise). Taking b above
-// a reads the shorter lists of a degree-ordered graph.
+// The 4-cycle is counted from the same counters (k_cycle4): with v0 its
+// largest vertex, the last level sums |N(v1) ∩ N(v2)| below v0 over the pairs of
+// smaller neighbours of v0, which is the sum over w < v0 of C(y_w, 2), y_w the
+// number of smaller neighbours of v0 adjacent to w.
+//
+// What bounds it: the counter updates, sum of squared degrees in all for the
+// House (shared memory atomics where n counters fit, L2 atomics otherwise).
+// Taking b above a reads the shorter lists of a degree-ordered graph.
 #include <algorithm>
 
 #include "acc.cuh"
@@ -127,6 +132,75 @@ k_wedge(const __grid_constant__ WedgeArgs a) {
     if (lane == 0) atomicAdd(&a.words->busy, (unsigned long long)(clock64() - t_start));
 }
 
+// C(y, 2) is the sum of the counts found at each increment, so the walk of the
+// smaller neighbours' lists, each up to v0, is all there is.
+template <bool kShared>
+__global__ void __launch_bounds__(1024)
+k_cycle4(const __grid_constant__ WedgeArgs a) {
+    extern __shared__ __align__(16) uint32_t smem[];
+    __shared__ unsigned long long s_item;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const long long t_start = clock64();
+    uint32_t* const y = kShared ? smem : a.counters + (size_t)blockIdx.x * a.n;
+    Acc acc;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_item = atomicAdd(&a.words->cursor[0], 1ull);
+        __syncthreads();
+        if (s_item >= (unsigned long long)a.n) break;
+        const int v = __ldg(a.g.roots + s_item);     // by the number of smaller neighbours, largest first
+        const int d = __ldg(a.g.dplus + v);
+        if (d < 2) break;                            // and so have all that follow
+        const int64_t rb = __ldg(a.g.row_ptr + v);
+        if (kShared) {
+            for (int i = 4 * threadIdx.x; i < v; i += 4 * blockDim.x)
+                *reinterpret_cast<uint4*>(y + i) = make_uint4(0, 0, 0, 0);
+            __syncthreads();
+        }
+        // lane l holds the l-th of this warp's next 32 neighbours
+        auto walk = [&](auto touch) {
+            for (int base = warp; base < d; base += 32 * nwarps) {
+                const int mine = base + lane * nwarps;
+                int64_t b = 0;
+                int len = 0;
+                if (mine < d) {
+                    const int u = __ldg(a.g.col + rb + mine);
+                    b = __ldg(a.g.row_ptr + u);
+                    len = (int)(__ldg(a.g.row_ptr + u + 1) - b);
+                }
+                const int count = min(32, (d - base + nwarps - 1) / nwarps);
+                for (int q = 0; q < count; ++q) {
+                    const int64_t qb = __shfl_sync(kAllLanes, b, q);
+                    const int ql = __shfl_sync(kAllLanes, len, q);
+                    for (int i = lane; i < ql; i += 32) {
+                        const int w = __ldg(a.g.col + qb + i);
+                        if (w >= v) break;
+                        touch(w);
+                    }
+                }
+            }
+        };
+        unsigned long long sum = 0;
+        walk([&](int w) { sum += atomicAdd(y + w, 1u); });
+        acc.add(sum);
+        if (!kShared) {
+            __syncthreads();
+            walk([&](int w) { __stcg(y + w, 0u); });
+        }
+    }
+    flush(acc, a.words->total);
+    if (lane == 0) atomicAdd(&a.words->busy, (unsigned long long)(clock64() - t_start));
+}
+
+bool is_cycle4(const GpPlan& P) {
+    if (P.labeled || P.k != 4 || P.iep) return false;
+    int deg[4] = {0, 0, 0, 0};
+    for (int d = 1; d < 4; ++d)
+        for (int j = 0; j < d; ++j)
+            if (P.lvl[d].op_mask >> j & 1) { ++deg[d]; ++deg[j]; }
+    return deg[0] == 2 && deg[1] == 2 && deg[2] == 2 && deg[3] == 2;
+}
+
 // The House as an inclusion-exclusion plan: v2 joined to one end of the edge
 // (v0, v1), one inner vertex to the other end and v2, the other to both ends;
 // the only restriction left orders v0 and v1.
@@ -145,11 +219,11 @@ bool is_house_plan(const GpPlan& P) {
 bool wedge_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt) {
     if (opt.stats || opt.no_core || opt.bitmap_mode != 2 || opt.budget_cycles > 0 || opt.task_cycles > 0) return false;
     // the exchanged sums hold for all tasks together
-    return g->dplus && job.task_begin == 0 && job.ntasks == g->nnz && is_house_plan(job.plan);
+    return g->dplus && job.task_begin == 0 && job.ntasks == g->nnz && (is_house_plan(job.plan) || is_cycle4(job.plan));
 }
 
 gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps) {
-    (void)job;
+    const bool cycle = is_cycle4(job.plan);
     int dev = 0, nsm = 0;
     GP_CUDA_TRY(cudaGetDevice(&dev));
     GP_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -162,7 +236,7 @@ gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, 
     const size_t bytes = ((size_t)g->n * sizeof(uint32_t) + 15) & ~(size_t)15;
     const bool shared = bytes <= 224 * 1024;
     const int threads = shared && bytes > 110 * 1024 ? 1024 : 512;
-    auto fn = shared ? k_wedge<true> : k_wedge<false>;
+    auto fn = cycle ? (shared ? k_cycle4<true> : k_cycle4<false>) : (shared ? k_wedge<true> : k_wedge<false>);
     const size_t smem = shared ? bytes : 0;
     if (smem > 40 * 1024)
         GP_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

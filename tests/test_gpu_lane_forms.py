@@ -101,3 +101,42 @@ def test_batch_mixes_kernels(oracle_lib):
         scheds.append(s)
     got = N.gp_count_batch([g] * len(names), scheds)
     assert [int(x) for x in got] == [oracle_lib.count(adjacency(name), ref) for name in names]
+
+
+def falling_total(degrees, leaves):
+    return sum(int(np.prod([int(d) - t for t in range(leaves)], dtype=object)) for d in degrees)
+
+
+@pytest.mark.parametrize("leaves", [3, 4, 5, 6])
+def test_stars_share_one_inner_set(leaves):
+    """Three to five inner leaves drawing from one list: a falling factorial."""
+    from math import factorial
+    N = native()
+    src, dst = rmat_edges(7, 8, 0.57, 0.19, 0.19, seed=6)
+    g = N.gp_graph_create_edges(src, dst, 1 << 7, N.GP_DEGREE_ORDER)
+    rows = g.csr()[0]
+    expect = falling_total(np.diff(rows), leaves) // factorial(leaves)
+    s = N.gp_schedule(N.gp_pattern_create(named_pattern(f"star{leaves + 1}")), g, 3)
+    s.set_iep(True)
+    assert [N.gp_count(g, s, i)[1] for i in range(len(s))] == [expect] * len(s)
+
+
+@pytest.mark.parametrize("ordered", [True, False])
+@pytest.mark.parametrize("n,m", [(31, 60), (300, 2500), (5000, 40_000), (70_000, 200_000)])
+def test_four_cycles_by_counters(n, m, ordered):
+    N = native()
+    src, dst = er_edges(n, m, seed=n)
+    g = N.gp_graph_create_edges(src, dst, n, N.GP_DEGREE_ORDER if ordered else 0)
+    mine, general = both(N, g, "c4", False, 6)
+    assert mine == general
+
+
+@pytest.mark.parametrize("name", ["tailed_triangle", "path4", "diamond", "path3", "star4"])
+@pytest.mark.parametrize("n,m,spokes", [(40, 7, 9), (300, 1500, 63), (300, 1500, 70), (9000, 30_000, 400)])
+def test_one_task_per_lane(name, n, m, spokes):
+    N = native()
+    for flags in (N.GP_DEGREE_ORDER, 0):
+        g = N.gp_graph_create_edges(*hub_graph(n, m, n + m, spokes), n + spokes + 11, flags)
+        for iep in (True, False):
+            mine, general = both(N, g, name, iep, 3)
+            assert mine == general

@@ -76,6 +76,14 @@ bool local_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& lo)
            root_applies(job, g, lo);
 }
 
+gp_status launch_local(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps,
+                       uint64_t* need = nullptr) {
+    const LaunchOpts lo;
+    if (root_applies(job, g, lo)) return launch_root(job, g, st, words, warps, need);
+    if (wedge_applies(job, g, lo)) return launch_wedge(job, g, st, words, warps, need);
+    return job.plan.iep ? launch_join(job, g, st, words, warps, need) : launch_clique(job, g, st, words, warps, need);
+}
+
 // Count such jobs: one launch each, their results read back together. res has
 // two words a job; busy as for run_count.
 gp_status run_local(const CountJob* const* jobs, gp_graph* const* graphs, int n, cudaStream_t st,
@@ -94,11 +102,7 @@ gp_status run_local(const CountJob* const* jobs, gp_graph* const* graphs, int n,
     busy[0] = busy[1] = 0;
     for (int j = 0; j < n && e == cudaSuccess && rc == GP_OK; ++j) {
         int64_t warps = 0;
-        const GpPlan& P = jobs[j]->plan;
-        if (root_applies(*jobs[j], graphs[j], LaunchOpts())) rc = launch_root(*jobs[j], graphs[j], st, words + j, &warps);
-        else if (wedge_applies(*jobs[j], graphs[j], LaunchOpts())) rc = launch_wedge(*jobs[j], graphs[j], st, words + j, &warps);
-        else if (!P.iep) rc = launch_clique(*jobs[j], graphs[j], st, words + j, &warps);
-        else rc = launch_join(*jobs[j], graphs[j], st, words + j, &warps);
+        rc = launch_local(*jobs[j], graphs[j], st, words + j, &warps);
         busy[1] = std::max<uint64_t>(busy[1], (uint64_t)warps);
     }
     if (e == cudaSuccess && ms) e = cudaEventRecord(ev[1], st);
@@ -905,7 +909,16 @@ gp_status gp_count_scratch_bytes(const gp_graph* g, const gp_schedules* s, int32
     std::memset(&job, 0, sizeof(job));
     job.plan = s->plans[idx];
     job.slot_cap = g->max_deg > 0 ? g->max_deg : 1;
-    return scratch_bytes(&job, 1, launch_opts(opts), bytes);
+    // the general kernel's sets (time slices use them whatever the plan), or
+    // what the plan's own kernel takes where that is more
+    gp_status rc = scratch_bytes(&job, 1, launch_opts(opts), bytes);
+    job.ntasks = g->nnz;
+    if (rc != GP_OK || job.plan.labeled || !local_applies(job, g, launch_opts(opts))) return rc;
+    uint64_t own = 0;
+    int64_t warps = 0;
+    rc = launch_local(job, g, nullptr, nullptr, &warps, &own);
+    if (rc == GP_OK) *bytes = std::max(*bytes, own);
+    return rc;
 }
 
 }  // extern "C"

@@ -132,6 +132,10 @@ k_wedge(const __grid_constant__ WedgeArgs a) {
     if (lane == 0) atomicAdd(&a.words->busy, (unsigned long long)(clock64() - t_start));
 }
 
+constexpr size_t kSharedCounters = 224 * 1024;
+
+size_t counter_bytes(const gp_graph* g) { return ((size_t)g->n * sizeof(uint32_t) + 15) & ~(size_t)15; }
+
 // C(y, 2) is the sum of the counts found at each increment, so the walk of the
 // smaller neighbours' lists, each up to v0, is all there is.
 template <bool kShared>
@@ -218,11 +222,20 @@ bool is_house_plan(const GpPlan& P) {
 
 bool wedge_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt) {
     if (opt.stats || opt.no_core || opt.bitmap_mode != 2 || opt.budget_cycles > 0 || opt.task_cycles > 0) return false;
-    // the exchanged sums hold for all tasks together
-    return g->dplus && job.task_begin == 0 && job.ntasks == g->nnz && (is_house_plan(job.plan) || is_cycle4(job.plan));
+    // the exchanged sums hold for all tasks together. On sparse graphs of many
+    // vertices the block's turn per vertex (clearing, barriers) outweighs the
+    // lists: House at mean degree 2, 50 K vertices 0.73 against 0.52 ms, 100 K
+    // 1.15 against 0.83 (at 4: 1.33 against 1.75); 4-cycles with counters in
+    // global memory at mean degree 8, 100 K vertices 1.57 against 1.42 ms (at
+    // 20, 200 K: 2.9 against 5.6)
+    const bool cycle = is_cycle4(job.plan);
+    if (cycle ? counter_bytes(g) > kSharedCounters && g->nnz < 14 * (int64_t)g->n
+              : g->n > 16 * 1024 && g->nnz < 4 * (int64_t)g->n - g->n / 4) return false;
+    return g->dplus && job.task_begin == 0 && job.ntasks == g->nnz && (cycle || is_house_plan(job.plan));
 }
 
-gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps) {
+gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps,
+                       uint64_t* need) {
     const bool cycle = is_cycle4(job.plan);
     int dev = 0, nsm = 0;
     GP_CUDA_TRY(cudaGetDevice(&dev));
@@ -233,8 +246,8 @@ gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, 
     a.ordered = g->perm != nullptr;
     // counters in shared memory up to 56 K vertices: several blocks an SM
     // while they fit, one of 1024 threads beyond
-    const size_t bytes = ((size_t)g->n * sizeof(uint32_t) + 15) & ~(size_t)15;
-    const bool shared = bytes <= 224 * 1024;
+    const size_t bytes = counter_bytes(g);
+    const bool shared = bytes <= kSharedCounters;
     const int threads = shared && bytes > 110 * 1024 ? 1024 : 512;
     auto fn = cycle ? (shared ? k_cycle4<true> : k_cycle4<false>) : (shared ? k_wedge<true> : k_wedge<false>);
     const size_t smem = shared ? bytes : 0;
@@ -248,9 +261,12 @@ gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, 
     if (!shared) {
         size_t free_b = 0, total_b = 0;
         GP_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
-        while (blocks > 1 && bytes * (size_t)blocks > free_b / 4) blocks = (blocks + 1) / 2;
+        // no more counters than a fraction of the walks that use them would clear
+        const size_t most = std::min(free_b / 4, std::max<size_t>((size_t)64 << 20, 64 * (size_t)g->nnz));
+        while (blocks > 1 && bytes * (size_t)blocks > most) blocks = (blocks + 1) / 2;
         extra = sizeof(uint32_t) * (size_t)g->n * (size_t)blocks;
     }
+    if (need) { *need = extra; return GP_OK; }
     LaunchScratch mem(st);
     GP_CUDA_TRY(mem.alloc(extra));
     if (extra) GP_CUDA_TRY(cudaMemsetAsync(mem.p, 0, extra, st));

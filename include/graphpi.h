@@ -125,9 +125,8 @@ gp_status gp_pattern_create(const uint8_t* adj, int32_t k, gp_pattern** out);
 /* Vertex-labelled pattern (Section II-A: the method extends to labelled
  * graphs): as gp_pattern_create, plus labels[k]; a vertex matched to
  * pattern vertex a must carry labels[a], and automorphisms must preserve
- * labels. Labelled plans are counted by gp_count (which runs them through
- * the listing kernel's counting pass, without the bit-matrix shortcuts) and
- * listed by gp_list; the batched, time-sliced and no-allocation calls
+ * labels. Labelled plans are counted by gp_count (by a kernel that visits the
+ * edge tasks whose two vertices carry their labels) and listed by gp_list; the batched, time-sliced and no-allocation calls
  * reject them. */
 gp_status gp_pattern_create_labeled(const uint8_t* adj, const int32_t* labels, int32_t k,
                                     gp_pattern** out);
@@ -287,17 +286,19 @@ typedef struct gp_count_opts {
 } gp_count_opts;
 
 /* gp_count_opts.flags */
-#define GP_COUNT_STATS 1   /* run the instrumented kernel that tallies algo_bytes
-                              and algo_ops on the same paths as the plain kernel
-                              (slower; for measurement only)                      */
-#define GP_COUNT_NO_CORE 2 /* never use the core adjacency bit matrix: every
-                              membership test is a binary search                  */
-#define GP_COUNT_WARP_BITMAP 4 /* bitmap subtree: count the last level one
+#define GP_COUNT_STATS 1   /* run the instrumented general kernel that tallies
+                              algo_bytes and algo_ops (slower; for measurement
+                              only: plans that a kernel of their own counts --
+                              cliques, joins of a clique and independent
+                              vertices, the House, cycles -- need less work)      */
+#define GP_COUNT_NO_CORE 2 /* the general kernel without the core adjacency bit
+                              matrix: every membership test is a binary search    */
+#define GP_COUNT_WARP_BITMAP 4 /* general kernel, bitmap subtree: count the last level one
                               candidate at a time with the whole warp (default:
                               one candidate per lane, and for plans whose last
                               two sets are incremental one candidate of depth
                               k-3 per lane running the last three levels)         */
-#define GP_COUNT_LANE_BITMAP 8 /* bitmap subtree: one candidate per lane for the
+#define GP_COUNT_LANE_BITMAP 8 /* general kernel, bitmap subtree: one candidate per lane for the
                               last two levels only (GP_COUNT_WARP_BITMAP wins
                               when both are set)                                  */
 
@@ -314,7 +315,8 @@ gp_status gp_count(gp_graph* g, const gp_schedules* s, int32_t idx, const gp_cou
 
 /* Count several (graph, schedule, plan) jobs in one persistent launch per
  * kernel build (jobs wanting the same register budget and inclusion-
- * exclusion code share one; at most four builds exist); work items of the
+ * exclusion code share one), and one launch for each job that a kernel of
+ * its own counts, read back together; work items of the
  * jobs of a launch share one device work queue. out[j] receives job j's
  * count. All graphs must live on the current device. With opts->raw_total
  * (2 x njobs words) each job's undivided 128-bit total is written there too,
@@ -381,7 +383,7 @@ gp_status gp_list(gp_graph* g, const gp_schedules* s, int32_t idx, int64_t task_
  * must start at zero): calls that overlap on the GPU, from any thread or
  * stream, race and must be serialised by the caller. Counts all edge tasks;
  * writes *out on GP_OK; synchronises `stream`. Also: labelled plans give
- * GP_ERR_ARG (they count through the listing kernel, which allocates);
+ * GP_ERR_ARG (the kernel that counts them allocates);
  * under CUDA's lazy module loading the driver creates the 64 MiB array when
  * the first call on a device loads this code, so that first call reserves
  * the memory; and the call makes the graph's device current and leaves it

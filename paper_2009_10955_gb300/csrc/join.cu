@@ -35,6 +35,7 @@ constexpr int kOwnWords = 1024;     // a warp's matrices (two of 512 words, or o
 constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kListWords = kWarpCols / 2;   // a warp's member list (16-bit positions)
+constexpr int kListPositions = 1 << 16;     // columns such a position can name
 // Root matrices up to this many words stay in shared memory: with the warps'
 // areas 108 KB a block, two blocks an SM.
 constexpr int kBlockWords = 7168;
@@ -314,7 +315,11 @@ k_join(const __grid_constant__ JoinArgs a) {
             if constexpr (M == 3) {
                 count_pairs(F, stride, cols, lo, hi, warp, kWarps, a.kk, lane, acc);
             } else {
-                // rows whose compacted matrix fits a warp's area
+                // rows whose compacted matrix fits a warp's area (and whose
+                // members a warp's list can name)
+                const auto warp_holds = [cols](int2 size) {
+                    return cols <= kListPositions && size.x <= kWarpCols && size.y * stride_of(size.x) <= kOwnWords;
+                };
                 for (;;) {
                     int q = 0;
                     if (lane == 0) q = atomicAdd(&bs.next, 1);
@@ -325,7 +330,7 @@ k_join(const __grid_constant__ JoinArgs a) {
                     const int2 size = row_sizes(row, W, i, lane);
                     const int cs = stride_of(size.x);
                     if (size.y < 2) continue;
-                    if (size.x > kWarpCols || size.y * cs > kOwnWords) {
+                    if (!warp_holds(size)) {
                         if (lane == 0) {
                             const int at = atomicAdd(&bs.n_large, 1);
                             if (at < kMostLarge) bs.large[at] = i;
@@ -346,7 +351,7 @@ k_join(const __grid_constant__ JoinArgs a) {
                 for (int q = 0; q < (noted ? n_large : hi - lo); ++q) {
                     const int i = noted ? bs.large[q] : lo + q;
                     const int2 size = row_sizes(F + (size_t)i * stride, W, i, lane);
-                    if (size.y < 2 || !(size.x > kWarpCols || size.y * stride_of(size.x) > kOwnWords)) continue;
+                    if (size.y < 2 || warp_holds(size)) continue;
                     block_row(F, stride, W, i, size, big_F + a.big_words, big_F + 2 * a.big_words, a.kk, &bs, acc);
                 }
             }

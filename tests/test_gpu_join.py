@@ -77,3 +77,36 @@ def test_against_general_kernel(name, n, edges):
     for a, b in ((0, 0), (0, nnz // 3), (nnz // 3, nnz // 3 + 7), (nnz // 2, nnz)):
         got = N.gp_count_raw(g, s, 0, task_begin=a, task_end=b)
         assert got == N.gp_count_raw(g, s, 0, task_begin=a, task_end=b, flags=N.GP_COUNT_NO_CORE)
+
+
+def hub_and_ring(ring, common):
+    """Four mutually adjacent hubs and `common` vertices adjacent to all of
+    them; the last hub is also joined to a ring of vertices of degree five, so
+    that the common vertices are its last neighbours, behind 3 + ring others;
+    leaves keep the other hubs ahead of it in the degree order."""
+    src, dst = [0, 0, 0, 1, 1, 2], [1, 2, 3, 2, 3, 3]
+    for c in range(4, 4 + common):
+        src += [0, 1, 2, 3]
+        dst += [c] * 4
+    at = 4 + common
+    parts = [(np.array(src), np.array(dst))]
+    r = np.arange(ring)
+    parts += [(np.full(ring, 3), at + r), (at + r, at + (r + 1) % ring), (at + r, at + (r + 2) % ring)]
+    at += ring
+    for hub, leaves in ((2, ring + 1000), (1, ring + 2000), (0, ring + 3000)):
+        parts.append((np.full(leaves, hub), at + np.arange(leaves)))
+        at += leaves
+    return at, np.concatenate([a for a, _ in parts]).astype(np.int32), \
+        np.concatenate([b for _, b in parts]).astype(np.int32)
+
+
+# the common vertices' positions among the last hub's neighbours end at
+# 65535, straddle 65536 and lie beyond it; with 700 of them the row of the
+# other hubs has more members than a warp compacts
+@pytest.mark.parametrize("ring,common", [(65_531, 2), (65_532, 2), (65_533, 3), (70_000, 4), (70_000, 700)])
+def test_positions_beyond_16_bits(ring, common):
+    N = native()
+    n, src, dst = hub_and_ring(ring, common)
+    g = N.gp_graph_create_edges(src, dst, n, N.GP_DEGREE_ORDER)
+    for name in ("k6e", "k4_3"):
+        assert N.gp_count(g, plan(N, g, name), 0)[1] == comb(common, PATTERNS[name][1])

@@ -196,13 +196,41 @@ k_cycle4(const __grid_constant__ WedgeArgs a) {
     if (lane == 0) atomicAdd(&a.words->busy, (unsigned long long)(clock64() - t_start));
 }
 
+// The 4-cycle under restrictions that keep exactly one of its eight maps onto
+// every cycle, whatever the order of the ids. Their number over all 24 orders
+// (what gp_schedule_explicit validates) does not say so: 0 > 1 > 2, 0 > 3 keeps
+// two maps for some orders and none for others, and then the count is the
+// plan's own.
 bool is_cycle4(const GpPlan& P) {
     if (P.labeled || P.k != 4 || P.iep) return false;
-    int deg[4] = {0, 0, 0, 0};
+    uint8_t adj[4] = {};                       // depths joined to depth d
     for (int d = 1; d < 4; ++d)
         for (int j = 0; j < d; ++j)
-            if (P.lvl[d].op_mask >> j & 1) { ++deg[d]; ++deg[j]; }
-    return deg[0] == 2 && deg[1] == 2 && deg[2] == 2 && deg[3] == 2;
+            if (P.lvl[d].op_mask >> j & 1) { adj[d] |= 1 << j; adj[j] |= 1 << d; }
+    for (int d = 0; d < 4; ++d)
+        if (__builtin_popcount(adj[d]) != 2) return false;
+    // four ids form three cycles, each named by the id opposite id 3 and the
+    // image of 8 of the 24 orders: how many of those are kept?
+    int maps[3] = {0, 0, 0};
+    int id[4] = {0, 1, 2, 3};
+    const int across = __builtin_ctz(0xf & ~(adj[0] | 1));
+    do {
+        bool ok = true;
+        for (int d = 1; d < 4; ++d)
+            for (int j = 0; j < d; ++j) {
+                if (P.lvl[d].lo_mask >> j & 1) ok &= id[d] > id[j];
+                if (P.lvl[d].hi_mask >> j & 1) ok &= id[d] < id[j];
+            }
+        if (!ok) continue;
+        int other = 0, at = 0;
+        for (int d = 0; d < 4; ++d)
+            if (id[d] == 3) at = d;
+        if (at == 0 || at == across) other = id[at ^ across];
+        else for (int d = 1; d < 4; ++d)
+            if (d != at && d != across) other = id[d];
+        ++maps[other];
+    } while (std::next_permutation(id, id + 4));
+    return maps[0] == 1 && maps[1] == 1 && maps[2] == 1;
 }
 
 // The House as an inclusion-exclusion plan: v2 joined to one end of the edge

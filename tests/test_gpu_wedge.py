@@ -56,3 +56,19 @@ def test_against_general_kernel(n, m, hub):
         g = N.gp_graph_create_edges(src, dst, n, flags)
         s = plans(N, g, 1)
         assert N.gp_count(g, s, 0) == N.gp_count(g, s, 0, N.make_opts(flags=N.GP_COUNT_NO_CORE))
+
+
+# (0 > 1 > 2, 0 > 3) passes the validation on the complete graph (3 of 24
+# orders) but not on every 4-cycle: it counts some twice and some never
+@pytest.mark.parametrize("res", [[(0, 1), (1, 2), (0, 3)], [(1, 0), (2, 1), (3, 0)], [(0, 1), (0, 2), (0, 3), (1, 3)]])
+def test_four_cycle_under_an_explicit_restriction_set(oracle_lib, res):
+    N = native()
+    src, dst = rmat_edges(8, 8, 0.57, 0.19, 0.19, seed=3)
+    g = N.gp_graph_create_edges(src, dst, 1 << 8)
+    s = N.gp_schedule_explicit(N.gp_pattern_create(named_pattern("c4")), [0, 1, 2, 3], res)
+    expect = oracle_lib.count_restricted(named_pattern("c4"), [0, 1, 2, 3], res,
+                                         oracle_lib.build_csr(1 << 8, src, dst))
+    assert N.gp_count(g, s, 0)[1] == expect
+    nnz = g.device_csr()[2]
+    assert sum(N.gp_count(g, s, 0, N.make_opts(task_begin=a, task_end=b))[1]
+               for a, b in ((0, nnz // 3), (nnz // 3, nnz))) == expect

@@ -54,4 +54,15 @@ struct LaunchScratch {
     cudaError_t alloc(size_t bytes) { return bytes ? cudaMallocAsync((void**)&p, bytes, st) : cudaSuccess; }
 };
 
+// Launches that ask for more dynamic shared memory than this raise their
+// kernel's limit first: the default is 48 KB with the static part, at most
+// 8 KB in the kernels that ever ask for less than this.
+constexpr size_t kDefaultShared = 40 * 1024;
+
+// Raise the dynamic shared memory limit of a kernel, once per device, to
+// `most`: the largest size any launch of it can ask for. The limit belongs to
+// the function, not to a launch, so one set to a launch's own size would be
+// lowered by another thread's smaller launch before this one starts (capi.cu).
+gp_status raise_shared_limit(const void* kernel, size_t most);
+
 }  // namespace gp

@@ -6,7 +6,9 @@
 #include <cstdio>
 #include <cstring>
 #include <memory>
+#include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "bits.cuh"
@@ -254,6 +256,19 @@ bool opts_ok(const gp_count_opts* o) {
 }
 
 }  // namespace
+
+gp_status raise_shared_limit(const void* kernel, size_t most) {
+    static std::mutex mu;
+    static std::vector<std::pair<int, const void*>> raised;       // (device, kernel)
+    int dev = 0;
+    GP_CUDA_TRY(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(mu);
+    const std::pair<int, const void*> key(dev, kernel);
+    if (std::find(raised.begin(), raised.end(), key) != raised.end()) return GP_OK;
+    GP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+    raised.push_back(key);
+    return GP_OK;
+}
 
 gp_status single_job(gp_graph* g, const gp_schedules* s, int32_t idx, CountJob* job) {
     gp_status rc = make_job(g, s, idx, nullptr, job);

@@ -628,10 +628,10 @@ gp_status launch_clique(const CountJob& job, const gp_graph* g, cudaStream_t st,
     a.block_rows = a.n_block > 0 ? std::min(g->max_dplus, kBlockRows) : 0;
     const size_t smem = k == 3 ? 0 : sizeof(uint32_t) * (size_t)var.words(a.block_rows);
     auto fn = var.fn;
-    cudaFuncAttributes fa;
-    GP_CUDA_TRY(cudaFuncGetAttributes(&fa, fn));
-    if (smem + fa.sharedSizeBytes > 48 * 1024)
-        GP_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > kDefaultShared) {
+        const gp_status rc = raise_shared_limit((const void*)fn, sizeof(uint32_t) * (size_t)var.words(kBlockRows));
+        if (rc != GP_OK) return rc;
+    }
     int occ = 0;
     GP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem));
     const int64_t blocks = (int64_t)nsm * std::max(occ, 1);

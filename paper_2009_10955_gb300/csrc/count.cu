@@ -2420,12 +2420,12 @@ gp_status geometry(const CountJob* jobs, int njobs, const LaunchOpts& opt, Geome
     g->smem = (size_t)kWarps * (size_t)g->bm_sets * (size_t)g->bm_stride * sizeof(uint32_t);
     // opt in beyond the 48 KB a block gets by default only when static and
     // dynamic shared memory together need it (seven-vertex cliques on a full
-    // core: 48 KB of bitmaps alone); raising the limit for every launch moved
-    // the shared-memory/L1 split and slowed L1-bound counts
-    cudaFuncAttributes fa;
-    GP_CUDA_TRY(cudaFuncGetAttributes(&fa, g->kern));
-    if (g->smem + fa.sharedSizeBytes > 48 * 1024)
-        GP_CUDA_TRY(cudaFuncSetAttribute(g->kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem));
+    // core: 48 KB of bitmaps alone)
+    if (g->smem > kDefaultShared) {
+        const gp_status rc = raise_shared_limit((const void*)g->kern,
+                                                (size_t)kWarps * (GP_MAX_K - 1) * (kCoreMax / 32) * sizeof(uint32_t));
+        if (rc != GP_OK) return rc;
+    }
     GP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, g->kern, kWarps * 32, g->smem));
     int per_sm = std::min(want, occ);
     if (per_sm < 1) per_sm = 1;
@@ -2664,8 +2664,10 @@ bool root_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt)
 gp_status launch_root(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps,
                        uint64_t* need) {
     const size_t smem = (((size_t)g->n + 1) / 2 * sizeof(uint32_t) + 15) & ~(size_t)15;
-    if (smem > 32 * 1024)
-        GP_CUDA_TRY(cudaFuncSetAttribute(k_count_root, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > kDefaultShared) {
+        const gp_status rc = raise_shared_limit((const void*)k_count_root, kRootCounters / 2 * sizeof(uint32_t));
+        if (rc != GP_OK) return rc;
+    }
     int dev = 0, nsm = 0, occ = 0;
     GP_CUDA_TRY(cudaGetDevice(&dev));
     GP_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));

@@ -458,7 +458,10 @@ gp_status launch_join(const CountJob& job, const gp_graph* g, cudaStream_t st, R
     a.n_roots = std::max(a.n_roots, a.n_block);
     auto fn = m == 2 ? k_join<2> : m == 3 ? k_join<3> : k_join<4>;
     const size_t smem = m == 2 ? 0 : sizeof(uint32_t) * (size_t)(kWarps * (kListWords + kOwnWords) + kBlockWords);
-    if (smem) GP_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem) {
+        const gp_status rc = raise_shared_limit((const void*)fn, smem);
+        if (rc != GP_OK) return rc;
+    }
     int occ = 0;
     GP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kThreads, smem));
     int64_t blocks = (int64_t)nsm * std::max(occ, 1);

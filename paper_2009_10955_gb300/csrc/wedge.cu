@@ -279,8 +279,10 @@ gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, 
     const int threads = shared && bytes > 110 * 1024 ? 1024 : 512;
     auto fn = cycle ? (shared ? k_cycle4<true> : k_cycle4<false>) : (shared ? k_wedge<true> : k_wedge<false>);
     const size_t smem = shared ? bytes : 0;
-    if (smem > 40 * 1024)
-        GP_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > kDefaultShared) {
+        const gp_status rc = raise_shared_limit((const void*)fn, kSharedCounters);
+        if (rc != GP_OK) return rc;
+    }
     int occ = 0;
     GP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem));
     int64_t blocks = (int64_t)nsm * std::max(occ, 1);

@@ -344,8 +344,10 @@ gp_status gp_count_batch_ranges(gp_graph* const* graphs, const gp_schedules* con
                                 const gp_count_opts* opts, void* stream, uint64_t* out,
                                 int64_t* next_task);
 
-/* Device scratch (bytes) a gp_count of plan idx on g allocates for its
- * intermediate sets with the given options (for admission control). */
+/* Device scratch (bytes) the general kernel allocates for the intermediate
+ * sets of plan idx on g with the given options (for admission control): that
+ * of a time slice, whatever the plan, and of every gp_count but those that a
+ * kernel of its own counts, which may take more or less. */
 gp_status gp_count_scratch_bytes(const gp_graph* g, const gp_schedules* s, int32_t idx,
                                  const gp_count_opts* opts, uint64_t* bytes);
 

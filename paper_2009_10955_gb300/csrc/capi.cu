@@ -78,12 +78,11 @@ bool local_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& lo)
            root_applies(job, g, lo);
 }
 
-gp_status launch_local(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps,
-                       uint64_t* need = nullptr) {
+gp_status launch_local(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps) {
     const LaunchOpts lo;
-    if (root_applies(job, g, lo)) return launch_root(job, g, st, words, warps, need);
-    if (wedge_applies(job, g, lo)) return launch_wedge(job, g, st, words, warps, need);
-    return job.plan.iep ? launch_join(job, g, st, words, warps, need) : launch_clique(job, g, st, words, warps, need);
+    if (root_applies(job, g, lo)) return launch_root(job, g, st, words, warps);
+    if (wedge_applies(job, g, lo)) return launch_wedge(job, g, st, words, warps);
+    return job.plan.iep ? launch_join(job, g, st, words, warps) : launch_clique(job, g, st, words, warps);
 }
 
 // Count such jobs: one launch each, their results read back together. res has
@@ -924,16 +923,7 @@ gp_status gp_count_scratch_bytes(const gp_graph* g, const gp_schedules* s, int32
     std::memset(&job, 0, sizeof(job));
     job.plan = s->plans[idx];
     job.slot_cap = g->max_deg > 0 ? g->max_deg : 1;
-    // the general kernel's sets (time slices use them whatever the plan), or
-    // what the plan's own kernel takes where that is more
-    gp_status rc = scratch_bytes(&job, 1, launch_opts(opts), bytes);
-    job.ntasks = g->nnz;
-    if (rc != GP_OK || job.plan.labeled || !local_applies(job, g, launch_opts(opts))) return rc;
-    uint64_t own = 0;
-    int64_t warps = 0;
-    rc = launch_local(job, g, nullptr, nullptr, &warps, &own);
-    if (rc == GP_OK) *bytes = std::max(*bytes, own);
-    return rc;
+    return scratch_bytes(&job, 1, launch_opts(opts), bytes);
 }
 
 }  // extern "C"

@@ -606,8 +606,7 @@ bool clique_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& op
     return descending || (job.task_begin == 0 && job.ntasks == g->nnz);
 }
 
-gp_status launch_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps,
-                       uint64_t* need) {
+gp_status launch_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps) {
     const int k = job.plan.k;
     int dev = 0, nsm = 0;
     GP_CUDA_TRY(cudaGetDevice(&dev));
@@ -648,7 +647,6 @@ gp_status launch_clique(const CountJob& job, const gp_graph* g, cudaStream_t st,
     const size_t big_b = big ? sizeof(uint32_t) * (size_t)blocks * (2 * (size_t)a.big_words + 2 * kMostRows) : 0;
     const size_t sets_b = k >= 6 && a.n_block > 0
         ? sizeof(uint32_t) * (size_t)blocks * (size_t)(threads / 32) * 4 * (kMostRows / 32) : 0;
-    if (need) { *need = big_b + sets_b; return GP_OK; }
     LaunchScratch mem(st);
     GP_CUDA_TRY(mem.alloc(big_b + sets_b));
     a.words = words;

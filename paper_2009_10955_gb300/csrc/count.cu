@@ -2661,8 +2661,7 @@ bool root_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt)
            (int64_t)g->max_deg * g->n <= 8 * g->nnz && root_form(job.plan);
 }
 
-gp_status launch_root(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps,
-                       uint64_t* need) {
+gp_status launch_root(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps) {
     const size_t smem = (((size_t)g->n + 1) / 2 * sizeof(uint32_t) + 15) & ~(size_t)15;
     if (smem > kDefaultShared) {
         const gp_status rc = raise_shared_limit((const void*)k_count_root, kRootCounters / 2 * sizeof(uint32_t));
@@ -2685,7 +2684,6 @@ gp_status launch_root(const CountJob& job, const gp_graph* g, cudaStream_t st, R
     // tasks per grab: enough to use the counters on (their cost is that of a
     // few tasks), about 8 grabs a block
     const int chunk = (int)std::max<int64_t>(4, std::min<int64_t>(64, job.ntasks / (blocks * 8)));
-    if (need) { *need = 256 + per_block * (size_t)blocks; return GP_OK; }
     LaunchScratch mem(st);
     GP_CUDA_TRY(mem.alloc(256 + per_block * (size_t)blocks));
     GP_CUDA_TRY(cudaMemsetAsync(mem.p, 0, 256, st));

@@ -121,30 +121,25 @@ gp_status run_count(const CountJob* jobs, int njobs, const LaunchOpts& lo, cudaS
 // whose lists below each vertex are short enough.
 bool clique_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt);
 // Launch it (clique.cu): the 128-bit total and the busy cycles go to `words`
-// on the device; *warps receives the number of warps. With `need` nothing is
-// launched: it receives the bytes of scratch the launch would allocate.
-gp_status launch_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps,
-                       uint64_t* need = nullptr);
+// on the device; *warps receives the number of warps.
+gp_status launch_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps);
 
 // True when join.cu counts the job: an inclusion-exclusion plan of a clique
 // and vertices adjacent to all of it, on a degree-ordered graph whose root
 // matrices are small enough.
 bool join_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt);
-gp_status launch_join(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps,
-                       uint64_t* need = nullptr);
+gp_status launch_join(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps);
 
 // True when wedge.cu counts the job: the House's inclusion-exclusion plan or
 // the 4-cycle, over all tasks.
 bool wedge_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt);
-gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps,
-                       uint64_t* need = nullptr);
+gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps);
 
 // True when k_count_root (count.cu) counts the job: the last set is
 // N(v0) ∩ N(v(k-2)) in a window set by v0, on a graph small enough for its
 // counters.
 bool root_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt);
-gp_status launch_root(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps,
-                       uint64_t* need = nullptr);
+gp_status launch_root(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps);
 
 // run_count without allocating: results, job table and intermediate sets all
 // live in the caller's device buffer d_scratch (256-byte aligned); the grid

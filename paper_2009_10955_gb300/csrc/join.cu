@@ -439,8 +439,7 @@ bool join_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt)
     return descending || (job.task_begin == 0 && job.ntasks == g->nnz);
 }
 
-gp_status launch_join(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps,
-                       uint64_t* need) {
+gp_status launch_join(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps) {
     bool descending = false;
     const int m = join_outer(job.plan, &descending);
     int dev = 0, nsm = 0;
@@ -481,7 +480,6 @@ gp_status launch_join(const CountJob& job, const gp_graph* g, cudaStream_t st, R
         set_error("root matrices need %zu bytes per block; %zu free", per_block, free_b);
         return GP_ERR_SCRATCH;
     }
-    if (need) { *need = per_block * (size_t)blocks; return GP_OK; }
     LaunchScratch mem(st);
     GP_CUDA_TRY(mem.alloc(per_block * (size_t)blocks));
     a.words = words;

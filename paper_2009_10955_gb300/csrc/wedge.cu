@@ -262,8 +262,7 @@ bool wedge_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt
     return g->dplus && job.task_begin == 0 && job.ntasks == g->nnz && (cycle || is_house_plan(job.plan));
 }
 
-gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps,
-                       uint64_t* need) {
+gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps) {
     const bool cycle = is_cycle4(job.plan);
     int dev = 0, nsm = 0;
     GP_CUDA_TRY(cudaGetDevice(&dev));
@@ -296,7 +295,6 @@ gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, 
         while (blocks > 1 && bytes * (size_t)blocks > most) blocks = (blocks + 1) / 2;
         extra = sizeof(uint32_t) * (size_t)g->n * (size_t)blocks;
     }
-    if (need) { *need = extra; return GP_OK; }
     LaunchScratch mem(st);
     GP_CUDA_TRY(mem.alloc(extra));
     if (extra) GP_CUDA_TRY(cudaMemsetAsync(mem.p, 0, extra, st));

@@ -347,7 +347,8 @@ gp_status gp_count_batch_ranges(gp_graph* const* graphs, const gp_schedules* con
 /* Device scratch (bytes) the general kernel allocates for the intermediate
  * sets of plan idx on g with the given options (for admission control): that
  * of a time slice, whatever the plan, and of every gp_count but those that a
- * kernel of its own counts, which may take more or less. */
+ * kernel of its own counts. Those take up to half of the free memory; where
+ * their scratch does not fit there, the general kernel counts. */
 gp_status gp_count_scratch_bytes(const gp_graph* g, const gp_schedules* s, int32_t idx,
                                  const gp_count_opts* opts, uint64_t* bytes);
 

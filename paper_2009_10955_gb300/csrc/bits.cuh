@@ -51,8 +51,22 @@ struct LaunchScratch {
     char* p = nullptr;
     explicit LaunchScratch(cudaStream_t s) : st(s) {}
     ~LaunchScratch() { if (p) cudaFreeAsync(p, st); }
-    cudaError_t alloc(size_t bytes) { return bytes ? cudaMallocAsync((void**)&p, bytes, st) : cudaSuccess; }
+    // GP_ERR_SCRATCH when the device has no room: the general kernel counts then.
+    gp_status alloc(size_t bytes) {
+        if (bytes == 0) return GP_OK;
+        const cudaError_t e = cudaMallocAsync((void**)&p, bytes, st);
+        if (e == cudaSuccess) return GP_OK;
+        p = nullptr;
+        cudaGetLastError();
+        set_error("cannot allocate %zu bytes of scratch: %s", bytes, cudaGetErrorString(e));
+        return e == cudaErrorMemoryAllocation ? GP_ERR_SCRATCH : GP_ERR_CUDA;
+    }
 };
+
+// Reduce the *blocks of a launch that takes per_block bytes of scratch for each,
+// in whole waves of SMs, until they take a quarter of the free device memory;
+// GP_ERR_SCRATCH where one block an SM takes more than half of it (capi.cu).
+gp_status fit_blocks(int64_t nsm, size_t per_block, int64_t* blocks);
 
 // Launches that ask for more dynamic shared memory than this raise their
 // kernel's limit first: the default is 48 KB with the static part, at most

@@ -86,12 +86,16 @@ gp_status launch_local(const CountJob& job, const gp_graph* g, cudaStream_t st, 
 }
 
 // Count such jobs: one launch each, their results read back together. res has
-// two words a job; busy as for run_count.
+// two words a job; busy as for run_count. counted[j] is 0 for a job whose
+// scratch does not fit the free memory: the general kernel, which takes as few
+// blocks as it must, is left with it.
 gp_status run_local(const CountJob* const* jobs, gp_graph* const* graphs, int n, cudaStream_t st,
-                    uint64_t* const* res, float* ms, uint64_t* busy) {
+                    uint64_t* const* res, float* ms, uint64_t* busy, char* counted) {
     LaunchScratch mem(st);
     const size_t bytes = sizeof(ResultWords) * (size_t)n;
-    GP_CUDA_TRY(mem.alloc(bytes));
+    for (int j = 0; j < n; ++j) counted[j] = 0;
+    gp_status rc = mem.alloc(bytes);
+    if (rc != GP_OK) return rc == GP_ERR_SCRATCH ? GP_ERR_NOMEM : rc;
     ResultWords* words = reinterpret_cast<ResultWords*>(mem.p);
     std::vector<ResultWords> h((size_t)n);
     cudaEvent_t ev[2] = {nullptr, nullptr};
@@ -99,11 +103,12 @@ gp_status run_local(const CountJob* const* jobs, gp_graph* const* graphs, int n,
     for (int i = 0; ms && i < 2 && e == cudaSuccess; ++i) e = cudaEventCreate(&ev[i]);
     if (e == cudaSuccess) e = cudaMemsetAsync(words, 0, bytes, st);
     if (e == cudaSuccess && ms) e = cudaEventRecord(ev[0], st);
-    gp_status rc = GP_OK;
     busy[0] = busy[1] = 0;
     for (int j = 0; j < n && e == cudaSuccess && rc == GP_OK; ++j) {
         int64_t warps = 0;
         rc = launch_local(*jobs[j], graphs[j], st, words + j, &warps);
+        counted[j] = rc == GP_OK;
+        if (rc == GP_ERR_SCRATCH) rc = GP_OK;
         busy[1] = std::max<uint64_t>(busy[1], (uint64_t)warps);
     }
     if (e == cudaSuccess && ms) e = cudaEventRecord(ev[1], st);
@@ -122,11 +127,12 @@ gp_status run_local(const CountJob* const* jobs, gp_graph* const* graphs, int n,
     return GP_OK;
 }
 
-gp_status run_local(const CountJob& job, gp_graph* g, cudaStream_t st, uint64_t* res, float* ms, uint64_t* busy) {
+gp_status run_local(const CountJob& job, gp_graph* g, cudaStream_t st, uint64_t* res, float* ms, uint64_t* busy,
+                    char* counted) {
     const CountJob* jobs[1] = {&job};
     gp_graph* graphs[1] = {g};
     uint64_t* out[1] = {res};
-    return run_local(jobs, graphs, 1, st, out, ms, busy);
+    return run_local(jobs, graphs, 1, st, out, ms, busy, counted);
 }
 
 // Triangle plan: schedule (0, 1, 2) with id(0) > id(1) > id(2).
@@ -156,8 +162,10 @@ gp_status triangle_count(gp_graph* g, cudaStream_t st, uint64_t* out) {
     uint64_t res2[2] = {0, 0};
     int64_t done = 0;
     uint64_t busy[2] = {0, 0};
-    gp_status rc = local_applies(job, g, LaunchOpts()) ? run_local(job, g, st, res2, nullptr, busy)
-                                                       : run_count(&job, 1, LaunchOpts(), st, res2, &done);
+    char counted = 0;
+    gp_status rc = GP_OK;
+    if (local_applies(job, g, LaunchOpts())) rc = run_local(job, g, st, res2, nullptr, busy, &counted);
+    if (rc == GP_OK && !counted) rc = run_count(&job, 1, LaunchOpts(), st, res2, &done);
     if (rc != GP_OK) return rc;
     if (res2[1]) return fail(GP_ERR_OVERFLOW, "triangle count overflows 64 bits");
     *out = res2[0];
@@ -267,6 +275,16 @@ gp_status raise_shared_limit(const void* kernel, size_t most) {
     GP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
     raised.push_back(key);
     return GP_OK;
+}
+
+gp_status fit_blocks(int64_t nsm, size_t per_block, int64_t* blocks) {
+    if (per_block == 0) return GP_OK;
+    size_t free_b = 0, total_b = 0;
+    GP_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
+    while (*blocks > nsm && per_block * (size_t)*blocks > free_b / 4) *blocks -= nsm;
+    if (per_block * (size_t)*blocks <= free_b / 2) return GP_OK;
+    set_error("scratch of %zu bytes per block; %zu free", per_block, free_b);
+    return GP_ERR_SCRATCH;
 }
 
 gp_status single_job(gp_graph* g, const gp_schedules* s, int32_t idx, CountJob* job) {
@@ -661,10 +679,12 @@ gp_status gp_count(gp_graph* g, const gp_schedules* s, int32_t idx, const gp_cou
     const bool want_ms = opts && opts->kernel_ms;
     int aborted = 0;
     uint64_t ops = 0, busy[2] = {0, 0};
+    char counted = 0;
     if (local_applies(job, g, launch_opts(opts))) {
         done = job.nvirt;
-        rc = run_local(job, g, static_cast<cudaStream_t>(stream), res, want_ms ? &ms : nullptr, busy);
-    } else {
+        rc = run_local(job, g, static_cast<cudaStream_t>(stream), res, want_ms ? &ms : nullptr, busy, &counted);
+    }
+    if (rc == GP_OK && !counted) {
         rc = run_count(&job, 1, launch_opts(opts), static_cast<cudaStream_t>(stream), res, &done,
                        want_ms ? &ms : nullptr, &bytes, &aborted, &ops, busy);
     }
@@ -722,11 +742,33 @@ gp_status gp_count_batch(gp_graph* const* graphs, const gp_schedules* const* sch
     const bool want_ms = opts && opts->kernel_ms;
     std::vector<int> aborted((size_t)njobs, 0);
     uint64_t ops = 0, busy[2] = {0, 0};
+    std::vector<int> key((size_t)njobs, 0);   // -1: counted by a kernel of its own
+    {                                         // those: a launch each, one wait for all
+        std::vector<const CountJob*> own;
+        std::vector<gp_graph*> own_graphs;
+        std::vector<uint64_t*> own_res;
+        std::vector<int32_t> members;
+        for (int32_t j = 0; j < njobs; ++j)
+            if (local_applies(jobs[j], graphs[j], lo)) {
+                own.push_back(&jobs[j]);
+                own_graphs.push_back(graphs[j]);
+                own_res.push_back(&res[2 * (size_t)j]);
+                members.push_back(j);
+            }
+        std::vector<char> counted(own.size(), 0);
+        if (!own.empty()) {
+            rc = run_local(own.data(), own_graphs.data(), (int)own.size(), static_cast<cudaStream_t>(stream),
+                           own_res.data(), want_ms ? &ms : nullptr, busy, counted.data());
+            if (rc != GP_OK) return rc;
+        }
+        for (size_t q = 0; q < members.size(); ++q)
+            if (counted[q]) key[members[q]] = -1;
+    }
     // one persistent launch per kernel build: jobs that want different
     // register budgets (or the general inclusion-exclusion code) would
     // otherwise all run with the build the most demanding one needs
-    std::vector<int> key((size_t)njobs);
-    for (int32_t j = 0; j < njobs; ++j) key[j] = local_applies(jobs[j], graphs[j], lo) ? -1 : kernel_variant(jobs[j], lo);
+    for (int32_t j = 0; j < njobs; ++j)
+        if (key[j] != -1) key[j] = kernel_variant(jobs[j], lo);
     std::vector<int> keys(key);
     std::sort(keys.begin(), keys.end());
     keys.erase(std::unique(keys.begin(), keys.end()), keys.end());
@@ -734,22 +776,6 @@ gp_status gp_count_batch(gp_graph* const* graphs, const gp_schedules* const* sch
     GP_CUDA_TRY(cudaGetDevice(&dev));
     GP_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     const int user_chunk = lo.chunk;
-    {                                         // kernels of their own: a launch each, one wait for all
-        std::vector<const CountJob*> own;
-        std::vector<gp_graph*> own_graphs;
-        std::vector<uint64_t*> own_res;
-        for (int32_t j = 0; j < njobs; ++j)
-            if (key[j] == -1) {
-                own.push_back(&jobs[j]);
-                own_graphs.push_back(graphs[j]);
-                own_res.push_back(&res[2 * (size_t)j]);
-            }
-        if (!own.empty()) {
-            rc = run_local(own.data(), own_graphs.data(), (int)own.size(), static_cast<cudaStream_t>(stream),
-                           own_res.data(), want_ms ? &ms : nullptr, busy);
-            if (rc != GP_OK) return rc;
-        }
-    }
     for (int kv : keys) {
         if (kv == -1) continue;
         std::vector<CountJob> group;

@@ -633,25 +633,27 @@ gp_status launch_clique(const CountJob& job, const gp_graph* g, cudaStream_t st,
     }
     int occ = 0;
     GP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem));
-    const int64_t blocks = (int64_t)nsm * std::max(occ, 1);
-    // roots are cut into parts where they are too few to fill the grid evenly
-    a.parts = k <= 4 || a.n_block == 0 ? 1
-              : (int)std::max<int64_t>(1, std::min<int64_t>(k == 5 ? 8 : 64, (k == 5 ? 16 : 64) * blocks / a.n_block));
-    const int64_t n_warp = a.n_roots - a.n_block;
-    a.warp_chunk = (int)std::max<int64_t>(1, std::min<int64_t>(32, n_warp / (blocks * (threads / 32) * 8)));
+    int64_t blocks = (int64_t)nsm * std::max(occ, 1);
     const bool big = (k > 3 && g->max_dplus > kBlockRows) || (k > 4 && g->max_dplus > kWarpRows);
     if (big) {
         a.big_stride = row_stride(g->max_dplus);
         a.big_words = ((int64_t)g->max_dplus * a.big_stride + 3) & ~(int64_t)3;
     }
-    const size_t big_b = big ? sizeof(uint32_t) * (size_t)blocks * (2 * (size_t)a.big_words + 2 * kMostRows) : 0;
-    const size_t sets_b = k >= 6 && a.n_block > 0
-        ? sizeof(uint32_t) * (size_t)blocks * (size_t)(threads / 32) * 4 * (kMostRows / 32) : 0;
+    const size_t big_b = big ? sizeof(uint32_t) * (2 * (size_t)a.big_words + 2 * kMostRows) : 0;
+    const size_t sets_b = k >= 6 && a.n_block > 0 ? sizeof(uint32_t) * (size_t)(threads / 32) * 4 * (kMostRows / 32) : 0;
+    gp_status rc = fit_blocks(nsm, big_b + sets_b, &blocks);
+    if (rc != GP_OK) return rc;
+    // roots are cut into parts where they are too few to fill the grid evenly
+    a.parts = k <= 4 || a.n_block == 0 ? 1
+              : (int)std::max<int64_t>(1, std::min<int64_t>(k == 5 ? 8 : 64, (k == 5 ? 16 : 64) * blocks / a.n_block));
+    const int64_t n_warp = a.n_roots - a.n_block;
+    a.warp_chunk = (int)std::max<int64_t>(1, std::min<int64_t>(32, n_warp / (blocks * (threads / 32) * 8)));
     LaunchScratch mem(st);
-    GP_CUDA_TRY(mem.alloc(big_b + sets_b));
+    rc = mem.alloc((big_b + sets_b) * (size_t)blocks);
+    if (rc != GP_OK) return rc;
     a.words = words;
     a.big = reinterpret_cast<uint32_t*>(mem.p);
-    a.sets = reinterpret_cast<uint32_t*>(mem.p + big_b);
+    a.sets = reinterpret_cast<uint32_t*>(mem.p + big_b * (size_t)blocks);
     fn<<<(unsigned)blocks, threads, smem, st>>>(a);
     count_launch();
     GP_CUDA_TRY(cudaGetLastError());

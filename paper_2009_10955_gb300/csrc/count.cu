@@ -2430,15 +2430,8 @@ gp_status geometry(const CountJob* jobs, int njobs, const LaunchOpts& opt, Geome
     int per_sm = std::min(want, occ);
     if (per_sm < 1) per_sm = 1;
     g->blocks = (int64_t)nsm * per_sm;
-    size_t free_b = 0, total_b = 0;
-    GP_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
     g->per_block = (size_t)kWarps * (size_t)g->warp_elems * sizeof(int32_t);
-    while (g->blocks > nsm && g->per_block * (size_t)g->blocks > free_b / 4) g->blocks -= nsm;
-    if (g->per_block * (size_t)g->blocks > free_b / 2) {
-        set_error("intermediate sets need %zu bytes per block; %zu free", g->per_block, free_b);
-        return GP_ERR_SCRATCH;
-    }
-    return GP_OK;
+    return fit_blocks(nsm, g->per_block, &g->blocks);
 }
 
 }  // namespace
@@ -2673,19 +2666,15 @@ gp_status launch_root(const CountJob& job, const gp_graph* g, cudaStream_t st, R
     GP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_count_root, kWarps * 32, smem));
     const int64_t warp_elems = std::max<int64_t>(1, (int64_t)job.plan.nslots * job.slot_cap);
     const size_t per_block = (size_t)kWarps * (size_t)warp_elems * sizeof(int32_t);
-    size_t free_b = 0, total_b = 0;
-    GP_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
     int64_t blocks = (int64_t)nsm * std::max(occ, 1);
-    while (blocks > nsm && per_block * (size_t)blocks > free_b / 4) blocks -= nsm;
-    if (per_block * (size_t)blocks > free_b / 2) {
-        set_error("intermediate sets need %zu bytes per block; %zu free", per_block, free_b);
-        return GP_ERR_SCRATCH;
-    }
+    gp_status rc = fit_blocks(nsm, per_block, &blocks);
+    if (rc != GP_OK) return rc;
     // tasks per grab: enough to use the counters on (their cost is that of a
     // few tasks), about 8 grabs a block
     const int chunk = (int)std::max<int64_t>(4, std::min<int64_t>(64, job.ntasks / (blocks * 8)));
     LaunchScratch mem(st);
-    GP_CUDA_TRY(mem.alloc(256 + per_block * (size_t)blocks));
+    rc = mem.alloc(256 + per_block * (size_t)blocks);
+    if (rc != GP_OK) return rc;
     GP_CUDA_TRY(cudaMemsetAsync(mem.p, 0, 256, st));
     k_count_root<<<(unsigned)blocks, kWarps * 32, smem, st>>>(job, chunk, words, reinterpret_cast<int32_t*>(mem.p + 256),
                                                              warp_elems, reinterpret_cast<int*>(mem.p));

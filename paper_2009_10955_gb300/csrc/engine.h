@@ -121,7 +121,8 @@ gp_status run_count(const CountJob* jobs, int njobs, const LaunchOpts& lo, cudaS
 // whose lists below each vertex are short enough.
 bool clique_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt);
 // Launch it (clique.cu): the 128-bit total and the busy cycles go to `words`
-// on the device; *warps receives the number of warps.
+// on the device; *warps receives the number of warps. GP_ERR_SCRATCH, and
+// nothing is launched, where its scratch does not fit the free memory.
 gp_status launch_clique(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps);
 
 // True when join.cu counts the job: an inclusion-exclusion plan of a clique

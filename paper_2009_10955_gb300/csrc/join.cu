@@ -472,16 +472,11 @@ gp_status launch_join(const CountJob& job, const gp_graph* g, cudaStream_t st, R
         a.list_words = ((int64_t)g->max_deg + 4) & ~(int64_t)3;
     }
     const size_t per_block = sizeof(uint32_t) * (size_t)(2 * a.big_words + a.list_words);
-    size_t free_b = 0, total_b = 0;
-    GP_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
-    while (blocks > nsm && per_block * (size_t)blocks > free_b / 4) blocks -= nsm;
-    while (blocks > 1 && per_block * (size_t)blocks > free_b / 2) blocks = (blocks + 1) / 2;
-    if (per_block * (size_t)blocks > free_b / 2) {
-        set_error("root matrices need %zu bytes per block; %zu free", per_block, free_b);
-        return GP_ERR_SCRATCH;
-    }
+    gp_status rc = fit_blocks(nsm, per_block, &blocks);
+    if (rc != GP_OK) return rc;
     LaunchScratch mem(st);
-    GP_CUDA_TRY(mem.alloc(per_block * (size_t)blocks));
+    rc = mem.alloc(per_block * (size_t)blocks);
+    if (rc != GP_OK) return rc;
     a.words = words;
     a.big = reinterpret_cast<uint32_t*>(mem.p);
     fn<<<(unsigned)blocks, kThreads, smem, st>>>(a);

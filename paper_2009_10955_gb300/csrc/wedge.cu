@@ -296,7 +296,8 @@ gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, 
         extra = sizeof(uint32_t) * (size_t)g->n * (size_t)blocks;
     }
     LaunchScratch mem(st);
-    GP_CUDA_TRY(mem.alloc(extra));
+    const gp_status rc = mem.alloc(extra);
+    if (rc != GP_OK) return rc;
     if (extra) GP_CUDA_TRY(cudaMemsetAsync(mem.p, 0, extra, st));
     a.words = words;
     a.counters = reinterpret_cast<uint32_t*>(mem.p);

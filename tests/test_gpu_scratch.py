@@ -1,5 +1,7 @@
 """Scratch of the plans that a kernel of their own counts: what the admission
-query answers."""
+query answers, and counts on a device with little memory left."""
+
+from contextlib import contextmanager
 
 import numpy as np
 import pytest
@@ -42,3 +44,43 @@ def test_query_answers_for_time_slices(pattern, graph):
     g = N.gp_graph_create_edges(src, dst, n, N.GP_DEGREE_ORDER)
     s = plan(N, g, pattern)
     assert N.gp_count_scratch_bytes(g, s, 0) == N.gp_count_scratch_bytes(g, s, 0, N.make_opts(budget_cycles=1 << 30))
+
+
+@contextmanager
+def free_megabytes(left):
+    """All device memory but `left` megabytes taken (and never touched)."""
+    torch.cuda.empty_cache()
+    held = []
+    try:
+        while True:
+            free = torch.cuda.mem_get_info()[0] - (left << 20)
+            if free < 4 << 20:
+                break
+            held.append(torch.empty(min(free, 16 << 30) >> 21 << 21, dtype=torch.uint8, device="cuda"))
+        yield
+    finally:
+        held.clear()
+        torch.cuda.empty_cache()
+
+
+# root matrices of 2500 rows take 1.7 MB a block (1.6 MB of K4 plans with two
+# inner vertices), 0.26 GB with one block an SM: with 300 MB left that is more
+# than half of it and the general kernel counts, with 700 MB the grid shrinks.
+# Counters of a million vertices take 4 MB a block
+@pytest.mark.parametrize("pattern,graph,left", [
+    ("k4", lambda: bipartite(2500, 8), 300), ("k5", lambda: bipartite(2500, 8), 300),
+    ("k5", lambda: bipartite(2500, 8), 700), ("k6", lambda: bipartite(2500, 8), 300),
+    ("k6e", lambda: bipartite(2500, 8), 300), ("k6e", lambda: bipartite(2500, 8), 700),
+    ("house", lambda: uniform(1_000_003, 8), 60), ("house", lambda: uniform(1_000_003, 8), 800),
+])
+def test_counts_with_little_memory_left(pattern, graph, left):
+    N = native()
+    n, (src, dst) = graph()
+    g = N.gp_graph_create_edges(src, dst, n, N.GP_DEGREE_ORDER)
+    s = plan(N, g, pattern)
+    t = plan(N, g, "triangle")
+    expect = N.gp_count(g, s, 0)
+    triangles = N.gp_count(g, t, 0)[1]
+    with free_megabytes(left):
+        assert N.gp_count(g, s, 0) == expect
+        assert N.gp_count_batch([g, g, g], [s, t, s], [0] * 3).tolist() == [expect[1], triangles, expect[1]]

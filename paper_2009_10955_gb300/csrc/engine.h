@@ -178,10 +178,13 @@ gp_status scratch_bytes(const CountJob* jobs, int njobs, const LaunchOpts& lo, u
 
 }  // namespace gp
 
+// (a failed call's error is taken out of cudaGetLastError: the next launch's
+// check would find it there)
 #define GP_CUDA_TRY(expr)                                                          \
     do {                                                                           \
         cudaError_t _e = (expr);                                                   \
         if (_e != cudaSuccess) {                                                   \
+            cudaGetLastError();                                                    \
             gp::set_error("%s failed: %s (%s:%d)", #expr, cudaGetErrorString(_e),  \
                           __FILE__, __LINE__);                                     \
             return GP_ERR_CUDA;                                                    \

@@ -84,3 +84,16 @@ def test_counts_with_little_memory_left(pattern, graph, left):
     with free_megabytes(left):
         assert N.gp_count(g, s, 0) == expect
         assert N.gp_count_batch([g, g, g], [s, t, s], [0] * 3).tolist() == [expect[1], triangles, expect[1]]
+
+
+def test_a_failed_call_leaves_no_error_for_the_next():
+    N = native()
+    n, (src, dst) = uniform(2000, 20)
+    g = N.gp_graph_create_edges(src, dst, n, N.GP_DEGREE_ORDER)
+    s = plan(N, g, "triangle")
+    expect = N.gp_count(g, s, 0)
+    many = torch.zeros(1 << 25, dtype=torch.int32, device="cuda")
+    with free_megabytes(300):
+        with pytest.raises(N.GraphPiError):
+            N.gp_graph_create_edges(many, many, 1000, N.GP_DEVICE_PTRS)
+        assert N.gp_count(g, s, 0) == expect

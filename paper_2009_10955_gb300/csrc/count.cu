@@ -2624,7 +2624,10 @@ gp_status run_count_in_scratch(const CountJob* jobs, int njobs, void* d_scratch,
 namespace {
 
 // Grid of a listing kernel: all resident blocks, reduced (in whole waves of
-// SMs) until the per-warp sets fit a quarter of the free device memory.
+// SMs) until the per-warp sets fit a quarter of the free device memory, and
+// below one block an SM where they take more than half of it: a labelled plan
+// has up to three times the sets of the unlabelled one (each holds one label's
+// vertices), and what fitted with those sets still runs.
 gp_status list_grid(const void* fn, const CountJob& job, int64_t* blocks, int64_t* warp_elems, size_t* per_block) {
     int dev = 0, nsm = 0, occ = 0;
     GP_CUDA_TRY(cudaGetDevice(&dev));
@@ -2632,12 +2635,13 @@ gp_status list_grid(const void* fn, const CountJob& job, int64_t* blocks, int64_
     GP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kWarps * 32, 0));
     *warp_elems = (int64_t)(job.plan.nslots + 1) * job.slot_cap;
     *per_block = (size_t)kWarps * (size_t)*warp_elems * sizeof(int32_t);
+    *blocks = (int64_t)nsm * std::max(occ, 1);
+    const gp_status rc = fit_blocks(nsm, *per_block, blocks);
+    if (rc != GP_ERR_SCRATCH || !job.plan.labeled) return rc;
     size_t free_b = 0, total_b = 0;
     GP_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
-    *blocks = (int64_t)nsm * std::max(occ, 1);
-    while (*blocks > nsm && *per_block * (size_t)*blocks > free_b / 4) *blocks -= nsm;
-    if (*per_block * (size_t)*blocks > free_b / 2) { set_error("listing scratch does not fit"); return GP_ERR_SCRATCH; }
-    return GP_OK;
+    *blocks = std::min<int64_t>(*blocks, (int64_t)(free_b / 2 / *per_block));
+    return *blocks > 0 ? GP_OK : rc;
 }
 
 }  // namespace

@@ -97,3 +97,20 @@ def test_a_failed_call_leaves_no_error_for_the_next():
         with pytest.raises(N.GraphPiError):
             N.gp_graph_create_edges(many, many, 1000, N.GP_DEVICE_PTRS)
         assert N.gp_count(g, s, 0) == expect
+
+
+# seven labels: fourteen sets of up to 40,006 vertices a warp and a spare one,
+# 2.9 GB with one block an SM; the four sets of the prefixes alone take 1 GB
+def test_labelled_count_and_list_with_little_memory_left():
+    N = native()
+    leaves = 40_000
+    a, b = np.triu_indices(7, 1)
+    src = np.concatenate([a, np.zeros(leaves)]).astype(np.int32)
+    dst = np.concatenate([b, 7 + np.arange(leaves)]).astype(np.int32)
+    g = N.gp_graph_create_edges(src, dst, 7 + leaves, N.GP_DEGREE_ORDER)
+    N.gp_graph_set_labels(g, (np.arange(7 + leaves) % 7).astype(np.int32))
+    s = N.gp_schedule(N.gp_pattern_create_labeled(named_pattern("k7"), list(range(7))), g, 1)
+    out = torch.zeros((16, 7), dtype=torch.int32, device="cuda")
+    with free_megabytes(2600):
+        assert N.gp_count(g, s, 0) == (N.GP_OK, 1)
+        assert N.gp_list(g, s, 0, 0, 0, out, 16)[:2] == (N.GP_OK, 1)

@@ -40,10 +40,27 @@ static __device__ __forceinline__ void clear_words(uint32_t* M, int words, int f
 }
 
 // Result words of one counting launch, zero before it: the 128-bit total,
-// work cursors, the busy-cycle sum.
+// work cursors, the busy-cycle sum, the error word.
 struct ResultWords {
     unsigned long long total[2], cursor[3], busy;
+    int err;
 };
+
+// The totals of n launches from their words as read back (res: two words
+// each) and the sum of their busy cycles; an error word fails the call.
+inline gp_status read_results(const ResultWords* words, int n, uint64_t* const* res, uint64_t* busy) {
+    *busy = 0;
+    for (int j = 0; j < n; ++j) {
+        if (words[j].err) {
+            set_error("count kernel reported internal error %d", words[j].err);
+            return GP_ERR_INTERNAL;
+        }
+        res[j][0] = words[j].total[0];
+        res[j][1] = words[j].total[1];
+        *busy += words[j].busy;
+    }
+    return GP_OK;
+}
 
 // Stream-ordered scratch of one launch, released behind it.
 struct LaunchScratch {

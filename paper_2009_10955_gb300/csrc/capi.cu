@@ -119,12 +119,7 @@ gp_status run_local(const CountJob* const* jobs, gp_graph* const* graphs, int n,
     for (cudaEvent_t x : ev) if (x) cudaEventDestroy(x);
     if (rc != GP_OK) return rc;
     if (e != cudaSuccess) { set_error("count kernel failed: %s", cudaGetErrorString(e)); return GP_ERR_CUDA; }
-    for (int j = 0; j < n; ++j) {
-        res[j][0] = h[j].total[0];
-        res[j][1] = h[j].total[1];
-        busy[0] += h[j].busy;
-    }
-    return GP_OK;
+    return read_results(h.data(), n, res, &busy[0]);
 }
 
 gp_status run_local(const CountJob& job, gp_graph* g, cudaStream_t st, uint64_t* res, float* ms, uint64_t* busy,

@@ -2236,7 +2236,7 @@ __device__ __forceinline__ void root_last_three(const TaskCtx& c, const uint32_t
 
 __global__ void __launch_bounds__(kWarps * 32, 4)
 k_count_root(const __grid_constant__ CountJob job, int chunk, ResultWords* __restrict__ words,
-             int32_t* __restrict__ slot_pool, int64_t warp_elems, int* __restrict__ err) {
+             int32_t* __restrict__ slot_pool, int64_t warp_elems) {
     extern __shared__ __align__(16) uint32_t s_y[];
     __shared__ GpPlan s_plan[kWarps];
     __shared__ int s_len[kWarps][GP_MAX_SLOTS];
@@ -2247,7 +2247,7 @@ k_count_root(const __grid_constant__ CountJob job, int chunk, ResultWords* __res
     const int64_t gw = (int64_t)blockIdx.x * kWarps + warp;
     const long long t_start = clock64();
     const TaskCtx c = list_context(&job, &s_plan[warp], s_len[warp], &s_deadline[warp], slot_pool + gw * warp_elems,
-                                   err, lane);
+                                   &words->err, lane);
     const GpPlan& P = s_plan[warp];
     const int k = P.k;
     const int64_t end = job.task_begin + job.ntasks;
@@ -2677,11 +2677,10 @@ gp_status launch_root(const CountJob& job, const gp_graph* g, cudaStream_t st, R
     // few tasks), about 8 grabs a block
     const int chunk = (int)std::max<int64_t>(4, std::min<int64_t>(64, job.ntasks / (blocks * 8)));
     LaunchScratch mem(st);
-    rc = mem.alloc(256 + per_block * (size_t)blocks);
+    rc = mem.alloc(per_block * (size_t)blocks);
     if (rc != GP_OK) return rc;
-    GP_CUDA_TRY(cudaMemsetAsync(mem.p, 0, 256, st));
-    k_count_root<<<(unsigned)blocks, kWarps * 32, smem, st>>>(job, chunk, words, reinterpret_cast<int32_t*>(mem.p + 256),
-                                                             warp_elems, reinterpret_cast<int*>(mem.p));
+    k_count_root<<<(unsigned)blocks, kWarps * 32, smem, st>>>(job, chunk, words, reinterpret_cast<int32_t*>(mem.p),
+                                                             warp_elems);
     count_launch();
     GP_CUDA_TRY(cudaGetLastError());
     *warps = blocks * kWarps;

@@ -68,11 +68,38 @@ __device__ __forceinline__ bool adjacent(const CliqueArgs& a, int x, int y) {
     return base < __ldg(a.g.dplus + x) && __ldg(p + base) == y;
 }
 
+// A row of a graph without the degree order by the list of its own vertex x,
+// one warp: a hub of the larger ids has many smaller neighbours with lists
+// shorter than the row, and such a list is looked up in U (5-cliques of R-MAT 14
+// with the ids reversed: 14.9 -> 7.3 ms); short rows cost no more by their
+// pairs. False, nothing written, for the others.
+__device__ __forceinline__ bool walk_row(const CliqueArgs& a, const int32_t* U, int i, int x, uint32_t* row, int stride,
+                                      int lane) {
+    const int len = __ldg(a.g.dplus + x);
+    if (i < 256 || 4 * len >= i) return false;
+    for (int w = lane; w < stride; w += 32) row[w] = 0u;
+    __syncwarp();
+    const int32_t* list = a.g.col + __ldg(a.g.row_ptr + x);
+    for (int e = lane; e < len; e += 32) {
+        const int y = __ldg(list + e);
+        int base = 0, n = i;
+        while (n > 0) {
+            const int half = n >> 1;
+            if (__ldg(U + base + half) < y) { base += half + 1; n -= half + 1; } else n = half;
+        }
+        if (base < i && __ldg(U + base) == y) atomicOr(row + (base >> 5), 1u << (base & 31));
+    }
+    return true;
+}
+
 // Row i of the root's matrix, one warp: a ballot per 32 columns. The words
-// above the diagonal are zero: a compaction reads them.
+// above the diagonal are zero: a compaction reads them. kWalk: 5-cliques and
+// larger ones only, as 4-cliques of such graphs are the general kernel's.
+template <bool kWalk>
 __device__ __forceinline__ void build_row(const CliqueArgs& a, const int32_t* U, int i, uint32_t* row, int stride,
                                           int lane) {
     const int x = __ldg(U + i);
+    if (kWalk && a.g.core_n == 0 && walk_row(a, U, i, x, row, stride, lane)) return;
     const int nw = (i >> 5) + 1;
     for (int w = 0; w < nw; ++w) {
         const int j = 32 * w + lane;
@@ -84,6 +111,7 @@ __device__ __forceinline__ void build_row(const CliqueArgs& a, const int32_t* U,
 }
 
 // Four consecutive rows at once, so that their probes overlap.
+template <bool kWalk>
 __device__ __forceinline__ void build_rows4(const CliqueArgs& a, const int32_t* U, int i0, int n, uint32_t* M,
                                             int stride, int lane) {
     const int last = min(i0 + 3, n - 1);
@@ -92,7 +120,7 @@ __device__ __forceinline__ void build_rows4(const CliqueArgs& a, const int32_t* 
     for (int t = 0; t < 4; ++t) x[t] = __ldg(U + min(i0 + t, last));
     // ids grow with the position: the last row is outside the core first
     if (x[3] >= a.g.core_n) {
-        for (int i = i0; i <= last; ++i) build_row(a, U, i, M + (size_t)i * stride, stride, lane);
+        for (int i = i0; i <= last; ++i) build_row<kWalk>(a, U, i, M + (size_t)i * stride, stride, lane);
         return;
     }
     const int nw = (last >> 5) + 1;
@@ -382,7 +410,7 @@ __device__ __forceinline__ void block_root(const CliqueArgs& a, const int32_t* U
                                            Members bmem, uint32_t* own, Members mem, BlockState* bs, uint32_t* sets,
                                            Acc& acc) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    for (int i = 4 * warp; i < hi; i += 4 * nwarps) build_rows4(a, U, i, hi, L, stride, lane);
+    for (int i = 4 * warp; i < hi; i += 4 * nwarps) build_rows4<(K > 4)>(a, U, i, hi, L, stride, lane);
     if (threadIdx.x == 0) { bs->next = 0; bs->n_large = 0; }
     __syncthreads();
     if constexpr (K == 4) {
@@ -548,7 +576,7 @@ k_clique(const __grid_constant__ CliqueArgs a) {
             } else {
                 const int stride = (hi <= 32) ? 1 : kWarpWords;
                 if (hi <= 32 && lane < (-hi & 3)) own[hi + lane] = 0u;             // one-word rows: zero up to a multiple of four
-                for (int i = 0; i < hi; i += 4) build_rows4(a, U, i, hi, own, stride, lane);
+                for (int i = 0; i < hi; i += 4) build_rows4<(K > 4)>(a, U, i, hi, own, stride, lane);
                 __syncwarp();
                 if (lo == 0) warp_cliques<K - 1, false>(own, mem, hi, 0, hi, lane, acc);
                 else warp_cliques<K - 1, true>(own, mem, hi, lo, hi, lane, acc);
@@ -599,8 +627,13 @@ bool clique_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& op
     // without the degree order a hub's list below it is long and all its pairs
     // are probed, where the general kernel walks the shorter list of each
     // (triangles of an unordered R-MAT 14: 1.58 against 1.44 ms; 5-cliques 1.8
-    // against 35 ms)
-    if (!g->perm && job.plan.k <= 4 && (int64_t)g->max_deg * g->n > 8 * g->nnz) return false;
+    // against 35 ms). Hubs over a sparse rest hold few cliques: with pairs of
+    // smaller neighbours beyond 200 an entry the matrices cost more than the
+    // lists (500 hubs of 3000 neighbours among the largest ids, 658 an entry:
+    // 5-cliques 6.8 against 2.7 ms, 6-cliques 40 against 2.7; R-MAT 14 with the
+    // ids reversed, 109: 7.3 against 232)
+    if (!g->perm && (job.plan.k <= 4 ? (int64_t)g->max_deg * g->n > 8 * g->nnz : g->dplus_pairs > 200.0 * (double)g->nnz))
+        return false;
     // a clique's count over all tasks is the same under every plan; over some
     // of them it is the plan's own
     return descending || (job.task_begin == 0 && job.ntasks == g->nnz);
@@ -643,9 +676,12 @@ gp_status launch_clique(const CountJob& job, const gp_graph* g, cudaStream_t st,
     const size_t sets_b = k >= 6 && a.n_block > 0 ? sizeof(uint32_t) * (size_t)(threads / 32) * 4 * (kMostRows / 32) : 0;
     gp_status rc = fit_blocks(nsm, big_b + sets_b, &blocks);
     if (rc != GP_OK) return rc;
-    // roots are cut into parts where they are too few to fill the grid evenly
+    // roots are cut into parts where they are too few to fill the grid evenly.
+    // Each part builds the root's matrix anew, which is most of the work where
+    // it is large and sparse, as under hubs of a graph without the degree order:
+    // 6-cliques of 500 hubs of 600 neighbours 5.4 ms in 58 parts, 2.4 in 16
     a.parts = k <= 4 || a.n_block == 0 ? 1
-              : (int)std::max<int64_t>(1, std::min<int64_t>(k == 5 ? 8 : 64, (k == 5 ? 16 : 64) * blocks / a.n_block));
+              : (int)std::max<int64_t>(1, std::min<int64_t>(k == 5 ? 8 : g->perm ? 64 : 16, (k == 5 ? 16 : 64) * blocks / a.n_block));
     const int64_t n_warp = a.n_roots - a.n_block;
     a.warp_chunk = (int)std::max<int64_t>(1, std::min<int64_t>(32, n_warp / (blocks * (threads / 32) * 8)));
     LaunchScratch mem(st);

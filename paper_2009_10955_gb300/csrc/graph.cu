@@ -168,12 +168,25 @@ __global__ void k_core_bits(const int64_t* __restrict__ row_ptr, const int32_t* 
     }
 }
 
+// What the host keeps about the finished graph.
+struct GraphInfo {
+    int64_t roots_ge[32];     // entries of the non-increasing `sorted` that are >= 2^i
+    int64_t heavy_end;        // degree-ordered graphs: first entry of the first row shorter than kHeavyDegree
+    int64_t n_hubs;           // degree-ordered graphs: rows longer than kHubDegree
+    unsigned long long max_root_words;
+    double dplus_pairs;       // sum of dplus (dplus - 1) / 2
+    int32_t max_dplus;
+    int32_t max_deg;
+};
+
 // dplus[u]: entries of row u below u (a prefix of the sorted row); the keys
-// and ids to sort by it.
+// and ids to sort by it; the facts that are sums or maxima over all vertices.
 __global__ void k_dplus(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int32_t n,
-                        int32_t* __restrict__ dplus, int32_t* __restrict__ ids,
-                        unsigned long long* __restrict__ max_words) {
+                        int32_t* __restrict__ dplus, int32_t* __restrict__ ids, GraphInfo* __restrict__ out) {
+    __shared__ unsigned long long s_best[kThreads / 32];
+    __shared__ double s_pairs[kThreads / 32];
     unsigned long long best = 0;
+    double pairs = 0;
     for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n;
          u += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = row_ptr[u];
@@ -182,23 +195,23 @@ __global__ void k_dplus(const int64_t* __restrict__ row_ptr, const int32_t* __re
             const int64_t mid = (lo + hi) >> 1;
             if (col[mid] < u) lo = mid + 1; else hi = mid;
         }
-        dplus[u] = (int32_t)(lo - b);
+        const int64_t below = lo - b;
+        dplus[u] = (int32_t)below;
         ids[u] = (int32_t)u;
-        best = max(best, (unsigned long long)(lo - b) * (4 * (unsigned long long)((row_ptr[u + 1] - b + 127) >> 7)));
+        best = max(best, (unsigned long long)below * (4 * (unsigned long long)((row_ptr[u + 1] - b + 127) >> 7)));
+        pairs += 0.5 * (double)below * (double)(below - 1);
     }
-    for (int o = 16; o; o >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, o));
-    if ((threadIdx.x & 31) == 0 && best) atomicMax(max_words, best);
+    for (int o = 16; o; o >>= 1) {
+        best = max(best, __shfl_xor_sync(0xffffffffu, best, o));
+        pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
+    }
+    if ((threadIdx.x & 31) == 0) { s_best[threadIdx.x >> 5] = best; s_pairs[threadIdx.x >> 5] = pairs; }
+    __syncthreads();
+    if (threadIdx.x) return;
+    for (int w = 1; w < kThreads / 32; ++w) { best = max(best, s_best[w]); pairs += s_pairs[w]; }
+    if (best) atomicMax(&out->max_root_words, best);
+    if (pairs > 0) atomicAdd(&out->dplus_pairs, pairs);
 }
-
-// What the host keeps about the finished graph.
-struct GraphInfo {
-    int64_t roots_ge[32];     // entries of the non-increasing `sorted` that are >= 2^i
-    int64_t heavy_end;        // degree-ordered graphs: first entry of the first row shorter than kHeavyDegree
-    int64_t n_hubs;           // degree-ordered graphs: rows longer than kHubDegree
-    unsigned long long max_root_words;
-    int32_t max_dplus;
-    int32_t max_deg;
-};
 
 // One thread per fact; max_deg arrives from k_max_deg unless the rows are
 // ordered by degree.
@@ -267,8 +280,7 @@ gp_status finish_graph(gp_graph* g, cudaStream_t st) {
     GP_CUDA_TRY(info.alloc(sizeof(GraphInfo)));
     GraphInfo* d_info = info.as<GraphInfo>();
     GP_CUDA_TRY(cudaMemsetAsync(d_info, 0, sizeof(GraphInfo), st));
-    k_dplus<<<blocks_for(n), kThreads, 0, st>>>(g->row_ptr, g->col, n, g->dplus, ids.as<int32_t>(),
-                                               &d_info->max_root_words);
+    k_dplus<<<blocks_for(n), kThreads, 0, st>>>(g->row_ptr, g->col, n, g->dplus, ids.as<int32_t>(), d_info);
     size_t tb = 0;
     const int bits = std::max(1, bits_for((uint64_t)n - 1));
     GP_CUDA_TRY(cub::DeviceRadixSort::SortPairsDescending(nullptr, tb, g->dplus, keys.as<int32_t>(), ids.as<int32_t>(),
@@ -294,6 +306,7 @@ gp_status finish_graph(gp_graph* g, cudaStream_t st) {
     g->heavy_end = h.heavy_end;
     g->n_hubs = h.n_hubs;
     g->max_root_words = (int64_t)h.max_root_words;
+    g->dplus_pairs = h.dplus_pairs;
     return GP_OK;
 }
 

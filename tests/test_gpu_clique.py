@@ -77,3 +77,35 @@ def test_general_kernel_agrees_on_ranges():
         for a, b in ((0, nnz // 7), (nnz // 7, nnz // 2), (nnz // 2, nnz // 2 + 33)):
             assert count(g, pattern, task_begin=a, task_end=b) == \
                 count(g, pattern, task_begin=a, task_end=b, flags=N.GP_COUNT_NO_CORE)
+
+
+# without the degree order: hubs of the largest ids whose smaller neighbours
+# have lists much shorter than their rows (looked up in the row's vertices), as
+# long as them (pairs probed) and in between; roots beyond shared memory
+@pytest.mark.parametrize("hubs,rows,low", [(3, 65, 300), (40, 300, 600), (30, 700, 900), (20, 1400, 2000)])
+@pytest.mark.parametrize("k", [5, 6, 7])
+def test_hubs_of_the_largest_ids(k, hubs, rows, low):
+    N = native()
+    rs = np.random.RandomState(rows)
+    core = np.arange(60)                       # a dense part, so that there are cliques
+    a, b = dense_edges(60, 0.7, rows)
+    src = np.concatenate([a, rs.randint(0, low, 3 * low), np.repeat(low + np.arange(hubs), rows + 60)])
+    dst = np.concatenate([b, rs.randint(0, low, 3 * low)] +
+                         [np.concatenate([core, rs.choice(low, rows, replace=False)]) for _ in range(hubs)])
+    g = N.gp_graph_create_edges(src.astype(np.int32), dst.astype(np.int32), low + hubs)
+    assert count(g, f"k{k}") == count(g, f"k{k}", flags=N.GP_COUNT_NO_CORE) > 0
+
+
+# roots of more smaller neighbours than a matrix in shared memory has rows,
+# random ones: over ranges of tasks and whole, against the general kernel
+@pytest.mark.parametrize("n,p", [(700, 0.25), (1300, 0.1)])
+@pytest.mark.parametrize("k", [4, 5, 6, 7])
+def test_random_matrices_beyond_shared_memory(k, n, p):
+    N = native()
+    rs = np.random.RandomState(n)
+    a, b = dense_edges(n, p, n)
+    hub = np.repeat(n + np.arange(4), n)       # joined to every vertex, the last ids in id order
+    src = np.concatenate([a, hub]).astype(np.int32)
+    dst = np.concatenate([b, np.tile(rs.permutation(n), 4)]).astype(np.int32)
+    g = N.gp_graph_create_edges(src, dst, n + 4)
+    assert count(g, f"k{k}") == count(g, f"k{k}", flags=N.GP_COUNT_NO_CORE)

@@ -34,6 +34,7 @@ struct gp_graph {
     int64_t n_hubs = 0;           // degree-ordered graphs: vertices of degree > kHubDegree (a prefix)
     int64_t max_root_words = 0;   // largest dplus x words of a row of degree bits (join.cu)
     double dplus_pairs = 0;       // pairs of smaller neighbours, over all vertices
+    double sum_deg2 = 0;          // sum of squared degrees
     std::mutex mu;
     bool tri_done = false;
     uint64_t tri_cnt = 0;         // ordered triangles (6 x triangles)

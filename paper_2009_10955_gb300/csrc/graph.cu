@@ -175,6 +175,7 @@ struct GraphInfo {
     int64_t n_hubs;           // degree-ordered graphs: rows longer than kHubDegree
     unsigned long long max_root_words;
     double dplus_pairs;       // sum of dplus (dplus - 1) / 2
+    double sum_deg2;          // sum of squared degrees
     int32_t max_dplus;
     int32_t max_deg;
 };
@@ -184,9 +185,9 @@ struct GraphInfo {
 __global__ void k_dplus(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int32_t n,
                         int32_t* __restrict__ dplus, int32_t* __restrict__ ids, GraphInfo* __restrict__ out) {
     __shared__ unsigned long long s_best[kThreads / 32];
-    __shared__ double s_pairs[kThreads / 32];
+    __shared__ double s_pairs[kThreads / 32], s_deg2[kThreads / 32];
     unsigned long long best = 0;
-    double pairs = 0;
+    double pairs = 0, deg2 = 0;
     for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n;
          u += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = row_ptr[u];
@@ -195,22 +196,26 @@ __global__ void k_dplus(const int64_t* __restrict__ row_ptr, const int32_t* __re
             const int64_t mid = (lo + hi) >> 1;
             if (col[mid] < u) lo = mid + 1; else hi = mid;
         }
-        const int64_t below = lo - b;
+        const int64_t below = lo - b, deg = row_ptr[u + 1] - b;
         dplus[u] = (int32_t)below;
         ids[u] = (int32_t)u;
-        best = max(best, (unsigned long long)below * (4 * (unsigned long long)((row_ptr[u + 1] - b + 127) >> 7)));
+        best = max(best, (unsigned long long)below * (4 * (unsigned long long)((deg + 127) >> 7)));
         pairs += 0.5 * (double)below * (double)(below - 1);
+        deg2 += (double)deg * (double)deg;
     }
     for (int o = 16; o; o >>= 1) {
         best = max(best, __shfl_xor_sync(0xffffffffu, best, o));
         pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
+        deg2 += __shfl_xor_sync(0xffffffffu, deg2, o);
     }
-    if ((threadIdx.x & 31) == 0) { s_best[threadIdx.x >> 5] = best; s_pairs[threadIdx.x >> 5] = pairs; }
+    const int warp = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) { s_best[warp] = best; s_pairs[warp] = pairs; s_deg2[warp] = deg2; }
     __syncthreads();
     if (threadIdx.x) return;
-    for (int w = 1; w < kThreads / 32; ++w) { best = max(best, s_best[w]); pairs += s_pairs[w]; }
+    for (int w = 1; w < kThreads / 32; ++w) { best = max(best, s_best[w]); pairs += s_pairs[w]; deg2 += s_deg2[w]; }
     if (best) atomicMax(&out->max_root_words, best);
     if (pairs > 0) atomicAdd(&out->dplus_pairs, pairs);
+    if (deg2 > 0) atomicAdd(&out->sum_deg2, deg2);
 }
 
 // One thread per fact; max_deg arrives from k_max_deg unless the rows are
@@ -307,6 +312,7 @@ gp_status finish_graph(gp_graph* g, cudaStream_t st) {
     g->n_hubs = h.n_hubs;
     g->max_root_words = (int64_t)h.max_root_words;
     g->dplus_pairs = h.dplus_pairs;
+    g->sum_deg2 = h.sum_deg2;
     return GP_OK;
 }
 

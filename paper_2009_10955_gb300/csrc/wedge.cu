@@ -248,18 +248,47 @@ bool is_house_plan(const GpPlan& P) {
 
 }  // namespace
 
+namespace {
+
+// Blocks of a launch with counters in global memory: four of 512 threads an SM,
+// halved until clearing the counters costs no more than a fraction of the walks
+// that use them.
+int64_t global_blocks(const gp_graph* g, int64_t nsm) {
+    int64_t blocks = nsm * 4;
+    const size_t most = std::max<size_t>((size_t)64 << 20, 64 * (size_t)g->nnz);
+    while (blocks > 1 && counter_bytes(g) * (size_t)blocks > most) blocks = (blocks + 1) / 2;
+    return blocks;
+}
+
+// Is the House worth counters in global memory in this many blocks? The general
+// kernel takes about 0.15 ns per wedge (sum of squared degrees), a block 2 to 3
+// us per vertex, more where all counters together exceed the L2. Measured on
+// uniform graphs (general : counters, ms): 100 K vertices of mean degree 4
+// 1.35 : 1.28, 8 1.72 : 1.46; 200 K of 8 2.4 : 5.5, 12 4.1 : 4.0; 1 M of 8
+// 10.0 : 38, 12 18.8 : 25, 16 31.8 : 29.7, 20 50 : 22.
+bool house_pays(const gp_graph* g, int64_t blocks) {
+    const double line = g->n <= 128 * 1024 ? 2800.0 : counter_bytes(g) * (double)blocks <= 128e6 ? 22000.0 : 38000.0;
+    return (double)blocks * g->sum_deg2 >= line * (double)g->n;
+}
+
+}  // namespace
+
 bool wedge_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt) {
     if (opt.stats || opt.no_core || opt.bitmap_mode != 2 || opt.budget_cycles > 0 || opt.task_cycles > 0) return false;
-    // the exchanged sums hold for all tasks together. On sparse graphs of many
-    // vertices the block's turn per vertex (clearing, barriers) outweighs the
-    // lists: House at mean degree 2, 50 K vertices 0.73 against 0.52 ms, 100 K
-    // 1.15 against 0.83 (at 4: 1.33 against 1.75); 4-cycles with counters in
-    // global memory at mean degree 8, 100 K vertices 1.57 against 1.42 ms (at
-    // 20, 200 K: 2.9 against 5.6)
-    const bool cycle = is_cycle4(job.plan);
-    if (cycle ? counter_bytes(g) > kSharedCounters && g->nnz < 14 * (int64_t)g->n
-              : g->n > 16 * 1024 && g->nnz < 4 * (int64_t)g->n - g->n / 4) return false;
-    return g->dplus && job.task_begin == 0 && job.ntasks == g->nnz && (cycle || is_house_plan(job.plan));
+    // the exchanged sums hold for all tasks together
+    if (!g->dplus || job.task_begin != 0 || job.ntasks != g->nnz) return false;
+    const bool global = counter_bytes(g) > kSharedCounters;
+    // On sparse graphs of many vertices the block's turn per vertex (clearing,
+    // barriers) outweighs the lists: House at mean degree 2, 50 K vertices 0.73
+    // against 0.52 ms; 4-cycles with counters in global memory at mean degree 8,
+    // 100 K vertices 1.57 against 1.42 ms (at 20, 200 K: 2.9 against 5.6)
+    if (is_cycle4(job.plan)) return !global || g->nnz >= 14 * (int64_t)g->n;
+    if (!is_house_plan(job.plan)) return false;
+    if (!global) return g->n <= 16 * 1024 || g->nnz >= 4 * (int64_t)g->n - g->n / 4;
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
+    return house_pays(g, global_blocks(g, nsm));
 }
 
 gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps) {
@@ -282,17 +311,22 @@ gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, 
         const gp_status rc = raise_shared_limit((const void*)fn, kSharedCounters);
         if (rc != GP_OK) return rc;
     }
-    int occ = 0;
-    GP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem));
-    int64_t blocks = (int64_t)nsm * std::max(occ, 1);
-    blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, g->n));
+    int64_t blocks = 0;
     size_t extra = 0;
-    if (!shared) {
+    if (shared) {
+        int occ = 0;
+        GP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem));
+        blocks = std::max<int64_t>(1, std::min<int64_t>((int64_t)nsm * std::max(occ, 1), g->n));
+    } else {
         size_t free_b = 0, total_b = 0;
         GP_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
-        // no more counters than a fraction of the walks that use them would clear
-        const size_t most = std::min(free_b / 4, std::max<size_t>((size_t)64 << 20, 64 * (size_t)g->nnz));
-        while (blocks > 1 && bytes * (size_t)blocks > most) blocks = (blocks + 1) / 2;
+        blocks = global_blocks(g, nsm);
+        const int64_t wanted = blocks;
+        while (blocks > 1 && bytes * (size_t)blocks > free_b / 4) blocks = (blocks + 1) / 2;
+        if (bytes * (size_t)blocks > free_b / 4 || (cycle ? 4 * blocks < wanted : !house_pays(g, blocks))) {
+            set_error("counters of %zu bytes per block; %zu free", bytes, free_b);
+            return GP_ERR_SCRATCH;
+        }
         extra = sizeof(uint32_t) * (size_t)g->n * (size_t)blocks;
     }
     LaunchScratch mem(st);

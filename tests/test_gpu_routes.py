@@ -37,11 +37,17 @@ def best(call):
     return min(times), got
 
 
-# without the check these took 18, 110 and 36 times as long as the general kernel
+def uniform(n, degree):
+    return n, er_edges(n, n * degree // 2, seed=n)
+
+
+# without the check these took 18, 110, 36, 5 and 4 times as long as the general kernel
 @pytest.mark.parametrize("pattern,ordered,graph", [
     ("k5", False, lambda: late_hubs(500, 3000)),
     ("k6", False, lambda: late_hubs(500, 3000)),
     ("k6", False, lambda: late_hubs(10, 4000)),
+    ("house", True, lambda: uniform(1_000_000, 4)),
+    ("house", False, lambda: uniform(500_000, 4)),
 ])
 def test_not_much_slower_than_the_general_kernel(pattern, ordered, graph):
     N = native()

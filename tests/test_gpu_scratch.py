@@ -71,7 +71,8 @@ def free_megabytes(left):
     ("k4", lambda: bipartite(2500, 8), 300), ("k5", lambda: bipartite(2500, 8), 300),
     ("k5", lambda: bipartite(2500, 8), 700), ("k6", lambda: bipartite(2500, 8), 300),
     ("k6e", lambda: bipartite(2500, 8), 300), ("k6e", lambda: bipartite(2500, 8), 700),
-    ("house", lambda: uniform(1_000_003, 8), 60), ("house", lambda: uniform(1_000_003, 8), 800),
+    ("house", lambda: uniform(1_000_003, 16), 60), ("house", lambda: uniform(1_000_003, 16), 800),
+    ("c4", lambda: uniform(1_000_003, 24), 300), ("c4", lambda: uniform(1_000_003, 24), 3000),
 ])
 def test_counts_with_little_memory_left(pattern, graph, left):
     N = native()

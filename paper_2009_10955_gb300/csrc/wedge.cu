@@ -136,20 +136,30 @@ constexpr size_t kSharedCounters = 224 * 1024;
 
 size_t counter_bytes(const gp_graph* g) { return ((size_t)g->n * sizeof(uint32_t) + 15) & ~(size_t)15; }
 
+// Lists longer than this are set aside by the warps and shared out in the
+// block afterwards (k_cycle4): one warp takes 270 cycles for 32 elements, and
+// under a hub the others wait for it (two hubs joined to 30 K vertices: 12.8 ->
+// 1.3 ms, Chung-Lu of 1 M vertices 500 -> 171; 500 hubs of 3000 neighbours lose
+// 6 % to the barrier).
+constexpr int kSetAside = 512;
+constexpr int kMostAside = 256;
+
 // C(y, 2) is the sum of the counts found at each increment, so the walk of the
-// smaller neighbours' lists, each up to v0, is all there is.
-template <bool kShared>
+// smaller neighbours' lists, each up to v0, is all there is. kLong: the graph
+// has lists to set aside (the extra barrier costs the others 3 %).
+template <bool kShared, bool kLong>
 __global__ void __launch_bounds__(1024)
 k_cycle4(const __grid_constant__ WedgeArgs a) {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ unsigned long long s_item;
+    __shared__ int s_aside[kLong ? kMostAside : 1], s_n_aside;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const long long t_start = clock64();
     uint32_t* const y = kShared ? smem : a.counters + (size_t)blockIdx.x * a.n;
     Acc acc;
     for (;;) {
         __syncthreads();
-        if (threadIdx.x == 0) s_item = atomicAdd(&a.words->cursor[0], 1ull);
+        if (threadIdx.x == 0) { s_item = atomicAdd(&a.words->cursor[0], 1ull); s_n_aside = 0; }
         __syncthreads();
         if (s_item >= (unsigned long long)a.n) break;
         const int v = __ldg(a.g.roots + s_item);     // by the number of smaller neighbours, largest first
@@ -171,6 +181,10 @@ k_cycle4(const __grid_constant__ WedgeArgs a) {
                     const int u = __ldg(a.g.col + rb + mine);
                     b = __ldg(a.g.row_ptr + u);
                     len = (int)(__ldg(a.g.row_ptr + u + 1) - b);
+                    if (kLong && len > kSetAside) {
+                        const int at = atomicAdd(&s_n_aside, 1);
+                        if (at < kMostAside) { s_aside[at] = u; len = 0; }
+                    }
                 }
                 const int count = min(32, (d - base + nwarps - 1) / nwarps);
                 for (int q = 0; q < count; ++q) {
@@ -183,12 +197,32 @@ k_cycle4(const __grid_constant__ WedgeArgs a) {
                     }
                 }
             }
+            if constexpr (kLong) {
+                __syncthreads();
+                // a warp each where they are enough to go around, the block
+                // one after the other where they are few
+                const int n_aside = min(s_n_aside, kMostAside);
+                const bool each = n_aside >= nwarps;
+                const int step = each ? 32 : (int)blockDim.x;
+                for (int q = each ? warp : 0; q < n_aside; q += each ? nwarps : 1) {
+                    const int64_t b = __ldg(a.g.row_ptr + s_aside[q]), e = __ldg(a.g.row_ptr + s_aside[q] + 1);
+                    for (int64_t i = b + (each ? lane : (int)threadIdx.x); i < e; i += step) {
+                        const int w = __ldg(a.g.col + i);
+                        if (w >= v) break;
+                        touch(w);
+                    }
+                }
+            }
         };
         unsigned long long sum = 0;
         walk([&](int w) { sum += atomicAdd(y + w, 1u); });
         acc.add(sum);
         if (!kShared) {
             __syncthreads();
+            if (kLong) {
+                if (threadIdx.x == 0) s_n_aside = 0;
+                __syncthreads();
+            }
             walk([&](int w) { __stcg(y + w, 0u); });
         }
     }
@@ -281,14 +315,20 @@ bool wedge_applies(const CountJob& job, const gp_graph* g, const LaunchOpts& opt
     // On sparse graphs of many vertices the block's turn per vertex (clearing,
     // barriers) outweighs the lists: House at mean degree 2, 50 K vertices 0.73
     // against 0.52 ms; 4-cycles with counters in global memory at mean degree 8,
-    // 100 K vertices 1.57 against 1.42 ms (at 20, 200 K: 2.9 against 5.6)
-    if (is_cycle4(job.plan)) return !global || g->nnz >= 14 * (int64_t)g->n;
-    if (!is_house_plan(job.plan)) return false;
-    if (!global) return g->n <= 16 * 1024 || g->nnz >= 4 * (int64_t)g->n - g->n / 4;
+    // 100 K vertices 1.57 against 1.42 ms (at 20, 200 K: 2.9 against 5.6); at 16,
+    // where the counters outgrow the L2 and the blocks are not all there, 1 M
+    // vertices 25 against 13 ms (at 20: 17 against 20; Chung-Lu, 1 M: 170 against
+    // 254)
+    const bool cycle = is_cycle4(job.plan);
+    if (!cycle && !is_house_plan(job.plan)) return false;
+    if (!global) return cycle || g->n <= 16 * 1024 || g->nnz >= 4 * (int64_t)g->n - g->n / 4;
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
-    return house_pays(g, global_blocks(g, nsm));
+    const int64_t blocks = global_blocks(g, nsm);
+    if (!cycle) return house_pays(g, blocks);
+    return g->nnz >= 14 * (int64_t)g->n &&
+           (g->max_deg > kSetAside || blocks >= (int64_t)nsm * 2 || counter_bytes(g) * (double)blocks <= 128e6);
 }
 
 gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, ResultWords* words, int64_t* warps) {
@@ -305,7 +345,10 @@ gp_status launch_wedge(const CountJob& job, const gp_graph* g, cudaStream_t st, 
     const size_t bytes = counter_bytes(g);
     const bool shared = bytes <= kSharedCounters;
     const int threads = shared && bytes > 110 * 1024 ? 1024 : 512;
-    auto fn = cycle ? (shared ? k_cycle4<true> : k_cycle4<false>) : (shared ? k_wedge<true> : k_wedge<false>);
+    const bool aside = g->max_deg > kSetAside;
+    auto fn = cycle ? (shared ? (aside ? k_cycle4<true, true> : k_cycle4<true, false>)
+                              : (aside ? k_cycle4<false, true> : k_cycle4<false, false>))
+                    : (shared ? k_wedge<true> : k_wedge<false>);
     const size_t smem = shared ? bytes : 0;
     if (smem > kDefaultShared) {
         const gp_status rc = raise_shared_limit((const void*)fn, kSharedCounters);

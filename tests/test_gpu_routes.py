@@ -41,13 +41,21 @@ def uniform(n, degree):
     return n, er_edges(n, n * degree // 2, seed=n)
 
 
-# without the check these took 18, 110, 36, 5 and 4 times as long as the general kernel
+def two_hubs(leaves):
+    """A ring of vertices joined to two hubs."""
+    leaf = 2 + np.arange(leaves)
+    return 2 + leaves, joined((leaf, 2 + (leaf - 1) % leaves), (0 * leaf, leaf), (0 * leaf + 1, leaf))
+
+
+# these took 18, 110, 36, 5, 4, 4 and 7 times as long as the general kernel
 @pytest.mark.parametrize("pattern,ordered,graph", [
     ("k5", False, lambda: late_hubs(500, 3000)),
     ("k6", False, lambda: late_hubs(500, 3000)),
     ("k6", False, lambda: late_hubs(10, 4000)),
     ("house", True, lambda: uniform(1_000_000, 4)),
     ("house", False, lambda: uniform(500_000, 4)),
+    ("c4", True, lambda: two_hubs(30_000)),
+    ("c4", False, lambda: two_hubs(30_000)),
 ])
 def test_not_much_slower_than_the_general_kernel(pattern, ordered, graph):
     N = native()

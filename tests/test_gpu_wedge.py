@@ -72,3 +72,33 @@ def test_four_cycle_under_an_explicit_restriction_set(oracle_lib, res):
     nnz = g.device_csr()[2]
     assert sum(N.gp_count(g, s, 0, N.make_opts(task_begin=a, task_end=b))[1]
                for a, b in ((0, nnz // 3), (nnz // 3, nnz))) == expect
+
+
+# lists that the block walks: two of them, more than it can set aside at once,
+# counters in shared and in global memory, with and without the degree order
+@pytest.mark.parametrize("ordered", [True, False])
+@pytest.mark.parametrize("leaves", [511, 513, 3000])
+def test_four_cycles_of_two_hubs(leaves, ordered):
+    N = native()
+    leaf = np.arange(2, 2 + leaves, dtype=np.int32)
+    g = N.gp_graph_create_edges(np.concatenate([0 * leaf, 0 * leaf + 1]), np.concatenate([leaf, leaf]), 2 + leaves,
+                                N.GP_DEGREE_ORDER if ordered else 0)
+    s = N.gp_schedule(N.gp_pattern_create(named_pattern("c4")), g, 1)
+    assert N.gp_count(g, s, 0)[1] == comb(leaves, 2)
+
+
+@pytest.mark.parametrize("ordered", [True, False])
+@pytest.mark.parametrize("core,n,m", [(250, 900, 3000), (800, 2000, 3000), (800, 57_400, 500_000)])
+def test_four_cycles_with_many_long_lists(core, n, m, ordered):
+    N = native()
+    rs = np.random.RandomState(core)
+    a, b = np.triu_indices(core, 1)
+    keep = rs.rand(len(a)) < 0.9
+    src, dst = er_edges(n, m, seed=n)
+    hubs = np.repeat(np.arange(core), 400)     # the core's lists exceed 512 entries
+    src = np.concatenate([src, a[keep], hubs]).astype(np.int32)
+    dst = np.concatenate([dst, b[keep], rs.randint(0, n, 400 * core)]).astype(np.int32)
+    order = rs.permutation(n).astype(np.int32)
+    g = N.gp_graph_create_edges(order[src], order[dst], n, N.GP_DEGREE_ORDER if ordered else 0)
+    s = N.gp_schedule(N.gp_pattern_create(named_pattern("c4")), g, 1)
+    assert N.gp_count(g, s, 0) == N.gp_count(g, s, 0, N.make_opts(flags=N.GP_COUNT_NO_CORE))

@@ -790,7 +790,7 @@ gp_status gp_count_batch(gp_graph* const* graphs, const gp_schedules* const* sch
             chunk = std::min<int64_t>(chunk, jobs[j].nvirt / ((int64_t)nsm * 4 * 8 * 64));
         }
         // (tasks that go one per lane take run_count's own rule)
-        lo.chunk = user_chunk > 0 ? user_chunk : lane_tasks(group[0].plan) ? 0 : (int)std::max<int64_t>(1, chunk);
+        lo.chunk = user_chunk > 0 ? user_chunk : lane_tasks(group[0]) ? 0 : (int)std::max<int64_t>(1, chunk);
         std::vector<uint64_t> gres(2 * group.size(), 0);
         std::vector<int> gab(group.size(), 0);
         int64_t done = 0;

@@ -1959,9 +1959,13 @@ __global__ void k_label_tasks(const CountJob* __restrict__ job, unsigned long lo
     }
 }
 
+// Lists of three-vertex labelled counts up to this length are walked by a lane,
+// one load after the other; nothing else shares out such a task.
+constexpr int kLabelTaskWalk = 32;
+
 // The last level's count for one lane's v[0..k-2], elements with the last
 // vertex's label only; false (nothing counted) above the work limit.
-__device__ __forceinline__ bool label_last_lane(const TaskCtx& c, const int* v, Acc& acc) {
+__device__ __forceinline__ bool label_last_lane(const TaskCtx& c, const int* v, Acc& acc, int most) {
     const GpPlan& P = *c.P;
     const int L = P.k - 1;
     const GpLevel& lv = P.lvl[L];
@@ -1974,7 +1978,7 @@ __device__ __forceinline__ bool label_last_lane(const TaskCtx& c, const int* v, 
     } else {
         q.it = clip((lv.src_kind == 1) ? nbr(c, v[lv.src]) : slot(c, lv.src), w);
     }
-    if (q.it.n > c.lane_work) return false;
+    if (q.it.n > most) return false;
     int cnt = 0, from = two && q.bitmap ? q.tail : 0;
     for (int i = 0; i < q.it.n; ++i) {
         const int x = __ldg(q.it.p + i);
@@ -2019,8 +2023,14 @@ k_label(const CountJob* __restrict__ job, const unsigned long long* __restrict__
     // spread; three-vertex patterns have no depth-2 loop to share out and go
     // one task per lane
     const int parts = k == 3 ? 1 : (int)min(64ll, max(1ll, 16 * warps / max(1ll, n)));
-    const int grab = k == 3 ? 32 : 1;
+    const bool chain = (P.lvl[2].lo_mask | P.lvl[2].hi_mask) == 3;      // its first three vertices in one order
+    // the lanes of a warp under hubs: fewer tasks a grab, so that theirs spread
+    // (triangles of R-MAT 14 with two labels 0.5 -> 0.21 ms); not where the
+    // restrictions put all three vertices in order, which cuts the hubs' lists
+    const bool hubs = (long long)job->slot_cap * job->n > 6 * job->ntasks && !chain;
+    const int grab = k != 3 ? 1 : hubs ? (int)min(32ll, max(1ll, n / (16 * warps))) : 32;
     const bool lanes_last = P.lvl[k - 2].nbuild == 0;
+    const int walk = k == 3 && !chain ? kLabelTaskWalk : c.lane_work;
     Acc acc;
     for (;;) {
         unsigned long long t0 = 0;
@@ -2031,13 +2041,13 @@ k_label(const CountJob* __restrict__ job, const unsigned long long* __restrict__
 #pragma unroll
         for (int i = 0; i < GP_MAX_K; ++i) v[i] = -1;
         if (k == 3) {
-            const bool have = (long long)t0 + lane < n;
+            const bool have = lane < grab && (long long)t0 + lane < n;
             const int2 t = have ? tasks[t0 + lane] : make_int2(0, 0);
             bool defer = false;
             if (P.lvl[1].nbuild == 0) {
                 v[0] = t.x;
                 v[1] = t.y;
-                defer = have && !label_last_lane(c, v, acc);
+                defer = have && !label_last_lane(c, v, acc, walk);
             } else {
                 defer = have;
             }
@@ -2085,7 +2095,7 @@ k_label(const CountJob* __restrict__ job, const unsigned long long* __restrict__
                     bool defer = false;
                     if (in) {
                         v[d] = x;
-                        defer = !label_last_lane(c, v, acc);
+                        defer = !label_last_lane(c, v, acc, walk);
                     }
                     unsigned dm = __ballot_sync(kFull, defer);
                     while (dm) {
@@ -2363,6 +2373,20 @@ struct Geometry {
     int64_t total;          // tasks over all jobs
 };
 
+// A graph without the degree order (no core, no heavy prefix) whose largest
+// degree is far above the mean: tasks of a hub may lie anywhere, many in a row.
+bool late_hubs(const CountJob& job) {
+    return !job.core_bits && (int64_t)job.slot_cap * job.n > 6 * job.ntasks;
+}
+
+// Does the job run in its lane form? Four-vertex plans that count an
+// intersection per edge task do not under such hubs, whose tasks would fill the
+// lanes of single warps (tailed triangles of R-MAT 14 without the order: 2.5
+// against 1.6 ms).
+bool lane_job(const CountJob& job) {
+    return lane_form(job.plan) && !(job.plan.k == 4 && job.plan.iep && job.plan.iep_fuse && late_hubs(job));
+}
+
 // Grid of the persistent launch: SM count x resident blocks per SM, reduced
 // (in whole waves of SMs) until the per-warp intermediate-set scratch fits in
 // a quarter of the free device memory.
@@ -2396,7 +2420,7 @@ gp_status geometry(const CountJob* jobs, int njobs, const LaunchOpts& opt, Geome
     bool general_iep = false;              // some job replaces three or more loops or fuses two
     for (int j = 0; j < njobs; ++j) general_iep |= jobs[j].plan.iep >= 3 || jobs[j].plan.iep_fuse;
     bool lanes = opt.blocks_per_sm <= 0;   // every job has a lane form
-    for (int j = 0; j < njobs; ++j) lanes &= lane_form(jobs[j].plan);
+    for (int j = 0; j < njobs; ++j) lanes &= lane_job(jobs[j]);
     if (opt.stats) {
         g->kern = (want == 1 || want == 2) ? k_count<true, 1, true>
                 : (want == 3) ? k_count<true, 3, true> : k_count<true, 4, true>;
@@ -2436,8 +2460,9 @@ gp_status geometry(const CountJob* jobs, int njobs, const LaunchOpts& opt, Geome
 
 }  // namespace
 
-bool lane_tasks(const GpPlan& P) {
-    return !P.labeled && P.lvl[1].nbuild == 0 && (P.k == 3 || (P.k == 4 && lane_form(P) && P.iep));
+bool lane_tasks(const CountJob& job) {
+    const GpPlan& P = job.plan;
+    return !P.labeled && P.lvl[1].nbuild == 0 && (P.k == 3 || (P.k == 4 && lane_job(job) && P.iep));
 }
 
 int kernel_variant(const CountJob& job, const LaunchOpts& opt) {
@@ -2450,8 +2475,8 @@ int kernel_variant(const CountJob& job, const LaunchOpts& opt) {
         P.lvl[P.k - 2].bm_inc && P.lvl[P.k - 1].bm_inc)
         want = 3;
     if (opt.blocks_per_sm <= 0 && !opt.stats) {
-        if (lane_tasks(P)) return P.iep ? 17 : 18;     // grabs of their own size
-        if (lane_form(P)) return 16;
+        if (lane_tasks(job)) return P.iep ? 17 : 18;   // grabs of their own size
+        if (lane_job(job)) return 16;
     }
     return (P.iep >= 3 || P.iep_fuse ? 8 : 0) + want;
 }
@@ -2477,11 +2502,16 @@ gp_status run_count(const CountJob* jobs, int njobs, const LaunchOpts& opt, cuda
     int chunk = opt.chunk;
     if (chunk <= 0) {
         // tasks that go one per lane want grabs that fill some of the warp even
-        // on small graphs (3-vertex paths of R-MAT 10: 119 us in grabs of one)
-        bool lanes = opt.blocks_per_sm <= 0 && !opt.stats;
-        for (int j = 0; j < njobs; ++j) lanes &= lane_tasks(jobs[j].plan);
-        const int64_t per_warp = total / (blocks * kWarps * (lanes ? 2 : 64));
-        chunk = (int)std::max<int64_t>(lanes ? 8 : 1, std::min<int64_t>(64, per_warp));
+        // on small graphs (3-vertex paths of R-MAT 10: 119 us in grabs of one);
+        // smaller ones where hubs' tasks that intersect lists lie anywhere
+        // (triangles of R-MAT 16 with the ids reversed: 2.6 -> 1.8 ms)
+        bool lanes = opt.blocks_per_sm <= 0 && !opt.stats, hubs = false;
+        for (int j = 0; j < njobs; ++j) {
+            lanes &= lane_tasks(jobs[j]);
+            hubs |= late_hubs(jobs[j]) && jobs[j].plan.last_count_only;
+        }
+        const int64_t per_warp = total / (blocks * kWarps * (!lanes ? 64 : hubs ? 4 : 2));
+        chunk = (int)std::max<int64_t>(!lanes ? 1 : hubs ? 4 : 8, std::min<int64_t>(lanes && hubs ? 32 : 64, per_warp));
     }
 
     // device buffers: job table, results (2 per job), cursor, error word

@@ -167,8 +167,8 @@ gp_status run_list(const CountJob& job, int32_t* d_out, int64_t capacity, cudaSt
 // The 128-bit count of a labelled plan's job (count.cu).
 gp_status run_labeled(const CountJob& job, cudaStream_t st, uint64_t* results);
 
-// True when the count kernel takes the plan's edge tasks one per lane.
-bool lane_tasks(const GpPlan& P);
+// True when the count kernel takes the job's edge tasks one per lane.
+bool lane_tasks(const CountJob& job);
 
 // Key of the kernel build geometry() would pick for this job alone (its
 // register budget and whether it carries general inclusion-exclusion); jobs

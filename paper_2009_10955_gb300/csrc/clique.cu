@@ -674,7 +674,9 @@ gp_status launch_clique(const CountJob& job, const gp_graph* g, cudaStream_t st,
     }
     const size_t big_b = big ? sizeof(uint32_t) * (2 * (size_t)a.big_words + 2 * kMostRows) : 0;
     const size_t sets_b = k >= 6 && a.n_block > 0 ? sizeof(uint32_t) * (size_t)(threads / 32) * 4 * (kMostRows / 32) : 0;
-    gp_status rc = fit_blocks(nsm, big_b + sets_b, &blocks);
+    // asking for the free memory takes 12 us, a quarter of a small count: scratch
+    // of up to 64 MB is simply asked for (without it the general kernel counts)
+    gp_status rc = (big_b + sets_b) * (size_t)blocks > ((size_t)64 << 20) ? fit_blocks(nsm, big_b + sets_b, &blocks) : GP_OK;
     if (rc != GP_OK) return rc;
     // roots are cut into parts where they are too few to fill the grid evenly.
     // Each part builds the root's matrix anew, which is most of the work where

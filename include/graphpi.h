@@ -126,8 +126,8 @@ gp_status gp_pattern_create(const uint8_t* adj, int32_t k, gp_pattern** out);
  * graphs): as gp_pattern_create, plus labels[k]; a vertex matched to
  * pattern vertex a must carry labels[a], and automorphisms must preserve
  * labels. Labelled plans are counted by gp_count (by a kernel that visits the
- * edge tasks whose two vertices carry their labels) and listed by gp_list; the batched, time-sliced and no-allocation calls
- * reject them. */
+ * edge tasks whose two vertices carry their labels) and listed by gp_list; the
+ * batched, time-sliced and no-allocation calls reject them. */
 gp_status gp_pattern_create_labeled(const uint8_t* adj, const int32_t* labels, int32_t k,
                                     gp_pattern** out);
 
@@ -230,7 +230,10 @@ void gp_schedule_destroy(gp_schedules* s);
 /* ----------------------------------------------------------------- count */
 
 /* Optional tuning and control for gp_count / gp_count_batch. Zero fields
- * take the library defaults. */
+ * take the library defaults. Plans that a kernel of their own counts (cliques,
+ * joins of a clique and independent vertices, the House, cycles) ignore
+ * warps_per_block, blocks_per_sm, chunk, split and lane_work; a flag below, a
+ * budget or a cycle limit takes them to the general kernel instead. */
 typedef struct gp_count_opts {
     int32_t struct_size;      /* sizeof(gp_count_opts)                               */
     int32_t warps_per_block;  /* 1..32                                               */
